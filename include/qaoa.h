@@ -216,8 +216,10 @@ int64_t qaoa_scratch_bytes(const qaoa_ctx *ctx);
  *   cost_dtype  QAOA_COST_U8 (integer costs; fails with QAOA_ERR_INVALID if a
  *               value can exceed 255) or QAOA_COST_F32
  *   dim         2^n for unconstrained problems, binom(n,k) for DKS
- * SK with couplings on the 2^-20 grid (|J| < 8) is summed exactly in integers
- * and rounded once to float32; other couplings are summed in float64. */
+ * SK couplings (MaxCut weights) that are multiples of one power of two, with
+ * sums below 2^50 of it -- every J on the 2^-20 grid with |J| < 8, say -- are
+ * summed exactly in integers and rounded once to float32; others are summed in
+ * float64. */
 qaoa_status qaoa_cost_precompute(qaoa_ctx *ctx, const qaoa_problem *prob, void *d_cost,
                                  int cost_dtype, int64_t dim);
 

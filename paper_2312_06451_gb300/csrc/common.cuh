@@ -352,11 +352,22 @@ cudaError_t launch_tile12(const SmallDesc *d_descs, int ndesc, int cost_dtype, i
 cudaError_t launch_wait_probe(int *d_err, cudaStream_t s);
 
 // Cost precompute (kernels_cost.cu).
-cudaError_t launch_cost_maxcut(int n, const uint64_t *nbr_hi_host, const float *d_w_edges,
-                               const int32_t *d_edges, int m, int weighted, int64_t dim,
-                               void *d_out, int dtype, cudaStream_t s);
-cudaError_t launch_cost_sk(int n, const int32_t *d_Jq, const double *d_Jd, int exact,
-                           int64_t dim, float *d_out, cudaStream_t s);
+constexpr int kQuadMaxN = 34;  // unconstrained cost vectors
+// C(x) = 2^-shift (base + sum_{i<j} K_ij z_i z_j) in integers (cost_quad_kernel).
+struct CostQuad {
+    int64_t K[kQuadMaxN][kQuadMaxN];
+    int64_t base;
+    int n, shift;
+    bool wide;  // the sums need 64 bits
+};
+// The form of sum_{i<j} w_ij z_i z_j (cut: of the cut weight, w_ij (1 - z_i z_j) / 2) for an
+// upper-triangular n x n matrix, or false when the couplings have no common grid that keeps its sums
+// exact in float64 too (then: the float64 kernels).
+bool cost_quad_exact(CostQuad &C, const double *w, int n, bool cut);
+cudaError_t launch_cost_quad(const CostQuad &C, int64_t dim, void *d_out, int dtype, cudaStream_t s);
+cudaError_t launch_cost_wmaxcut(const float *d_w, const int32_t *d_edges, int m, int64_t dim, float *d_out,
+                                cudaStream_t s);
+cudaError_t launch_cost_sk(int n, const double *d_Jd, int64_t dim, float *d_out, cudaStream_t s);
 cudaError_t launch_cost_dks(int n, int k, const uint64_t *nbr_hi, int64_t dim, void *d_out, int dtype,
                             int kvc, int m, cudaStream_t s);
 cudaError_t launch_dicke_states(int n, int k, int64_t dim, uint64_t *d_out, cudaStream_t s);

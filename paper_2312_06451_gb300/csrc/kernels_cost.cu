@@ -2,18 +2,22 @@
 // Sec. 2.1: C(x) is evaluated once for every feasible x and stored) and the
 // Hamming-weight-k feasible set itself.
 //
-//   MaxCut   C(x) = sum_u popcount(nbr_hi[u] & (x_u ? ~x : x)): every edge
-//            (u, v), v > u, is counted from its lower end when x_v != x_u.
+//   MaxCut   C(x) = #{edges (u, v) : x_u != x_v}, weighted: the sum of their weights.
+//   SK       C(x) = sum_{i<j} J_ij z_i z_j, z_i = 1 - 2 x_i.
+//            Both are quadratic forms in z.  When the couplings are multiples
+//            of one power of two and the sums fit, they are carried exactly in
+//            integers and rounded once to the output type (cost_quad_kernel);
+//            float32 couplings that spread too far are summed in float64.
 //   DkS      C(x) = sum_u x_u popcount(nbr_hi[u] & x) on weight-k states.
 //   k-VC     C(x) = m - (the DkS count of the complement of x).
-//   SK       C(x) = sum_{i<j} J_ij z_i z_j, z_i = 1 - 2 x_i.  When every
-//            J_ij is a multiple of 2^-20 the sum is carried exactly in int64
-//            (J scaled by 2^20) and rounded once to float32, so the result is
-//            independent of summation order.
 //   Dicke    state of rank r (increasing integer order = colex order of
 //            k-subsets) by the combinatorial number system:
 //            x = {c_k > ... > c_1}, r = sum_i binom(c_i, i).
 #include "common.cuh"
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
 
 namespace qg {
 
@@ -61,22 +65,6 @@ __device__ __forceinline__ int64_t rank_colex(uint64_t x) {
     return r;
 }
 
-__global__ void cost_maxcut_kernel(AdjParams A, int64_t dim, void *out, int dtype) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < dim;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        int c = 0;
-        const uint64_t ux = (uint64_t)x;
-        for (int u = 0; u < A.n; u++) {
-            const uint64_t m = A.nbr[u];
-            c += __popcll(m & (((ux >> u) & 1) ? ~ux : ux));
-        }
-        if (dtype == 1)
-            reinterpret_cast<unsigned char *>(out)[x] = (unsigned char)c;
-        else
-            reinterpret_cast<float *>(out)[x] = (float)c;
-    }
-}
-
 __global__ void cost_wmaxcut_kernel(const int32_t *edges, const float *w, int m, int64_t dim,
                                     float *out) {
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < dim;
@@ -92,23 +80,123 @@ __global__ void cost_wmaxcut_kernel(const int32_t *edges, const float *w, int m,
 
 constexpr int kSkMaxN = 40;
 
-__global__ void cost_sk_exact_kernel(int n, const int32_t *Jq, int64_t dim, float *out) {
-    __shared__ int32_t J[kSkMaxN * kSkMaxN];
-    for (int i = threadIdx.x; i < n * n; i += blockDim.x) J[i] = Jq[i];
+// MaxCut, weighted MaxCut and SK costs on all 2^n states as one integer
+// quadratic form: C(x) = 2^-shift (base + sum_{i<j} K_ij z_i z_j), z = 1 - 2 x,
+// carried exactly (so the result does not depend on the summation order) and
+// rounded once to the output type.  An edge of weight w contributes
+// w (1 - z_u z_v) / 2.
+//
+// One write per state bounds it (256 MiB of float32 at n = 26: 40 us), so a
+// state may cost a handful of adds, not one per pair.  Local qubits 0, 1, 10
+// and 11 are a thread's 16 outputs of a tile of 2^12, qubits 2..9 its index,
+// qubits 12..11+M the 2^M tiles a block walks in Gray-code order, the rest the
+// block index.  A thread sums its own qubits' pairs and the fields they exert
+// once; a tile then moves by one flipped qubit (a few adds), and the 16
+// outputs are +- combinations of five sums: about 4 adds an output instead of
+// n(n-1)/2 with a shared-memory load each.  n = 26, int32: a call 12.1 ms -> 81 us.
+template <typename A>
+struct QuadParams {
+    A K[kQuadMaxN][kQuadMaxN];  // symmetric, zero diagonal, zero beyond n
+    A base;
+    int n;
+    float scale;  // 2^-shift (float32 output)
+};
+
+template <typename A, int U8, int M>
+__global__ void __launch_bounds__(256) cost_quad_kernel(const __grid_constant__ QuadParams<A> Q, int64_t dim, void *out) {
+    __shared__ A s_f[12 + M];  // fields of the block's qubits on the local ones
+    __shared__ A s_e;          // base + the block qubits' own pairs
+    const int tid = threadIdx.x, nb = Q.n - 12 - M;  // block qubits 12 + M ..
+    const uint32_t hi = blockIdx.x;
+    auto sg = [](uint32_t bit, A v) -> A { return bit ? -v : v; };
+    if (tid < 12 + M) {
+        A f = 0;
+        for (int u = 0; u < nb; u++) f += sg((hi >> u) & 1u, Q.K[tid][12 + M + u]);
+        s_f[tid] = f;
+    } else if (tid >= 32 && tid < 64) {
+        const int u = tid - 32;  // at most kQuadMaxN - 12 block qubits
+        A e = 0;
+        for (int v = u + 1; v < nb; v++) e += sg(((hi >> u) ^ (hi >> v)) & 1u, Q.K[12 + M + u][12 + M + v]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+        if (u == 0) s_e = e + Q.base;
+    }
     __syncthreads();
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < dim;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const uint64_t ux = (uint64_t)x;
-        int64_t acc = 0;
-        for (int i = 0; i < n; i++) {
-            const uint64_t xi = (ux >> i) & 1;
-            const int32_t *row = J + i * n;
-            for (int j = i + 1; j < n; j++) {
-                const int32_t v = row[j];
-                acc += (((ux >> j) & 1) ^ xi) ? -(int64_t)v : (int64_t)v;
+    // this thread's qubits 2..9: their pairs and fields, and the fields on the
+    // output qubits (a) and the tile qubits (g)
+    A S = s_e, a[4], g[M > 0 ? M : 1];
+    const int rq[4] = {0, 1, 10, 11};
+#pragma unroll
+    for (int r = 0; r < 4; r++) a[r] = s_f[rq[r]];
+#pragma unroll
+    for (int j = 0; j < M; j++) g[j] = s_f[12 + j];
+#pragma unroll
+    for (int i = 2; i < 10; i++) {
+        const uint32_t bi = (uint32_t)tid >> (i - 2);
+        A f = s_f[i];
+#pragma unroll
+        for (int j = i + 1; j < 10; j++) f += sg(((uint32_t)tid >> (j - 2)) & 1u, Q.K[i][j]);
+        S += sg(bi & 1u, f);
+#pragma unroll
+        for (int r = 0; r < 4; r++) a[r] += sg(bi & 1u, Q.K[i][rq[r]]);
+#pragma unroll
+        for (int j = 0; j < M; j++) g[j] += sg(bi & 1u, Q.K[i][12 + j]);
+    }
+    // the first tile has every tile qubit at z = +1
+#pragma unroll
+    for (int j = 0; j < M; j++) {
+        S += g[j];
+#pragma unroll
+        for (int l = 0; l < M; l++)
+            if (l != j) {
+                if (l < j) S += Q.K[12 + j][12 + l];
+                g[j] += Q.K[12 + j][12 + l];
+            }
+#pragma unroll
+        for (int r = 0; r < 4; r++) a[r] += Q.K[rq[r]][12 + j];
+    }
+    const int64_t x0 = ((int64_t)hi << (12 + M)) + 4 * tid;
+#pragma unroll
+    for (int t = 0; t < (1 << M); t++) {
+        if (t) {  // Gray code: flip tile qubit j, from z = +1 to -1 (down) or back
+            const int j = (t & 1) ? 0 : (t & 2) ? 1 : (t & 4) ? 2 : 3;
+            const bool down = ((t ^ (t >> 1)) >> j) & 1;
+            S += down ? -2 * g[j] : 2 * g[j];
+#pragma unroll
+            for (int l = 0; l < M; l++)
+                if (l != j) g[l] += down ? -2 * Q.K[12 + j][12 + l] : 2 * Q.K[12 + j][12 + l];
+#pragma unroll
+            for (int r = 0; r < 4; r++) a[r] += down ? -2 * Q.K[12 + j][rq[r]] : 2 * Q.K[12 + j][rq[r]];
+        }
+        const int64_t xt = x0 + ((int64_t)(t ^ (t >> 1)) << 12);
+#pragma unroll
+        for (int h = 0; h < 4; h++) {  // qubits 10, 11
+            const A k1 = Q.K[10][11];
+            const A s = S + ((h & 1) ? -a[2] : a[2]) + ((h & 2) ? -a[3] : a[3]) + (((h >> 1) ^ h) & 1 ? -k1 : k1);
+            const A b0 = a[0] + ((h & 1) ? -Q.K[0][10] : Q.K[0][10]) + ((h & 2) ? -Q.K[0][11] : Q.K[0][11]);
+            const A b1 = a[1] + ((h & 1) ? -Q.K[1][10] : Q.K[1][10]) + ((h & 2) ? -Q.K[1][11] : Q.K[1][11]);
+            const A p = s + Q.K[0][1], m = s - Q.K[0][1], u = b0 + b1, v = b1 - b0;
+            const A c[4] = {p + u, m + v, m - v, p - u};  // (z_0, z_1) = ++, -+, +-, --
+            const int64_t x = xt + ((int64_t)h << 10);
+            if (U8) {
+                const uchar4 o = make_uchar4((unsigned char)(c[0] >> 1), (unsigned char)(c[1] >> 1),
+                                             (unsigned char)(c[2] >> 1), (unsigned char)(c[3] >> 1));
+                unsigned char *dst = reinterpret_cast<unsigned char *>(out) + x;
+                if (x + 4 <= dim) __stcs(reinterpret_cast<uchar4 *>(dst), o);
+                else
+                    for (int i = 0; i < 4; i++)
+                        if (x + i < dim) dst[i] = i == 0 ? o.x : i == 1 ? o.y : i == 2 ? o.z : o.w;
+            } else {
+                float f[4];
+#pragma unroll
+                for (int i = 0; i < 4; i++) f[i] = (sizeof(A) == 8 ? __ll2float_rn((long long)c[i]) : __int2float_rn((int)c[i])) * Q.scale;
+                float *dst = reinterpret_cast<float *>(out) + x;
+                if (x + 4 <= dim) __stcs(reinterpret_cast<float4 *>(dst), make_float4(f[0], f[1], f[2], f[3]));
+                else
+                    for (int i = 0; i < 4; i++)
+                        if (x + i < dim) dst[i] = f[i];
             }
         }
-        out[x] = __ll2float_rn(acc) * 9.5367431640625e-07f;  // * 2^-20, exact
     }
 }
 
@@ -206,25 +294,80 @@ AdjParams make_adj(int n, const uint64_t *nbr_hi) {
 
 }  // namespace
 
-cudaError_t launch_cost_maxcut(int n, const uint64_t *nbr_hi, const float *d_w, const int32_t *d_edges,
-                               int m, int weighted, int64_t dim, void *d_out, int dtype,
-                               cudaStream_t s) {
-    if (weighted) {
-        cost_wmaxcut_kernel<<<grid_for(dim, 256), 256, 0, s>>>(d_edges, d_w, m, dim,
-                                                               reinterpret_cast<float *>(d_out));
-    } else {
-        cost_maxcut_kernel<<<grid_for(dim, 256), 256, 0, s>>>(make_adj(n, nbr_hi), dim, d_out, dtype);
+namespace {
+
+template <typename A, int U8>
+cudaError_t go_quad(const CostQuad &C, int64_t dim, void *d_out, cudaStream_t s) {
+    QuadParams<A> Q;
+    for (int i = 0; i < kQuadMaxN; i++)
+        for (int j = 0; j < kQuadMaxN; j++) Q.K[i][j] = i < C.n && j < C.n ? (A)C.K[i][j] : (A)0;
+    Q.base = (A)C.base;
+    Q.n = std::max(C.n, 12);  // qubits a small instance lacks: no couplings, states past dim not written
+    Q.scale = ldexpf(1.f, -C.shift);
+    // 2^M tiles a block: all 16 once that leaves two or more blocks an SM (M = 4 from n = 25), fewer
+    // tiles and more blocks below
+    const int M = std::max(0, std::min(4, Q.n - 21));
+    const unsigned grid = 1u << (Q.n - 12 - M);
+    switch (M) {
+    case 0: cost_quad_kernel<A, U8, 0><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 1: cost_quad_kernel<A, U8, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 2: cost_quad_kernel<A, U8, 2><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 3: cost_quad_kernel<A, U8, 3><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    default: cost_quad_kernel<A, U8, 4><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
     }
     return cudaGetLastError();
 }
 
-cudaError_t launch_cost_sk(int n, const int32_t *d_Jq, const double *d_Jd, int exact, int64_t dim,
-                           float *d_out, cudaStream_t s) {
+}  // namespace
+
+bool cost_quad_exact(CostQuad &C, const double *w, int n, bool cut) {
+    if (n > kQuadMaxN) return false;
+    // the grid 2^-shift that holds every coupling
+    int shift = 0;
+    for (int i = 0; i < n; i++)
+        for (int j = i + 1; j < n; j++) {
+            const double v = w[i * n + j];
+            if (!std::isfinite(v)) return false;
+            if (v == 0.0) continue;
+            int e = 0;
+            const double f = std::frexp(v, &e);  // v = f 2^e, f of at most 53 bits
+            const int64_t m = (int64_t)std::ldexp(f, 53);
+            shift = std::max(shift, 53 - e - __builtin_ctzll((unsigned long long)m));
+        }
+    if (shift > 90) return false;  // float32 results stay far from the subnormals
+    // sums below 2^50 on the grid: exact in int64, and in the float64 sums they stand for
+    double total = 0.0;
+    for (int i = 0; i < n; i++)
+        for (int j = i + 1; j < n; j++) total += std::ldexp(std::fabs(w[i * n + j]), shift);
+    if (!(total < 1125899906842624.0)) return false;
+    std::memset(&C, 0, sizeof(C));
+    C.n = n;
+    C.shift = shift + (cut ? 1 : 0);
+    for (int i = 0; i < n; i++)
+        for (int j = i + 1; j < n; j++) {
+            const int64_t k = (int64_t)std::ldexp(w[i * n + j], shift);
+            C.K[i][j] = C.K[j][i] = cut ? -k : k;
+            C.base += cut ? k : 0;
+        }
+    C.wide = total + std::fabs((double)C.base) >= 1073741824.0;  // a thread's running sums reach twice this at most
+    return true;
+}
+
+cudaError_t launch_cost_quad(const CostQuad &C, int64_t dim, void *d_out, int dtype, cudaStream_t s) {
+    if (C.n < 1 || C.n > kQuadMaxN || (dtype == 1 && (C.shift != 1 || C.wide))) return cudaErrorInvalidValue;
+    if (dtype == 1) return go_quad<int32_t, 1>(C, dim, d_out, s);
+    return C.wide ? go_quad<int64_t, 0>(C, dim, d_out, s) : go_quad<int32_t, 0>(C, dim, d_out, s);
+}
+
+cudaError_t launch_cost_wmaxcut(const float *d_w, const int32_t *d_edges, int m, int64_t dim, float *d_out,
+                                cudaStream_t s) {
+    cost_wmaxcut_kernel<<<grid_for(dim, 256), 256, 0, s>>>(d_edges, d_w, m, dim, d_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_cost_sk(int n, const double *d_Jd, int64_t dim, float *d_out, cudaStream_t s) {
     if (n > kSkMaxN) return cudaErrorInvalidValue;
-    if (exact)
-        cost_sk_exact_kernel<<<grid_for(dim, 256), 256, 0, s>>>(n, d_Jq, dim, d_out);
-    else
-        cost_sk_f64_kernel<<<grid_for(dim, 256), 256, 0, s>>>(n, d_Jd, dim, d_out);
+    cost_sk_f64_kernel<<<grid_for(dim, 256), 256, 0, s>>>(n, d_Jd, dim, d_out);
     return cudaGetLastError();
 }
 

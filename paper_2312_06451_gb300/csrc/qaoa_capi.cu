@@ -2323,6 +2323,23 @@ qaoa_status qaoa_cost_precompute(qaoa_ctx *ctx, const qaoa_problem *prob, void *
             if (prob->kind == QAOA_PROBLEM_WMAXCUT) {
                 if (cost_dtype != QAOA_COST_F32 || !prob->weights)
                     return fail(ctx, QAOA_ERR_INVALID, "weighted MaxCut needs weights and float32 costs");
+            }
+            // the cut as an integer quadratic form (weights 1: always; float32
+            // weights: when they share a grid fine enough to keep the sum exact)
+            CostQuad Q;
+            bool quad = false;
+            if (!dks) {
+                std::vector<double> W((size_t)n * n, 0.0);
+                for (int e2 = 0; e2 < prob->m; e2++) {
+                    const int u = std::min(prob->edges[2 * e2], prob->edges[2 * e2 + 1]);
+                    const int v = std::max(prob->edges[2 * e2], prob->edges[2 * e2 + 1]);
+                    W[(size_t)u * n + v] = prob->kind == QAOA_PROBLEM_WMAXCUT ? (double)prob->weights[e2] : 1.0;
+                }
+                quad = cost_quad_exact(Q, W.data(), n, true);
+            }
+            if (quad) {
+                e = launch_cost_quad(Q, dim, d_cost, cost_dtype, ctx->stream);
+            } else if (prob->kind == QAOA_PROBLEM_WMAXCUT) {
                 void *dw = nullptr, *de = nullptr;
                 qaoa_status st = scratch(ctx, "pre_w", sizeof(float) * std::max(1, prob->m), &dw);
                 if (st) return st;
@@ -2332,14 +2349,11 @@ qaoa_status qaoa_cost_precompute(qaoa_ctx *ctx, const qaoa_problem *prob, void *
                                              ctx->stream), "weights upload");
                 QG_CUDA(ctx, cudaMemcpyAsync(de, prob->edges, sizeof(int32_t) * 2 * prob->m,
                                              cudaMemcpyHostToDevice, ctx->stream), "edges upload");
-                e = launch_cost_maxcut(n, nbr, static_cast<float *>(dw), static_cast<int32_t *>(de), prob->m, 1,
-                                       dim, d_cost, cost_dtype, ctx->stream);
-            } else if (dks) {
+                e = launch_cost_wmaxcut(static_cast<float *>(dw), static_cast<int32_t *>(de), prob->m, dim,
+                                        static_cast<float *>(d_cost), ctx->stream);
+            } else {
                 e = launch_cost_dks(n, prob->k, nbr, dim, d_cost, cost_dtype, prob->kind == QAOA_PROBLEM_KVC ? 1 : 0,
                                     prob->m, ctx->stream);
-            } else {
-                e = launch_cost_maxcut(n, nbr, nullptr, nullptr, prob->m, 0, dim, d_cost, cost_dtype,
-                                       ctx->stream);
             }
             if (e != cudaSuccess) return cuda_fail(ctx, e, "cost kernel launch");
             ctx->launches++;
@@ -2347,32 +2361,24 @@ qaoa_status qaoa_cost_precompute(qaoa_ctx *ctx, const qaoa_problem *prob, void *
             if (!prob->J) return fail(ctx, QAOA_ERR_INVALID, "SK needs J");
             if (cost_dtype != QAOA_COST_F32) return fail(ctx, QAOA_ERR_INVALID, "SK costs are float32");
             if (n > 40) return fail(ctx, QAOA_ERR_INVALID, "SK supports n <= 40");
-            bool exact = true;
-            std::vector<int32_t> Jq(n * n, 0);
             std::vector<double> Jd(n * n, 0.0);
             for (int i = 0; i < n; i++)
                 for (int j = 0; j < n; j++) {
                     const double v = (double)prob->J[i * n + j];
                     if (!std::isfinite(v)) return fail(ctx, QAOA_ERR_INVALID, "J[%d][%d] not finite", i, j);
                     Jd[i * n + j] = v;
-                    const double q = v * 1048576.0;
-                    if (std::fabs(v) >= 8.0 || q != std::rint(q)) exact = false;
-                    else Jq[i * n + j] = (int32_t)q;
                 }
-            void *dj = nullptr;
-            qaoa_status st = scratch(ctx, "pre_J", sizeof(double) * n * n, &dj);
-            if (st) return st;
             cudaError_t e;
-            if (exact) {
-                QG_CUDA(ctx, cudaMemcpyAsync(dj, Jq.data(), sizeof(int32_t) * n * n, cudaMemcpyHostToDevice,
-                                             ctx->stream), "J upload");
-                e = launch_cost_sk(n, static_cast<int32_t *>(dj), nullptr, 1, dim, static_cast<float *>(d_cost),
-                                   ctx->stream);
+            CostQuad Q;
+            if (cost_quad_exact(Q, Jd.data(), n, false)) {
+                e = launch_cost_quad(Q, dim, d_cost, cost_dtype, ctx->stream);
             } else {
+                void *dj = nullptr;
+                qaoa_status st = scratch(ctx, "pre_J", sizeof(double) * n * n, &dj);
+                if (st) return st;
                 QG_CUDA(ctx, cudaMemcpyAsync(dj, Jd.data(), sizeof(double) * n * n, cudaMemcpyHostToDevice,
                                              ctx->stream), "J upload");
-                e = launch_cost_sk(n, nullptr, static_cast<double *>(dj), 0, dim, static_cast<float *>(d_cost),
-                                   ctx->stream);
+                e = launch_cost_sk(n, static_cast<double *>(dj), dim, static_cast<float *>(d_cost), ctx->stream);
             }
             if (e != cudaSuccess) return cuda_fail(ctx, e, "cost kernel launch");
             ctx->launches++;
