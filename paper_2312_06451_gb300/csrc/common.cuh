@@ -41,7 +41,8 @@ struct RoundCoef {
     int rescale;   // 1: apply the cos factors after every stage (|cos b| < 1/4)
     float b_hi;    // beta / (2 pi), float32 head (eigenbasis mixers)
     float b_lo;    // beta / (2 pi) - b_hi
-    float pad;
+    float pw[13];  // cos b (of the rounded tan b) to the powers 0..12
+    float pad[2];
 };
 
 // Phase table entries per (unit, round) for uint8 costs: T[c] = e^{-i gamma c}.
@@ -338,11 +339,11 @@ cudaError_t launch_small(const SmallDesc *d_descs, int ndesc, int cost_dtype, in
 // bwd: 0 forward, 1 adjoint.  Persistent launch over total_tiles tiles.
 // var: 0 transverse field, 1 multi-angle, 2 general X mixer (half rounds)
 // d_sched: this launch's tile counter, zero when the launch starts.
-// cost_free: no descriptor of the launch reads the cost vector.
+// gather: the launch's tiles are gathered ones (every descriptor has c < 12), else contiguous.
 // fused: every descriptor is a round-boundary pass (PF_FUSED; var 0 only).
 cudaError_t launch_xpass(int bwd, int cost_dtype, int nbuf, int var, const PassDesc *d_descs,
                          const uint32_t *d_tile_begin, int ndesc, uint32_t total_tiles,
-                         int *d_err, uint32_t *d_sched, int cost_free, int fused, cudaStream_t s);
+                         int *d_err, uint32_t *d_sched, int gather, int fused, cudaStream_t s);
 int small_max_n();
 // n = 12, transverse-field mixer: one CTA per angle set keeps the whole state
 // as one register-staged tile (descriptors as for launch_small).

@@ -15,12 +15,10 @@
 //     passes gather 2^c contiguous amplitudes (c >= 4: whole 128-byte lines)
 //     times 2^(T-c) strided ones to reach the high qubits.
 //   * Each thread holds 16 amplitudes of each vector in registers (a tile of
-//     2^12 amplitudes, 256 threads).  A tile goes through three
-//     register layouts ("stages"): the first is the coalesced 16-byte load
-//     layout, the third the coalesced store layout; two shared-memory
-//     transposes (XOR-swizzled, bank-conflict free) move between them.  Every
-//     rotation happens in registers, on the stage where its bit is a register
-//     bit.
+//     2^12 amplitudes, 256 threads).  A tile goes through as many register
+//     layouts as its rotated bits need (four bits each: one to three), with a
+//     bank-conflict free shared-memory transpose between two.  Every rotation
+//     happens in registers, in the layout where its bit is a register bit.
 //   * The phase e^{-i gamma C} is applied as the tile is loaded, the
 //     expectation sum |psi|^2 C as it is stored, so neither costs a pass.
 //   * The adjoint pass carries lambda and psi together, undoing the rotations
@@ -117,7 +115,15 @@ __device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
     c.g_lo = (float)(g - (double)c.g_hi);
     c.b_hi = (float)bb;
     c.b_lo = (float)(bb - (double)c.b_hi);
-    c.pad = 0.f;
+    // cos b as the rounded tan b has it, so that the rotations keep the norm
+    // whatever t was rounded to, and its powers rounded once each
+    const double ce = c.bmode == 0 ? copysign(1.0 / sqrt(1.0 + (double)c.bt * (double)c.bt), (double)cb) : (double)cb;
+    double q = 1.0;
+    for (int k = 0; k <= kPassTileBits; k++) {
+        c.pw[k] = (float)q;
+        q *= ce;
+    }
+    c.pad[0] = c.pad[1] = 0.f;
     return c;
 }
 
@@ -251,13 +257,6 @@ __device__ __forceinline__ void stage_rot_ma(float2 (&a)[16], float2 (&l)[16], u
     }
 }
 
-// Register bits of the stage whose local bits are b0..b3, from the pass's
-// active-qubit mask.
-__device__ __forceinline__ uint32_t stage_mask(uint32_t active, int b0, int b1, int b2, int b3) {
-    return ((active >> b0) & 1u) | (((active >> b1) & 1u) << 1) | (((active >> b2) & 1u) << 2) |
-           (((active >> b3) & 1u) << 3);
-}
-
 template <int BWD>
 __device__ __forceinline__ void scale_all(float2 (&a)[16], float2 (&l)[16], float f) {
     const float2 ff = make_float2(f, f);
@@ -370,18 +369,37 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void *tmap, int 
 // --------------------------------------------------------------------------
 // The pass kernel (persistent).  A tile is 2^12 amplitudes; 256 threads hold
 // 16 amplitudes each (per vector).  Tile-local bit j is global bit gpos[j]
-// (bits 0..c-1 are the contiguous run).  Register layouts (local bits):
-//   stage 1: amp bit 0 -> 0 (16-byte pair), lanes -> 1..5, warps -> 6..8,
-//            amp bits 1..3 -> 9..11                (read from the TMA buffer)
-//   stage 2: amp bits 0..3 -> 1..4, lanes -> {0,6,7,8,5}, warps -> 9..11
-//   stage 3: amp bits 0..3 -> 5..8, lanes -> 0..4, warps -> 9..11  (stores)
-// Rotated on stage 1: local 0, 9, 10, 11; stage 2: 1..4; stage 3: 5..8.
+// (bits 0..c-1 are the contiguous run; a gathered tile rotates bits c..11, a
+// contiguous one all twelve).  Register layouts (local bits):
+//   P: amplitude bits -> 8..11, lanes -> 0..4, warps -> 5..7     (every store)
+//   Q: amplitude bits -> 4..7, lanes -> 0..3 and 8, warps -> 9..11
+//   R: amplitude bits -> 0..3, lanes -> 4..8, warps -> 9..11     (contiguous only)
+// Each layout rotates its amplitude bits.  A pass visits ST of them:
+//   ST 1  c >= 8: P alone, no transpose
+//   ST 2  c = 4..7: Q, P (one transpose; the rotated bits 4..11 are two
+//         layouts' worth, so gathered tiles need no third one)
+//   ST 3  contiguous: Q, R, P (two)
+// A round-boundary pass starts at P, reaches Q, applies the phase there and
+// goes back the same way.
+//
+// Transposes go through the tile's own buffer.  P and Q access it in natural
+// order: 16 lanes cover bits 0..3, one 128-byte line, so 8-byte accesses are
+// conflict free, the amplitude bits are immediate offsets, and a thread writes
+// back the very slots it read -- one barrier a transpose.  R's 16-byte pairs
+// need the 128-byte swizzle (sw) on both sides.  Q and R hold the same 512
+// amplitudes per warp, so moving between them takes a warp barrier only.
+//
+// Shared-memory traffic, instructions and registers bound the adjoint, not
+// HBM: an earlier layout rotated {0, 9..11}, {1..4}, {5..8} for every tile and
+// so took two transposes (four at a round boundary) whatever was rotated.
+// n = 28, p = 8 gradient, float32 costs: 43.6 -> 38.9 ms; 4 sets of <C> at n = 24,
+// p = 10, uint8 costs: 4.68 -> 4.08 ms; 64 uneven gradients (n = 14..22, p = 6):
+// 7.69 -> 6.35 ms.
 //
 // Pipeline: warp 0 loads the tiles of this CTA with TMA copies into NBUF
 // shared-memory buffers (completion on one mbarrier per buffer; the tile's
-// descriptor index and base offset travel with it through the barrier); a
-// tile is transposed in place in its buffer, which goes back to the loader as
-// soon as its last stage has been read.
+// descriptor index and base offset travel with it through the barrier); the
+// buffer goes back to the loader as soon as its last layout has been read.
 constexpr int kT = kPassTileBits;
 constexpr int kTile = 1 << kT;
 constexpr int kNT = 256;
@@ -393,9 +411,6 @@ struct PassGeom {
     static constexpr uint32_t kCostB = kTile * (COST == 0 ? 4 : 1);
     static constexpr uint32_t kBufB = kPsiB * (BWD ? 2 : 1) + kCostB;
     static constexpr uint32_t kStashB = (BWD && COST == 0) ? kTile * 4 : 0;  // after the buffers
-    // single-buffered adjoint with float costs: buffer 0's cost slot and the
-    // stash make one vector's worth of transpose space (see tile_body)
-    static constexpr bool kEarly = BWD && COST == 0 && kCostB + kStashB == kPsiB;
     static constexpr uint32_t kHead = 256 + kPhaseTable * 8;  // barriers, tile info, phase table
 };
 
@@ -529,55 +544,106 @@ __device__ __forceinline__ void post_end(uint32_t bar, TileInfo *info) {
     }
 }
 
-// Constants of the descriptor currently being processed.
+// Warp 0: claim the next tile for a buffer and start its loads.
+template <int BWD, int COST, int NBUF>
+__device__ __forceinline__ void claim_issue(unsigned char *buf, uint32_t bar, uint32_t *sched, uint32_t total,
+                                            TileInfo *info, const PassDesc *__restrict__ descs,
+                                            const uint32_t *__restrict__ tile_begin, int ndesc, int &cursor,
+                                            const PassDesc *Ds, const uint32_t *s_tr) {
+    uint32_t tn = 0;
+    if ((threadIdx.x & 31) == 0) tn = (uint32_t)NBUF * gridDim.x + atomicAdd(sched, 1u);
+    tn = __shfl_sync(0xffffffffu, tn, 0);
+    if (tn < total) issue_tile<BWD, COST>(tn, buf, bar, info, descs, tile_begin, ndesc, cursor, Ds, s_tr);
+    else post_end(bar, info);
+}
+
+// Constants of the descriptor being processed, in shared memory (one per
+// round of a boundary pass).
 struct PassConst {
     Rot R;
     float ghi, glo, amp0;
     float c0;                  // adjoint: cost shift (C - c0 as the operator)
-    float fs1, fs2, fs3, fse;  // cos b factors per stage / per pass
-    uint32_t flags, active, g3, g1;
-    uint32_t rs3[4], rs1[3];
+    float fsq, fsr, fsp, fse;  // cos b factors of the Q, R and P rotations, and of all of them
+    uint32_t flags, mq, mp;    // pass flags; rotated amplitude bits in Q and P
     int rescale;
 };
 
-// One tile: stages 1..3, in-place transposes in buffer b, fused epilogue.
-// MODE is the rotation form (0 tan, 2 direct); the two forms are separate
-// copies of this body so the common one stays compact in the instruction
-// cache.  Optional work (initial state, phase, epilogue) sits in loops of its
-// own that are skipped as a whole when a pass does not need them.  PAT fixes
-// the stages' active-qubit masks at compile time as in the round-boundary
-// body (1: all twelve tile bits, 2: tile bits 4..11, 0: from the descriptor);
-// the forward passes use it, the adjoint ones would spill.
-template <int BWD, int COST, int NBUF, int MODE, int VAR, int PAT>
-__device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D, const float2 *stab,
-                                          const float4 *s_rot, const float4 *s_w,
-                                          unsigned char *bufs, int b, uint32_t bar, uint32_t *sched, int cost_free,
+// A thread's place in the three layouts (local index of amplitude 0) and where
+// its P amplitudes go: element g + (amplitude i) * rs of the tile, or for ST 1
+// the offsets of its four amplitude bits.
+struct ThreadPos {
+    uint32_t lp, lq, lr;
+};
+__device__ __forceinline__ ThreadPos thread_pos() {
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    return {lane | (warp << 5), (lane & 15u) | ((lane >> 4) << 8) | (warp << 9), (lane << 4) | (warp << 9)};
+}
+// The 128-byte swizzle: bits 1..3 flipped by bits 4..6 (16-byte pairs stay whole).
+__device__ __forceinline__ uint32_t sw(uint32_t l) { return l ^ (((l >> 4) & 7u) << 1); }
+
+template <int SWZ>
+__device__ __forceinline__ void get_p(float2 (&v)[16], const float2 *s, uint32_t lp) {
+    const float2 *q = s + (SWZ ? sw(lp) : lp);
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = q[i << 8];
+}
+template <int SWZ>
+__device__ __forceinline__ void put_p(const float2 (&v)[16], float2 *s, uint32_t lp) {
+    float2 *q = s + (SWZ ? sw(lp) : lp);
+#pragma unroll
+    for (int i = 0; i < 16; i++) q[i << 8] = v[i];
+}
+template <int SWZ>
+__device__ __forceinline__ void get_q(float2 (&v)[16], const float2 *s, uint32_t lq) {
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = s[(SWZ ? lq ^ ((i & 7) << 1) : lq) + (i << 4)];
+}
+template <int SWZ>
+__device__ __forceinline__ void put_q(const float2 (&v)[16], float2 *s, uint32_t lq) {
+#pragma unroll
+    for (int i = 0; i < 16; i++) s[(SWZ ? lq ^ ((i & 7) << 1) : lq) + (i << 4)] = v[i];
+}
+__device__ __forceinline__ void get_r(float2 (&v)[16], const float2 *s, uint32_t lr) {
+#pragma unroll
+    for (int r = 0; r < 8; r++) {
+        const float4 w = *reinterpret_cast<const float4 *>(s + (sw(lr) ^ (r << 1)));
+        v[2 * r] = make_float2(w.x, w.y);
+        v[2 * r + 1] = make_float2(w.z, w.w);
+    }
+}
+__device__ __forceinline__ void put_r(const float2 (&v)[16], float2 *s, uint32_t lr) {
+#pragma unroll
+    for (int r = 0; r < 8; r++)
+        *reinterpret_cast<float4 *>(s + (sw(lr) ^ (r << 1))) =
+            make_float4(v[2 * r].x, v[2 * r].y, v[2 * r + 1].x, v[2 * r + 1].y);
+}
+
+// Global element offset of local index l within a tile.
+__device__ __forceinline__ uint32_t tile_offset(uint32_t l, int c, int lo) {
+    return c >= kT ? l : ((l & ((1u << c) - 1u)) | ((l >> c) << lo));
+}
+
+// One tile: rotations in the layouts Q, R, P (see above), fused epilogue.
+// MODE is the rotation form (0 tan, 2 direct); the forms are separate copies
+// of this body so the common one stays compact in the instruction cache.
+// Optional work (initial state, phase, epilogue) sits in loops of its own that
+// are skipped as a whole when a pass does not need them.  QF: Q rotates all
+// four bits (c = 4 or contiguous), known at compile time.
+template <int BWD, int COST, int NBUF, int MODE, int VAR, int ST, int QF>
+__device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D, const uint32_t (&rs)[4], uint32_t gp,
+                                          const float2 *stab, const float4 *s_rot, const float4 *s_w,
+                                          unsigned char *bufs, int b, uint32_t bar, uint32_t *sched,
                                           uint32_t total, uint32_t base, uint32_t tl, TileInfo *tinfo,
                                           const PassDesc *__restrict__ descs,
                                           const uint32_t *__restrict__ tile_begin, int ndesc, int &cursor,
                                           const uint32_t *s_tr) {
     using G = PassGeom<BWD, COST>;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t l1 = ((uint32_t)lane << 1) | ((uint32_t)warp << 6);
-    const uint32_t l2 = ((uint32_t)lane & 1u) | ((((uint32_t)lane >> 1) & 7u) << 6) |
-                        ((((uint32_t)lane >> 4) & 1u) << 5) | ((uint32_t)warp << 9);
-    const uint32_t l3 = (uint32_t)lane | ((uint32_t)warp << 9);
-    const uint32_t p1 = swz(l1), p2 = swz(l2), p3 = swz(l3);
-    const uint32_t flags = K.flags, active = K.active;
-    const uint32_t m1 = PAT == 1 ? 0xFu : PAT == 2 ? 0xEu : stage_mask(active, 0, 9, 10, 11),
-                   m2 = PAT == 1 ? 0xFu : PAT == 2 ? 0x8u : stage_mask(active, 1, 2, 3, 4),
-                   m3 = PAT != 0 ? 0xFu : stage_mask(active, 5, 6, 7, 8);
-    // warp 0: claim the next tile for this buffer and start its loads
-    auto claim_issue = [&]() {
-        uint32_t tn = 0;
-        if (lane == 0) tn = (uint32_t)NBUF * gridDim.x + atomicAdd(sched, 1u);
-        tn = __shfl_sync(0xffffffffu, tn, 0);
-        if (tn < total)
-            issue_tile<BWD, COST>(tn, bufs + b * G::kBufB, bar, &tinfo[b], descs, tile_begin, ndesc, cursor, &D,
-                                  s_tr);
-        else
-            post_end(bar, &tinfo[b]);
-    };
+    const ThreadPos T = thread_pos();
+    const uint32_t lf = ST == 1 ? T.lp : T.lq;  // first layout
+    constexpr int kF = ST == 1 ? 8 : 4;
+    const uint32_t flags = K.flags;
+    const uint32_t mq = QF ? 0xFu : K.mq, mp = ST >= 2 ? 0xFu : K.mp;
 
     float2 *sp = reinterpret_cast<float2 *>(bufs + b * G::kBufB);
     float2 *sl = sp + kTile;
@@ -591,162 +657,87 @@ __device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D,
 #pragma unroll
     for (int j = 0; j < (MA ? 12 : 1); j++) bq[j] = 0.f;
 
-    // ---------------- stage 1: read the landed tile
+    // ---------------- read the landed tile
     if (!BWD && (flags & PF_GEN_INIT)) {
         if (GM) {  // the general mixer's passes keep plain amplitudes
 #pragma unroll
             for (int i = 0; i < 16; i++) a[i] = make_float2(K.amp0, 0.f);
         } else {
             // uniform state in the twisted basis: amp0 * (-i)^{|x|}, |x| = |base| + |local|
-            const float2 a0 = twist(make_float2(K.amp0, 0.f), __popc(base) + __popc(l1));
+            const float2 a0 = twist(make_float2(K.amp0, 0.f), __popc(base) + __popc(lf));
 #pragma unroll
-            for (int r = 0; r < 8; r++) {
-                a[2 * r] = twist(a0, __popc(r));
-                a[2 * r + 1] = twist(a0, __popc(r) + 1);
-            }
+            for (int i = 0; i < 16; i++) a[i] = twist(a0, __popc(i));
         }
     } else {
-#pragma unroll
-        for (int r = 0; r < 8; r++) {
-            const float4 v = *reinterpret_cast<const float4 *>(sp + (l1 | ((uint32_t)r << 9)));
-            a[2 * r] = make_float2(v.x, v.y);
-            a[2 * r + 1] = make_float2(v.z, v.w);
-        }
+        if (ST == 1) get_p<0>(a, sp, T.lp);
+        else get_q<0>(a, sp, T.lq);
         if (!GM && !BWD && (flags & PF_TWIST_IN)) {
-            const float2 w0 = twist(make_float2(1.f, 0.f), __popc(base) + __popc(l1));
+            const float2 w0 = twist(make_float2(1.f, 0.f), __popc(base) + __popc(lf));
 #pragma unroll
-            for (int r = 0; r < 8; r++) {
-                a[2 * r] = cmul(twist(a[2 * r], __popc(r)), w0);
-                a[2 * r + 1] = cmul(twist(a[2 * r + 1], __popc(r) + 1), w0);
-            }
+            for (int i = 0; i < 16; i++) a[i] = cmul(twist(a[i], __popc(i)), w0);
         }
     }
     if (BWD && !(flags & PF_LAM_FROM_C)) {
-#pragma unroll
-        for (int r = 0; r < 8; r++) {
-            const float4 v = *reinterpret_cast<const float4 *>(sl + (l1 | ((uint32_t)r << 9)));
-            l[2 * r] = make_float2(v.x, v.y);
-            l[2 * r + 1] = make_float2(v.z, v.w);
-        }
+        if (ST == 1) get_p<0>(l, sl, T.lp);
+        else get_q<0>(l, sl, T.lq);
     }
     if (BWD ? (flags & PF_LAM_FROM_C) : (flags & PF_PHASE)) {
 #pragma unroll
-        for (int r = 0; r < 8; r++) {
-            const uint32_t idx = l1 | ((uint32_t)r << 9);
-            float c0, c1;
-            if (COST == 0) {
-                const float2 cc = *reinterpret_cast<const float2 *>(reinterpret_cast<const float *>(scost) + idx);
-                c0 = cc.x;
-                c1 = cc.y;
-            } else {
-                const uchar2 cc = *reinterpret_cast<const uchar2 *>(scost + idx);
-                c0 = (float)cc.x;
-                c1 = (float)cc.y;
-                if (!BWD) {
-                    a[2 * r] = cmul(a[2 * r], stab[cc.x]);
-                    a[2 * r + 1] = cmul(a[2 * r + 1], stab[cc.y]);
-                }
-            }
+        for (int i = 0; i < 16; i++) {
+            const uint32_t ci = lf + ((uint32_t)i << kF);
+            const float C = COST == 0 ? reinterpret_cast<const float *>(scost)[ci] : (float)scost[ci];
             if (BWD) {
-                const float d0 = c0 - K.c0, d1 = c1 - K.c0;
-                l[2 * r] = __fmul2_rn(make_float2(d0, d0), a[2 * r]);
-                l[2 * r + 1] = __fmul2_rn(make_float2(d1, d1), a[2 * r + 1]);
-            } else if (COST == 0) {
-                a[2 * r] = cmul(a[2 * r], phase_f32(c0, K.ghi, K.glo));
-                a[2 * r + 1] = cmul(a[2 * r + 1], phase_f32(c1, K.ghi, K.glo));
+                const float d = C - K.c0;
+                l[i] = __fmul2_rn(make_float2(d, d), a[i]);
+            } else {
+                a[i] = cmul(a[i], COST == 0 ? phase_f32(C, K.ghi, K.glo) : stab[scost[ci]]);
             }
         }
     }
     if (GM && !BWD && (flags & PF_WDIAG)) {
-        // general X mixer: e^{-i b G(|x|)} on the global index x of every
-        // amplitude (local bits below c stay, the others start at qubit lo)
+        // general X mixer: e^{-i b G(|x|)} on the global index x of every amplitude
         const int c = D.c, lo = c < kT ? D.gpos[c] : 0;
 #pragma unroll
-        for (int r = 0; r < 8; r++) {
-            const uint32_t lq = l1 | ((uint32_t)r << 9);
-            const uint32_t x = base + (c >= kT ? lq : ((lq & ((1u << c) - 1u)) | ((lq >> c) << lo)));
-            const float4 t0 = s_w[__popc(x)], t1 = s_w[__popc(x | 1u)];
-            a[2 * r] = cmul(a[2 * r], make_float2(t0.x, t0.y));
-            a[2 * r + 1] = cmul(a[2 * r + 1], make_float2(t1.x, t1.y));
+        for (int i = 0; i < 16; i++) {
+            const float4 t = s_w[__popc(base + tile_offset(lf + ((uint32_t)i << kF), c, lo))];
+            a[i] = cmul(a[i], make_float2(t.x, t.y));
         }
     }
-    if constexpr (MA) stage_rot_ma<BWD, MODE, 0, 9, 10, 11>(a, l, stage_mask(active, 0, 9, 10, 11), s_rot, bq, pscale, true);
-    else stage_rot<BWD, MODE>(a, l, m1, K.R, pscale, bacc, true, !GM);
-    if (K.rescale) {
-        scale_all<BWD>(a, l, K.fs1);
-        pscale = 1.f;
-    }
-
-    // ---------------- stage 1 -> 2, in place (swizzled)
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        const uint32_t idx = p1 ^ swz((uint32_t)r << 9);
-        *reinterpret_cast<float4 *>(sp + idx) = make_float4(a[2 * r].x, a[2 * r].y, a[2 * r + 1].x, a[2 * r + 1].y);
-        if (BWD)
-            *reinterpret_cast<float4 *>(sl + idx) = make_float4(l[2 * r].x, l[2 * r].y, l[2 * r + 1].x, l[2 * r + 1].y);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        a[i] = sp[p2 ^ ((uint32_t)i << 1)];
-        if (BWD) l[i] = sl[p2 ^ ((uint32_t)i << 1)];
-    }
-    // A single-buffered adjoint tile that reads no cost hands its buffer back
-    // here, after the stage-2 read, and runs the warp-private stage 2 -> 3
-    // transpose through buffer 0's cost slot and the float-cost stash (32 KB),
-    // which no load writes while the launch reads no cost at all (cost_free).
-    // The next tile's loads then run under stages 2 and 3 instead of stage 3
-    // alone.
-    const bool early = G::kEarly && NBUF == 1 && cost_free && !needs_cost<BWD>(flags);
-    if (early) {
+    // ---------------- Q (and R), back through the buffer to P
+    if constexpr (ST >= 2) {
+        if constexpr (MA) stage_rot_ma<BWD, MODE, 4, 5, 6, 7>(a, l, mq, s_rot, bq, pscale, true);
+        else stage_rot<BWD, MODE>(a, l, mq, K.R, pscale, bacc, true, !GM);
+        if (K.rescale) {
+            scale_all<BWD>(a, l, K.fsq);
+            pscale = 1.f;
+        }
+        if constexpr (ST == 3) {
+            __syncwarp();  // the warp's 512 amplitudes are read: rewrite them swizzled
+            put_q<1>(a, sp, T.lq);
+            if (BWD) put_q<1>(l, sl, T.lq);
+            __syncwarp();
+            get_r(a, sp, T.lr);
+            if (BWD) get_r(l, sl, T.lr);
+            if constexpr (MA) stage_rot_ma<BWD, MODE, 0, 1, 2, 3>(a, l, 0xFu, s_rot, bq, pscale, true);
+            else stage_rot<BWD, MODE>(a, l, 0xFu, K.R, pscale, bacc, true, !GM);
+            if (K.rescale) {
+                scale_all<BWD>(a, l, K.fsr);
+                pscale = 1.f;
+            }
+            put_r(a, sp, T.lr);
+            if (BWD) put_r(l, sl, T.lr);
+        } else {
+            put_q<0>(a, sp, T.lq);
+            if (BWD) put_q<0>(l, sl, T.lq);
+        }
         __syncthreads();
-        if (warp == 0) claim_issue();
+        get_p<ST == 3>(a, sp, T.lp);
+        if (BWD) get_p<ST == 3>(l, sl, T.lp);
     }
-    if constexpr (MA) stage_rot_ma<BWD, MODE, 1, 2, 3, 4>(a, l, stage_mask(active, 1, 2, 3, 4), s_rot, bq, pscale, true);
-    else stage_rot<BWD, MODE>(a, l, m2, K.R, pscale, bacc, true, !GM);
-    if (K.rescale) {
-        scale_all<BWD>(a, l, K.fs2);
-        pscale = 1.f;
-    }
-
-    // ---------------- stage 2 -> 3: local bits 9..11 are the warp index in
-    // both layouts and the swizzle moves bits 1..3 only, so each warp reads
-    // back just what it wrote: a warp barrier is enough
-    if (G::kEarly && NBUF == 1 && early) {
-        // one vector at a time through the 32 KB behind buffer 0's vectors
-        float2 *scr = reinterpret_cast<float2 *>(bufs + 2 * G::kPsiB);
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 16; i++) scr[p2 ^ ((uint32_t)i << 1)] = a[i];
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 16; i++) a[i] = scr[p3 ^ swz((uint32_t)i << 5)];
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 16; i++) scr[p2 ^ ((uint32_t)i << 1)] = l[i];
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 16; i++) l[i] = scr[p3 ^ swz((uint32_t)i << 5)];
-    } else {
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 16; i++) {
-            sp[p2 ^ ((uint32_t)i << 1)] = a[i];
-            if (BWD) sl[p2 ^ ((uint32_t)i << 1)] = l[i];
-        }
-        __syncwarp();
-#pragma unroll
-        for (int i = 0; i < 16; i++) {
-            const uint32_t idx = p3 ^ swz((uint32_t)i << 5);
-            a[i] = sp[idx];
-            if (BWD) l[i] = sl[idx];
-        }
-    }
-    // Cost values of this thread's stage-3 amplitudes, read before the buffer
-    // goes back to the loader: uint8 costs packed four to a register; float
-    // costs of the adjoint copied to this thread's own slots of a stash that
-    // the loader never writes (16 live registers there cause spills).
+    // Cost values of this thread's P amplitudes, read before the buffer goes
+    // back to the loader: uint8 costs packed four to a register; float costs of
+    // the adjoint copied to this thread's own slots of a stash that the loader
+    // never writes (16 live registers there cause spills).
     const bool epi_c = BWD ? (flags & PF_PHASE) : (flags & PF_E);
     float cst[16];
     uint32_t cpk[4];
@@ -756,54 +747,54 @@ __device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D,
 #pragma unroll
             for (int q = 0; q < 4; q++) cpk[q] = 0u;
 #pragma unroll
-            for (int i = 0; i < 16; i++)
-                cpk[i >> 2] |= (uint32_t)scost[l3 | ((uint32_t)i << 5)] << (8 * (i & 3));
+            for (int i = 0; i < 16; i++) cpk[i >> 2] |= (uint32_t)scost[T.lp + (i << 8)] << (8 * (i & 3));
         } else if (BWD) {
 #pragma unroll
-            for (int i = 0; i < 16; i++) {
-                const uint32_t ci = l3 | ((uint32_t)i << 5);
-                stash[ci] = reinterpret_cast<const float *>(scost)[ci];
-            }
+            for (int i = 0; i < 16; i++)
+                stash[T.lp + (i << 8)] = reinterpret_cast<const float *>(scost)[T.lp + (i << 8)];
         } else {
 #pragma unroll
-            for (int i = 0; i < 16; i++)
-                cst[i] = reinterpret_cast<const float *>(scost)[l3 | ((uint32_t)i << 5)];
+            for (int i = 0; i < 16; i++) cst[i] = reinterpret_cast<const float *>(scost)[T.lp + (i << 8)];
         }
     }
     auto cost_at = [&](int i) -> float {
         if (COST == 1) return (float)((cpk[i >> 2] >> (8 * (i & 3))) & 255u);
-        if (BWD) return stash[l3 | ((uint32_t)i << 5)];
+        if (BWD) return stash[T.lp + (i << 8)];
         return cst[i];
     };
     // the buffer is consumed: start the tile NBUF ahead
-    if (!early) {
-        __syncthreads();
-        if (warp == 0) claim_issue();
-    }
-    // psi after the last stage is needed only when it is stored or meets the
+    __syncthreads();
+    if (warp == 0)
+        claim_issue<BWD, COST, NBUF>(bufs + b * G::kBufB, bar, sched, total, &tinfo[b], descs, tile_begin, ndesc,
+                                     cursor, &D, s_tr);
+    // psi after the last rotation is needed only when it is stored or meets the
     // phase epilogue (the adjoint with per-pass checkpoints stores lambda only)
     const bool psi_live = !BWD || D.psi_out != nullptr || (flags & PF_PHASE) || (GM && (flags & PF_WDIAG));
-    if constexpr (MA) stage_rot_ma<BWD, MODE, 5, 6, 7, 8>(a, l, stage_mask(active, 5, 6, 7, 8), s_rot, bq, pscale, psi_live);
-    else stage_rot<BWD, MODE>(a, l, m3, K.R, pscale, bacc, psi_live, !GM);
-    scale_all<BWD>(a, l, K.rescale ? K.fs3 : K.fse);
+    if constexpr (MA) stage_rot_ma<BWD, MODE, 8, 9, 10, 11>(a, l, mp, s_rot, bq, pscale, psi_live);
+    else stage_rot<BWD, MODE>(a, l, mp, K.R, pscale, bacc, psi_live, !GM);
+    scale_all<BWD>(a, l, K.rescale ? K.fsp : K.fse);
+
+    // ---------------- fused epilogue, coalesced store
+    // offset of amplitude i: i rs[0] where the four amplitude bits are
+    // consecutive global bits (ST >= 2)
+    auto off = [&](int i) -> uint32_t {
+        if (ST >= 2) return (uint32_t)i * rs[0];
+        return ((i & 1) ? rs[0] : 0) + ((i & 2) ? rs[1] : 0) + ((i & 4) ? rs[2] : 0) + ((i & 8) ? rs[3] : 0);
+    };
+    const uint32_t g = base + gp;
     if (GM && BWD && (flags & PF_WDIAG)) {
         // general X mixer: the beta partial sum_x G(|x|) Im(conj(lam) psi) in
         // the frame between the two half rounds, then the diagonal undone
-        const uint32_t g0 = base + K.g3;
         float wacc = 0.f;
 #pragma unroll
         for (int i = 0; i < 16; i++) {
-            const uint32_t x = g0 + (((i & 1) ? K.rs3[0] : 0) + ((i & 2) ? K.rs3[1] : 0) + ((i & 4) ? K.rs3[2] : 0) +
-                                     ((i & 8) ? K.rs3[3] : 0));
-            const float4 t = s_w[__popc(x)];
+            const float4 t = s_w[__popc(g + off(i))];
             wacc = fmaf(t.z, fmaf(l[i].x, a[i].y, -l[i].y * a[i].x), wacc);
             l[i] = cmul_conj(l[i], make_float2(t.x, t.y));
             if (D.psi_out) a[i] = cmul_conj(a[i], make_float2(t.x, t.y));
         }
         bacc += wacc;
     }
-
-    // ---------------- stage 3: fused epilogue, coalesced store
     float eacc = 0.f;
     if (epi_c) {
         if (!BWD) {
@@ -821,22 +812,15 @@ __device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D,
             }
         }
     }
-    const uint32_t g = base + K.g3;
     if (D.psi_out) {
         float2 *out = D.psi_out + g;
 #pragma unroll
-        for (int i = 0; i < 16; i++)
-            __stcs(out + (((i & 1) ? K.rs3[0] : 0) + ((i & 2) ? K.rs3[1] : 0) + ((i & 4) ? K.rs3[2] : 0) +
-                          ((i & 8) ? K.rs3[3] : 0)),
-                   a[i]);
+        for (int i = 0; i < 16; i++) __stcs(out + off(i), a[i]);
     }
     if (BWD && D.lam_out) {
         float2 *out = D.lam_out + g;
 #pragma unroll
-        for (int i = 0; i < 16; i++)
-            __stcs(out + (((i & 1) ? K.rs3[0] : 0) + ((i & 2) ? K.rs3[1] : 0) + ((i & 4) ? K.rs3[2] : 0) +
-                          ((i & 8) ? K.rs3[3] : 0)),
-                   l[i]);
+        for (int i = 0; i < 16; i++) __stcs(out + off(i), l[i]);
     }
     // per-warp partial sums: slot tile * 8 + warp (no block barrier)
     if (BWD) {
@@ -846,7 +830,7 @@ __device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D,
             for (int j = 0; j < 16; j++) v[j] = j < 12 ? bq[j < 12 ? j : 0] : 0.f;
             const float tb = warp_sum16_f(v);
             const uint32_t j = (uint32_t)lane >> 1;
-            if (!(lane & 1) && j < 12u && ((active >> j) & 1u) && D.part_beta)
+            if (!(lane & 1) && j < 12u && ((D.active >> j) & 1u) && D.part_beta)
                 D.part_beta[((size_t)j * D.ntiles + tl) * kNW + warp] = (double)tb;
             if (flags & PF_PHASE) {
                 const float tg = warp_sum_f(eacc);
@@ -864,22 +848,22 @@ __device__ __forceinline__ void tile_body(const PassConst &K, const PassDesc &D,
 }
 
 // Rotation and phase constants of one round for the tiles of a descriptor
-// (K.active must be set): rotation form, the cos factors per stage / per pass.
-__device__ __forceinline__ void set_round(PassConst &K, const RoundCoef &cf, float sgn) {
+// (K.mq and K.mp must be set): rotation form, the cos factors per layout and
+// of the whole pass.  `all`: a contiguous tile (R rotates its four bits too).
+__device__ __forceinline__ void set_round(PassConst &K, const RoundCoef &cf, float sgn, bool all) {
+    const bool tan = cf.bmode == 0;
     K.R.mode = cf.bmode;
     K.R.tt = make_float2(sgn * cf.bt, sgn * cf.bt);
     K.R.ntt = make_float2(-sgn * cf.bt, -sgn * cf.bt);
     K.R.c = cf.cb;
     K.R.s = sgn * cf.sb;
-    K.R.psc = cf.bmode == 0 ? cf.cb * cf.cb : 1.f;
-    K.rescale = (cf.bmode == 0 && cf.rescale) ? 1 : 0;
-    const float c = cf.bmode == 0 ? cf.cb : 1.f;
-    const int k1 = __popc(K.active & 0xE01u), k2 = __popc(K.active & 0x1Eu), k3 = __popc(K.active & 0x1E0u);
-    K.fs1 = K.fs2 = K.fs3 = 1.f;
-    for (int k = 0; k < k1; k++) K.fs1 *= c;
-    for (int k = 0; k < k2; k++) K.fs2 *= c;
-    for (int k = 0; k < k3; k++) K.fs3 *= c;
-    K.fse = K.rescale ? 1.f : K.fs1 * K.fs2 * K.fs3;
+    K.R.psc = tan ? cf.pw[2] : 1.f;
+    K.rescale = (tan && cf.rescale) ? 1 : 0;
+    const int nq = __popc(K.mq), np = __popc(K.mp), nr = all ? 4 : 0;
+    K.fsq = tan ? cf.pw[nq] : 1.f;
+    K.fsr = tan ? cf.pw[nr] : 1.f;
+    K.fsp = tan ? cf.pw[np] : 1.f;
+    K.fse = tan && !K.rescale ? cf.pw[nq + nr + np] : 1.f;
     K.ghi = cf.g_hi;
     K.glo = cf.g_lo;
 }
@@ -888,182 +872,123 @@ __device__ __forceinline__ void set_round(PassConst &K, const RoundCoef &cf, flo
 // of round k and the first of round k+1, so one pass applies round k's
 // rotations, the phase of round k+1 and round k+1's rotations (forward), or
 // undoes them in reverse order with both rounds' pair terms and the gamma
-// partial in between (adjoint).  The register stages run 1 -> 2 -> 3, the
-// phase at stage 3 (cost values in the tile buffer, natural order), then back
-// 3 -> 2 -> 1 through the inverse transposes, and the result is stored from
-// the stage-1 (load) layout as 16-byte pairs.  KA is the round applied first
-// (forward: k; adjoint: k+1), KB the second; KP holds the phase (round k+1).
-// PAT fixes the stages' active-qubit masks at compile time for the two groups
-// the default schedules use most: 1 = all twelve tile bits (the contiguous
-// group), 2 = tile bits 4..11 (a gathered group with four contiguous bits);
-// 0 takes them from the descriptor.
-template <int BWD, int COST, int NBUF, int MA, int MB, int PAT>
+// partial in between (adjoint).  The layouts run P, R, Q, the phase at Q (P
+// for ST 1; cost values in the tile buffer, natural order), then Q, R, P.  KA
+// is the round applied first (forward: k; adjoint: k+1), KB the second; KP
+// holds the phase (round k+1).
+template <int BWD, int COST, int NBUF, int MA, int MB, int ST, int QF>
 __device__ __forceinline__ void tile_body_fused_impl(const PassConst &KA, const PassConst &KB, const PassConst &KP,
-                                                uint32_t g1, const uint32_t (&rs1)[3],
-                                                const PassDesc &D, const float2 *stab, unsigned char *bufs, int b,
-                                                uint32_t bar, uint32_t *sched, uint32_t total, uint32_t base,
-                                                uint32_t tl, TileInfo *tinfo, const PassDesc *__restrict__ descs,
-                                                const uint32_t *__restrict__ tile_begin, int ndesc, int &cursor,
-                                                const uint32_t *s_tr) {
+                                                     const uint32_t (&rs)[4], uint32_t gp,
+                                                     const PassDesc &D, const float2 *stab, unsigned char *bufs, int b,
+                                                     uint32_t bar, uint32_t *sched, uint32_t total, uint32_t base,
+                                                     uint32_t tl, TileInfo *tinfo, const PassDesc *__restrict__ descs,
+                                                     const uint32_t *__restrict__ tile_begin, int ndesc, int &cursor,
+                                                     const uint32_t *s_tr) {
     using G = PassGeom<BWD, COST>;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const uint32_t l1 = ((uint32_t)lane << 1) | ((uint32_t)warp << 6);
-    const uint32_t l2 = ((uint32_t)lane & 1u) | ((((uint32_t)lane >> 1) & 7u) << 6) |
-                        ((((uint32_t)lane >> 4) & 1u) << 5) | ((uint32_t)warp << 9);
-    const uint32_t l3 = (uint32_t)lane | ((uint32_t)warp << 9);
-    const uint32_t p1 = swz(l1), p2 = swz(l2), p3 = swz(l3);
-    const uint32_t active = KA.active;
+    const ThreadPos T = thread_pos();
     float2 *sp = reinterpret_cast<float2 *>(bufs + b * G::kBufB);
     float2 *sl = sp + kTile;
     const unsigned char *scost = bufs + b * G::kBufB + G::kPsiB * (BWD ? 2 : 1);
     float2 a[16], l[16];
     float pscale = 1.f, bA = 0.f, bB = 0.f, eacc = 0.f;
-    const uint32_t m1 = PAT == 1 ? 0xFu : PAT == 2 ? 0xEu : stage_mask(active, 0, 9, 10, 11),
-                   m2 = PAT == 1 ? 0xFu : PAT == 2 ? 0x8u : stage_mask(active, 1, 2, 3, 4),
-                   m3 = PAT != 0 ? 0xFu : stage_mask(active, 5, 6, 7, 8);
+    const uint32_t mq = QF ? 0xFu : KA.mq, mp = ST >= 2 ? 0xFu : KA.mp;
 
-    // ---------------- stage 1: read the landed tile
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        const float4 v = *reinterpret_cast<const float4 *>(sp + (l1 | ((uint32_t)r << 9)));
-        a[2 * r] = make_float2(v.x, v.y);
-        a[2 * r + 1] = make_float2(v.z, v.w);
-        if (BWD) {
-            const float4 w = *reinterpret_cast<const float4 *>(sl + (l1 | ((uint32_t)r << 9)));
-            l[2 * r] = make_float2(w.x, w.y);
-            l[2 * r + 1] = make_float2(w.z, w.w);
+    // ---------------- round A: P, R, Q
+    get_p<0>(a, sp, T.lp);
+    if (BWD) get_p<0>(l, sl, T.lp);
+    stage_rot<BWD, MA>(a, l, mp, KA.R, pscale, bA, true);
+    if constexpr (ST >= 2) {
+        if (KA.rescale) {
+            scale_all<BWD>(a, l, KA.fsp);
+            pscale = 1.f;
         }
+        if (ST == 3) __syncwarp();  // swizzled slots: those of the same 16 lanes
+        put_p<ST == 3>(a, sp, T.lp);
+        if (BWD) put_p<ST == 3>(l, sl, T.lp);
+        __syncthreads();
+        if constexpr (ST == 3) {
+            get_r(a, sp, T.lr);
+            if (BWD) get_r(l, sl, T.lr);
+            stage_rot<BWD, MA>(a, l, 0xFu, KA.R, pscale, bA, true);
+            if (KA.rescale) {
+                scale_all<BWD>(a, l, KA.fsr);
+                pscale = 1.f;
+            }
+            put_r(a, sp, T.lr);
+            if (BWD) put_r(l, sl, T.lr);
+            __syncwarp();
+        }
+        get_q<ST == 3>(a, sp, T.lq);
+        if (BWD) get_q<ST == 3>(l, sl, T.lq);
+        stage_rot<BWD, MA>(a, l, mq, KA.R, pscale, bA, true);
     }
-    // ---------------- round A, stages 1 -> 2 -> 3
-    stage_rot<BWD, MA>(a, l, m1, KA.R, pscale, bA, true);
-    if (KA.rescale) {
-        scale_all<BWD>(a, l, KA.fs1);
-        pscale = 1.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        const uint32_t idx = p1 ^ swz((uint32_t)r << 9);
-        *reinterpret_cast<float4 *>(sp + idx) = make_float4(a[2 * r].x, a[2 * r].y, a[2 * r + 1].x, a[2 * r + 1].y);
-        if (BWD)
-            *reinterpret_cast<float4 *>(sl + idx) = make_float4(l[2 * r].x, l[2 * r].y, l[2 * r + 1].x, l[2 * r + 1].y);
-    }
-    __syncthreads();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        a[i] = sp[p2 ^ ((uint32_t)i << 1)];
-        if (BWD) l[i] = sl[p2 ^ ((uint32_t)i << 1)];
-    }
-    stage_rot<BWD, MA>(a, l, m2, KA.R, pscale, bA, true);
-    if (KA.rescale) {
-        scale_all<BWD>(a, l, KA.fs2);
-        pscale = 1.f;
-    }
-    // stage 2 -> 3 inside each warp's 512 amplitudes
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        sp[p2 ^ ((uint32_t)i << 1)] = a[i];
-        if (BWD) sl[p2 ^ ((uint32_t)i << 1)] = l[i];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        const uint32_t idx = p3 ^ swz((uint32_t)i << 5);
-        a[i] = sp[idx];
-        if (BWD) l[i] = sl[idx];
-    }
-    stage_rot<BWD, MA>(a, l, m3, KA.R, pscale, bA, true);
-    scale_all<BWD>(a, l, KA.rescale ? KA.fs3 : KA.fse);
+    scale_all<BWD>(a, l, KA.rescale ? (ST >= 2 ? KA.fsq : KA.fsp) : KA.fse);
     pscale = 1.f;
 
     // ---------------- the phase of round k+1 between the two rounds
+    {
+        const uint32_t lx = ST == 1 ? T.lp : T.lq;
+        constexpr int kX = ST == 1 ? 8 : 4;
 #pragma unroll
-    for (int i = 0; i < 16; i++) {
-        const uint32_t ci = l3 | ((uint32_t)i << 5);
-        const float C = COST == 0 ? reinterpret_cast<const float *>(scost)[ci] : (float)scost[ci];
-        const float2 ph = COST == 0 ? phase_f32(C, KP.ghi, KP.glo) : stab[scost[ci]];
-        if (BWD) {
-            eacc = fmaf(C - KP.c0, fmaf(l[i].x, a[i].y, -l[i].y * a[i].x), eacc);
-            l[i] = cmul_conj(l[i], ph);
-            a[i] = cmul_conj(a[i], ph);
-        } else {
-            a[i] = cmul(a[i], ph);
+        for (int i = 0; i < 16; i++) {
+            const uint32_t ci = lx + ((uint32_t)i << kX);
+            const float C = COST == 0 ? reinterpret_cast<const float *>(scost)[ci] : (float)scost[ci];
+            const float2 ph = COST == 0 ? phase_f32(C, KP.ghi, KP.glo) : stab[scost[ci]];
+            if (BWD) {
+                eacc = fmaf(C - KP.c0, fmaf(l[i].x, a[i].y, -l[i].y * a[i].x), eacc);
+                l[i] = cmul_conj(l[i], ph);
+                a[i] = cmul_conj(a[i], ph);
+            } else {
+                a[i] = cmul(a[i], ph);
+            }
         }
     }
 
-    // ---------------- round B, stages 3 -> 2 -> 1
-    stage_rot<BWD, MB>(a, l, m3, KB.R, pscale, bB, true);
-    if (KB.rescale) {
-        scale_all<BWD>(a, l, KB.fs3);
-        pscale = 1.f;
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        const uint32_t idx = p3 ^ swz((uint32_t)i << 5);
-        sp[idx] = a[i];
-        if (BWD) sl[idx] = l[i];
-    }
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        a[i] = sp[p2 ^ ((uint32_t)i << 1)];
-        if (BWD) l[i] = sl[p2 ^ ((uint32_t)i << 1)];
-    }
-    stage_rot<BWD, MB>(a, l, m2, KB.R, pscale, bB, true);
-    if (KB.rescale) {
-        scale_all<BWD>(a, l, KB.fs2);
-        pscale = 1.f;
-    }
-    // stage 2 -> 1: each warp rewrites its own 512 amplitudes, then all read across warps
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < 16; i++) {
-        sp[p2 ^ ((uint32_t)i << 1)] = a[i];
-        if (BWD) sl[p2 ^ ((uint32_t)i << 1)] = l[i];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int r = 0; r < 8; r++) {
-        const uint32_t idx = p1 ^ swz((uint32_t)r << 9);
-        const float4 v = *reinterpret_cast<const float4 *>(sp + idx);
-        a[2 * r] = make_float2(v.x, v.y);
-        a[2 * r + 1] = make_float2(v.z, v.w);
-        if (BWD) {
-            const float4 w = *reinterpret_cast<const float4 *>(sl + idx);
-            l[2 * r] = make_float2(w.x, w.y);
-            l[2 * r + 1] = make_float2(w.z, w.w);
+    // ---------------- round B: Q, R, P
+    if constexpr (ST >= 2) {
+        stage_rot<BWD, MB>(a, l, mq, KB.R, pscale, bB, true);
+        if (KB.rescale) {
+            scale_all<BWD>(a, l, KB.fsq);
+            pscale = 1.f;
         }
+        put_q<ST == 3>(a, sp, T.lq);
+        if (BWD) put_q<ST == 3>(l, sl, T.lq);
+        if constexpr (ST == 3) {
+            __syncwarp();
+            get_r(a, sp, T.lr);
+            if (BWD) get_r(l, sl, T.lr);
+            stage_rot<BWD, MB>(a, l, 0xFu, KB.R, pscale, bB, true);
+            if (KB.rescale) {
+                scale_all<BWD>(a, l, KB.fsr);
+                pscale = 1.f;
+            }
+            put_r(a, sp, T.lr);
+            if (BWD) put_r(l, sl, T.lr);
+        }
+        __syncthreads();
+        get_p<ST == 3>(a, sp, T.lp);
+        if (BWD) get_p<ST == 3>(l, sl, T.lp);
     }
     // the buffer is consumed: start the tile NBUF ahead
     __syncthreads();
-    if (warp == 0) {
-        uint32_t tn = 0;
-        if (lane == 0) tn = (uint32_t)NBUF * gridDim.x + atomicAdd(sched, 1u);
-        tn = __shfl_sync(0xffffffffu, tn, 0);
-        if (tn < total)
-            issue_tile<BWD, COST>(tn, bufs + b * G::kBufB, bar, &tinfo[b], descs, tile_begin, ndesc, cursor, &D,
-                                  s_tr);
-        else
-            post_end(bar, &tinfo[b]);
-    }
-    // psi is dead after the last adjoint stage
-    stage_rot<BWD, MB>(a, l, m1, KB.R, pscale, bB, !BWD);
-    scale_all<BWD>(a, l, KB.rescale ? KB.fs1 : KB.fse);
-
-    // ---------------- store from the stage-1 layout: 16-byte amplitude pairs
-    {
-        float2 *out = BWD ? D.lam_out : D.psi_out;
-        if (out) {
-            const float2 *v = BWD ? l : a;
-            out += base + g1;
+    if (warp == 0)
+        claim_issue<BWD, COST, NBUF>(bufs + b * G::kBufB, bar, sched, total, &tinfo[b], descs, tile_begin, ndesc,
+                                     cursor, &D, s_tr);
+    // psi is dead after the last adjoint pair terms
+    stage_rot<BWD, MB>(a, l, mp, KB.R, pscale, bB, !BWD);
+    if (BWD) scale_all<0>(l, l, KB.rescale ? KB.fsp : KB.fse);
+    else scale_all<0>(a, a, KB.rescale ? KB.fsp : KB.fse);
+    float2 *out = BWD ? D.lam_out : D.psi_out;
+    if (out) {
+        const float2 *v = BWD ? l : a;
+        out += base + gp;
 #pragma unroll
-            for (int r = 0; r < 8; r++) {
-                const uint32_t o = ((r & 1) ? rs1[0] : 0u) + ((r & 2) ? rs1[1] : 0u) + ((r & 4) ? rs1[2] : 0u);
-                __stcs(reinterpret_cast<float4 *>(out + o),
-                       make_float4(v[2 * r].x, v[2 * r].y, v[2 * r + 1].x, v[2 * r + 1].y));
-            }
+        for (int i = 0; i < 16; i++) {
+            const uint32_t o = ST >= 2 ? (uint32_t)i * rs[0]
+                                       : ((i & 1) ? rs[0] : 0u) + ((i & 2) ? rs[1] : 0u) + ((i & 4) ? rs[2] : 0u) +
+                                             ((i & 8) ? rs[3] : 0u);
+            __stcs(out + o, v[i]);
         }
     }
     if (BWD) {  // round k+1's beta total in lane 0, round k's in lane 16; gamma by its own tree
@@ -1075,37 +1000,31 @@ __device__ __forceinline__ void tile_body_fused_impl(const PassConst &KA, const 
     }
 }
 
-// The common case (both rounds in the tan form, a mask pattern known at
-// compile time) inline; the direct form (|cos b| tiny, rare) and other
-// groups out of line, so that their registers do not set the register
-// allocation of the common path.
-template <int BWD, int COST, int NBUF, int MA, int MB, int PAT>
-__device__ __forceinline__ void tile_body_fused(const PassConst &KA, const PassConst &KB, const PassConst &KP,
-                                                uint32_t g1, const uint32_t (&rs1)[3],
-                                                const PassDesc &D, const float2 *stab, unsigned char *bufs, int b,
-                                                uint32_t bar, uint32_t *sched, uint32_t total, uint32_t base,
-                                                uint32_t tl, TileInfo *tinfo, const PassDesc *__restrict__ descs,
-                                                const uint32_t *__restrict__ tile_begin, int ndesc, int &cursor,
-                                                const uint32_t *s_tr) {
-    tile_body_fused_impl<BWD, COST, NBUF, MA, MB, PAT>(KA, KB, KP, g1, rs1, D, stab, bufs, b, bar, sched, total,
-                                                       base, tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
+// The common case (both rounds in the tan form) inline; the direct form
+// (|cos b| tiny, rare) out of line, so that its registers do not set the
+// register allocation of the common path.
+template <int BWD, int COST, int NBUF, int MA, int MB, int ST, int QF, class... Args>
+__device__ __forceinline__ void tile_body_fused(Args &&...args) {
+    tile_body_fused_impl<BWD, COST, NBUF, MA, MB, ST, QF>(args...);
 }
-template <int BWD, int COST, int NBUF, int MA, int MB>
+template <int BWD, int COST, int NBUF, int MA, int MB, int ST>
 __device__ __noinline__ void tile_body_fused_rare(const PassConst &KA, const PassConst &KB, const PassConst &KP,
-                                                  uint32_t g1, const uint32_t (&rs1)[3],
+                                                  const uint32_t (&rs)[4], uint32_t gp,
                                                   const PassDesc &D, const float2 *stab, unsigned char *bufs, int b,
                                                   uint32_t bar, uint32_t *sched, uint32_t total, uint32_t base,
                                                   uint32_t tl, TileInfo *tinfo, const PassDesc *__restrict__ descs,
                                                   const uint32_t *__restrict__ tile_begin, int ndesc, int &cursor,
                                                   const uint32_t *s_tr) {
-    tile_body_fused_impl<BWD, COST, NBUF, MA, MB, 0>(KA, KB, KP, g1, rs1, D, stab, bufs, b, bar, sched, total, base,
-                                                     tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
+    tile_body_fused_impl<BWD, COST, NBUF, MA, MB, ST, 0>(KA, KB, KP, rs, gp, D, stab, bufs, b, bar, sched, total,
+                                                         base, tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
 }
 
-template <int BWD, int COST, int NBUF, int VAR, int FUSED>
+// GATH: the launch's tiles are gathered ones (ST 1 or 2 by descriptor), else
+// contiguous (ST 3).
+template <int BWD, int COST, int NBUF, int VAR, int FUSED, int GATH>
 __global__ void __launch_bounds__(kNT, (BWD && NBUF > 1) ? 1 : 2)
 xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ tile_begin, int ndesc,
-             uint32_t total, int *err, uint32_t *__restrict__ sched, int cost_free) {
+             uint32_t total, int *err, uint32_t *__restrict__ sched) {
     using G = PassGeom<BWD, COST>;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem_raw);
@@ -1116,9 +1035,9 @@ xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ ti
     __shared__ float4 s_rot[12];  // multi-angle: (cos, +-sin, +-tan, cos^2) per local bit
     __shared__ float4 s_w[33];    // general X mixer: weight phases and G(w)
     __shared__ uint32_t s_tr[3];  // D's first tile, end tile and index
-    __shared__ PassConst s_kf[2];  // round-boundary launches: rounds k and k+1 (uniform fields)
+    __shared__ PassConst s_k[2];  // the round's constants (round-boundary launches: rounds k and k+1)
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5;
     if (tid == 0) {
         for (int b = 0; b < NBUF; b++) mbar_init(smem_u32(&bars[b]), 1);
         fence_mbar_init();
@@ -1136,9 +1055,8 @@ xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ ti
                 post_end(smem_u32(&bars[k]), &tinfo[k]);
         }
     }
-    const uint32_t l3 = (uint32_t)lane | ((uint32_t)warp << 9);
     int cur = -1;
-    PassConst K;
+    uint32_t gp = 0, rs[4] = {0, 0, 0, 0};
 
     for (uint32_t it = 0;; it++) {
         const int b = (int)(it % NBUF);
@@ -1167,121 +1085,105 @@ xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ ti
                 s_tr[2] = (uint32_t)di;
             }
             __syncthreads();
-            K.flags = D.flags;
-            K.active = D.active;
-            K.amp0 = D.amp0;
             // undoing a round (adjoint) uses the coefficients of -b
             const float sgn = BWD ? -1.f : 1.f;
-            set_round(K, *D.coef, sgn);
-            K.c0 = (BWD && D.c0 && (K.flags & (PF_LAM_FROM_C | PF_PHASE | PF_FUSED))) ? (float)*D.c0 : 0.f;
-            K.g3 = 0;
-            for (int j = 0; j < kT; j++)
-                if ((l3 >> j) & 1u) K.g3 += 1u << D.gpos[j];
-#pragma unroll
-            for (int k = 0; k < 4; k++) K.rs3[k] = 1u << D.gpos[5 + k];
-            if (FUSED) {  // stage-1 store offsets (round-boundary passes)
-                const uint32_t l1s = ((uint32_t)lane << 1) | ((uint32_t)warp << 6);
-                K.g1 = 0;
-                for (int j = 1; j < 9; j++)
-                    if ((l1s >> j) & 1u) K.g1 += 1u << D.gpos[j];
-#pragma unroll
-                for (int k = 0; k < 3; k++) K.rs1[k] = 1u << D.gpos[9 + k];
+            if (tid < (FUSED ? 2 : 1)) {
+                PassConst K;
+                K.flags = D.flags;
+                K.mq = (D.active >> 4) & 0xFu;
+                K.mp = (D.active >> 8) & 0xFu;
+                K.amp0 = D.amp0;
+                K.c0 = (BWD && D.c0 && (D.flags & (PF_LAM_FROM_C | PF_PHASE | PF_FUSED))) ? (float)*D.c0 : 0.f;
+                set_round(K, tid ? *D.coef2 : *D.coef, sgn, D.c >= kT);
+                s_k[tid] = K;
             }
-            if (FUSED && tid == 0) {  // both rounds of a boundary pass, for every thread
-                PassConst K2 = K;
-                set_round(K2, *D.coef2, sgn);
-                s_kf[0] = K;
-                s_kf[1] = K2;
-            }
-            if (COST == 1 && (K.flags & (PF_PHASE | PF_FUSED)))
+            gp = tile_offset(thread_pos().lp, D.c, D.c < kT ? D.gpos[D.c] : 0);
+#pragma unroll
+            for (int k = 0; k < 4; k++) rs[k] = 1u << D.gpos[8 + k];
+            if (COST == 1 && (D.flags & (PF_PHASE | PF_FUSED)))
                 for (int i = tid; i < kPhaseTable; i += kNT) stab[i] = D.table[i];
-            if (VAR == 2 && (K.flags & PF_WDIAG))
+            if (VAR == 2 && (D.flags & PF_WDIAG))
                 for (int i = tid; i <= D.n; i += kNT) s_w[i] = D.wtab[i];
             if (VAR == 1) {
                 // per-qubit rotations: D.coef is this round's n entries, indexed
                 // by global qubit.  The tan form when every rotated qubit allows
-                // it, with the cosines per stage (rescale: any |cos| < 1/4) or
+                // it, with the cosines per layout (rescale: any |cos| < 1/4) or
                 // once per pass, else the direct form.
                 bool tan_ok = true, resc = false;
                 if (tid < kT) {
-                    const RoundCoef q = D.coef[D.gpos[tid]];
-                    s_rot[tid] = make_float4(q.cb, sgn * q.sb, sgn * q.bt, q.cb * q.cb);
-                    const bool on = (K.active >> tid) & 1u;
+                    const RoundCoef &q = D.coef[D.gpos[tid]];
+                    const float c = q.bmode == 0 ? q.pw[1] : q.cb;
+                    s_rot[tid] = make_float4(q.cb, sgn * q.sb, sgn * q.bt, c * c);
+                    const bool on = (D.active >> tid) & 1u;
                     tan_ok = !on || q.bmode == 0;
                     resc = on && q.rescale;
                 }
                 tan_ok = __syncthreads_and(tan_ok);
                 resc = __syncthreads_or(resc) && tan_ok;
-                auto prod = [&](int b0, int b1, int b2, int b3) {
-                    float f = 1.f;
-                    const int bs[4] = {b0, b1, b2, b3};
-                    for (int j = 0; j < 4; j++)
-                        if ((K.active >> bs[j]) & 1u) f *= s_rot[bs[j]].x;
-                    return tan_ok ? f : 1.f;
-                };
-                K.R.mode = tan_ok ? 0 : 2;
-                K.rescale = resc ? 1 : 0;
-                K.fs1 = prod(0, 9, 10, 11);
-                K.fs2 = prod(1, 2, 3, 4);
-                K.fs3 = prod(5, 6, 7, 8);
-                K.fse = K.rescale ? 1.f : K.fs1 * K.fs2 * K.fs3;
+                if (tid == 0) {
+                    auto prod = [&](int b0) {
+                        float f = 1.f;
+                        for (int j = b0; j < b0 + 4; j++)
+                            if ((D.active >> j) & 1u) f *= D.coef[D.gpos[j]].pw[1];
+                        return tan_ok ? f : 1.f;
+                    };
+                    PassConst &K = s_k[0];
+                    K.R.mode = tan_ok ? 0 : 2;
+                    K.rescale = resc ? 1 : 0;
+                    K.fsq = prod(4);
+                    K.fsr = prod(0);
+                    K.fsp = prod(8);
+                    K.fse = resc ? 1.f : K.fsq * K.fsr * K.fsp;
+                }
             }
             __syncthreads();
             cur = di;
         }
+        const int c = D.c;
         if constexpr (FUSED) {
             // forward: round k then round k+1; adjoint: k+1 first; the phase is round k+1's
-            const PassConst &KA = s_kf[BWD ? 1 : 0], &KB = s_kf[BWD ? 0 : 1], &KP = s_kf[1];
+            const PassConst &KA = s_k[BWD ? 1 : 0], &KB = s_k[BWD ? 0 : 1], &KP = s_k[1];
             const int mk = (KA.R.mode == 0 ? 0 : 1) | (KB.R.mode == 0 ? 0 : 2);
-            if (mk == 0 && KA.active == 0xFFFu)
-                tile_body_fused<BWD, COST, NBUF, 0, 0, 1>(KA, KB, KP, K.g1, K.rs1, D, stab, bufs, b, bar, sched,
-                                                          total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,
-                                                          cursor, s_tr);
-            else if (mk == 0 && KA.active == 0xFF0u)
-                tile_body_fused<BWD, COST, NBUF, 0, 0, 2>(KA, KB, KP, K.g1, K.rs1, D, stab, bufs, b, bar, sched,
-                                                          total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,
-                                                          cursor, s_tr);
-            else if (mk == 0)
-                tile_body_fused_rare<BWD, COST, NBUF, 0, 0>(KA, KB, KP, K.g1, K.rs1, D, stab, bufs, b, bar, sched,
-                                                            total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,
-                                                            cursor, s_tr);
-            else if (mk == 1)
-                tile_body_fused_rare<BWD, COST, NBUF, 2, 0>(KA, KB, KP, K.g1, K.rs1, D, stab, bufs, b, bar, sched,
-                                                            total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,
-                                                            cursor, s_tr);
-            else if (mk == 2)
-                tile_body_fused_rare<BWD, COST, NBUF, 0, 2>(KA, KB, KP, K.g1, K.rs1, D, stab, bufs, b, bar, sched,
-                                                            total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,
-                                                            cursor, s_tr);
-            else
-                tile_body_fused_rare<BWD, COST, NBUF, 2, 2>(KA, KB, KP, K.g1, K.rs1, D, stab, bufs, b, bar, sched,
-                                                            total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,
-                                                            cursor, s_tr);
-        } else if constexpr (VAR == 0 && !BWD) {  // (adjoint copies spill: measured slower)
-            if (K.R.mode == 0 && K.active == 0xFFFu)
-                tile_body<BWD, COST, NBUF, 0, 0, 1>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total,
-                                                    ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-            else if (K.R.mode == 0 && K.active == 0xFF0u)
-                tile_body<BWD, COST, NBUF, 0, 0, 2>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total,
-                                                    ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-            else if (K.R.mode == 0)
-                tile_body<BWD, COST, NBUF, 0, 0, 0>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total,
-                                                    ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-            else
-                tile_body<BWD, COST, NBUF, 2, 0, 0>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total,
-                                                    ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-        } else if (VAR == 1 && K.R.mode == 0)
-            tile_body<BWD, COST, NBUF, 0, 1, 0>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total, ti.base,
-                                                ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-        else if (VAR == 1)
-            tile_body<BWD, COST, NBUF, 2, 1, 0>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total, ti.base,
-                                                ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-        else if (K.R.mode == 0)
-            tile_body<BWD, COST, NBUF, 0, VAR, 0>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total,
-                                                  ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
-        else
-            tile_body<BWD, COST, NBUF, 2, VAR, 0>(K, D, stab, s_rot, s_w, bufs, b, bar, sched, cost_free, total,
-                                                  ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, s_tr);
+#define QG_FUSED_ARGS                                                                                                \
+    KA, KB, KP, rs, gp, D, stab, bufs, b, bar, sched, total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc, cursor, \
+        s_tr
+            if constexpr (!GATH) {
+                if (mk == 0) tile_body_fused<BWD, COST, NBUF, 0, 0, 3, 1>(QG_FUSED_ARGS);
+                else if (mk == 1) tile_body_fused_rare<BWD, COST, NBUF, 2, 0, 3>(QG_FUSED_ARGS);
+                else if (mk == 2) tile_body_fused_rare<BWD, COST, NBUF, 0, 2, 3>(QG_FUSED_ARGS);
+                else tile_body_fused_rare<BWD, COST, NBUF, 2, 2, 3>(QG_FUSED_ARGS);
+            } else if (c >= 8) {
+                if (mk == 0) tile_body_fused<BWD, COST, NBUF, 0, 0, 1, 0>(QG_FUSED_ARGS);
+                else if (mk == 1) tile_body_fused_rare<BWD, COST, NBUF, 2, 0, 1>(QG_FUSED_ARGS);
+                else if (mk == 2) tile_body_fused_rare<BWD, COST, NBUF, 0, 2, 1>(QG_FUSED_ARGS);
+                else tile_body_fused_rare<BWD, COST, NBUF, 2, 2, 1>(QG_FUSED_ARGS);
+            } else {
+                if (mk == 0 && c == 4) tile_body_fused<BWD, COST, NBUF, 0, 0, 2, 1>(QG_FUSED_ARGS);
+                else if (mk == 0) tile_body_fused<BWD, COST, NBUF, 0, 0, 2, 0>(QG_FUSED_ARGS);
+                else if (mk == 1) tile_body_fused_rare<BWD, COST, NBUF, 2, 0, 2>(QG_FUSED_ARGS);
+                else if (mk == 2) tile_body_fused_rare<BWD, COST, NBUF, 0, 2, 2>(QG_FUSED_ARGS);
+                else tile_body_fused_rare<BWD, COST, NBUF, 2, 2, 2>(QG_FUSED_ARGS);
+            }
+#undef QG_FUSED_ARGS
+        } else {
+            const PassConst &K = s_k[0];
+            const bool tan = K.R.mode == 0;
+#define QG_TILE_ARGS                                                                                                \
+    K, D, rs, gp, stab, s_rot, s_w, bufs, b, bar, sched, total, ti.base, ti.tl, tinfo, descs, tile_begin, ndesc,    \
+        cursor, s_tr
+            if constexpr (!GATH) {
+                if (tan) tile_body<BWD, COST, NBUF, 0, VAR, 3, 1>(QG_TILE_ARGS);
+                else tile_body<BWD, COST, NBUF, 2, VAR, 3, 1>(QG_TILE_ARGS);
+            } else if (c >= 8) {
+                if (tan) tile_body<BWD, COST, NBUF, 0, VAR, 1, 0>(QG_TILE_ARGS);
+                else tile_body<BWD, COST, NBUF, 2, VAR, 1, 0>(QG_TILE_ARGS);
+            } else {
+                if (tan && c == 4) tile_body<BWD, COST, NBUF, 0, VAR, 2, 1>(QG_TILE_ARGS);
+                else if (tan) tile_body<BWD, COST, NBUF, 0, VAR, 2, 0>(QG_TILE_ARGS);
+                else tile_body<BWD, COST, NBUF, 2, VAR, 2, 0>(QG_TILE_ARGS);
+            }
+#undef QG_TILE_ARGS
+        }
     }
 }
 
@@ -1483,11 +1385,10 @@ __device__ __forceinline__ Round12 round12(const RoundCoef &cf, float sgn) {
     r.R.ntt = make_float2(-sgn * cf.bt, -sgn * cf.bt);
     r.R.c = cf.cb;
     r.R.s = sgn * cf.sb;
-    r.R.psc = cf.bmode == 0 ? cf.cb * cf.cb : 1.f;
+    r.R.psc = cf.bmode == 0 ? cf.pw[2] : 1.f;
     r.rescale = (cf.bmode == 0 && cf.rescale) ? 1 : 0;
-    const float c = cf.bmode == 0 ? cf.cb : 1.f;
-    r.fs = c * c * c * c;
-    r.fse = r.rescale ? 1.f : r.fs * r.fs * r.fs;
+    r.fs = cf.bmode == 0 ? cf.pw[4] : 1.f;
+    r.fse = r.rescale || cf.bmode != 0 ? 1.f : cf.pw[12];
     r.ghi = cf.g_hi;
     r.glo = cf.g_lo;
     return r;
@@ -1746,7 +1647,8 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
             const double g = ga * kInvTwoPi;
             c.g_hi = (float)g;
             c.g_lo = (float)(g - (double)c.g_hi);
-            c.b_hi = c.b_lo = c.pad = 0.f;
+            c.b_hi = c.b_lo = c.pad[0] = c.pad[1] = 0.f;
+            for (int j = 0; j <= kPassTileBits; j++) c.pw[j] = 1.f;  // direct form: no cosine factors
             D.coef[e] = c;
         }
         for (int e = threadIdx.x; e < D.p * (n + 1); e += blockDim.x) {
@@ -1795,9 +1697,9 @@ __global__ void __launch_bounds__(32) reduce2_kernel(const RedOut *__restrict__ 
     if (threadIdx.x == 0) *O.out = O.scale * acc;
 }
 
-template <int BWD, int COST, int NBUF, int VAR, int FUSED>
+template <int BWD, int COST, int NBUF, int VAR, int FUSED, int GATH>
 cudaError_t launch_one(const PassDesc *d, const uint32_t *tb, int nd, uint32_t tiles, int *err, uint32_t *sched,
-                       int cost_free, cudaStream_t s) {
+                       cudaStream_t s) {
     using G = PassGeom<BWD, COST>;
     const size_t smem = G::kHead + (size_t)NBUF * G::kBufB + G::kStashB;
     // per device: the shared-memory attribute and the persistent grid size
@@ -1807,19 +1709,19 @@ cudaError_t launch_one(const PassDesc *d, const uint32_t *tb, int nd, uint32_t t
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    e = smem_attr_once(xpass_kernel<BWD, COST, NBUF, VAR, FUSED>, (int)smem, attr_done);
+    e = smem_attr_once(xpass_kernel<BWD, COST, NBUF, VAR, FUSED, GATH>, (int)smem, attr_done);
     if (e != cudaSuccess) return e;
     int grid_cap = __atomic_load_n(&grid_caps[dev], __ATOMIC_ACQUIRE);
     if (!grid_cap) {
         int nsm = 0, per_sm = 0;
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xpass_kernel<BWD, COST, NBUF, VAR, FUSED>, kNT, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, xpass_kernel<BWD, COST, NBUF, VAR, FUSED, GATH>, kNT, smem);
         if (e != cudaSuccess) return e;
         grid_cap = std::max(1, nsm * std::max(1, per_sm));
         __atomic_store_n(&grid_caps[dev], grid_cap, __ATOMIC_RELEASE);
     }
     const uint32_t grid = std::min<uint32_t>(tiles, (uint32_t)grid_cap);
-    xpass_kernel<BWD, COST, NBUF, VAR, FUSED><<<grid, kNT, smem, s>>>(d, tb, nd, tiles, err, sched, cost_free);
+    xpass_kernel<BWD, COST, NBUF, VAR, FUSED, GATH><<<grid, kNT, smem, s>>>(d, tb, nd, tiles, err, sched);
     return cudaGetLastError();
 }
 
@@ -1843,31 +1745,38 @@ cudaError_t launch_wait_probe(int *err, cudaStream_t s) {
 
 int small_max_n() { return kSmallMaxN; }
 
-template <int VAR, int FUSED>
+template <int VAR, int FUSED, int GATH>
 cudaError_t launch_xpass_t(int bwd, int cost_dtype, int nbuf, const PassDesc *d, const uint32_t *tb, int nd,
-                           uint32_t tiles, int *err, uint32_t *sched, int cf, cudaStream_t s) {
-    if (!bwd) return cost_dtype == 0 ? launch_one<0, 0, 2, VAR, FUSED>(d, tb, nd, tiles, err, sched, cf, s)
-                                     : launch_one<0, 1, 2, VAR, FUSED>(d, tb, nd, tiles, err, sched, cf, s);
+                           uint32_t tiles, int *err, uint32_t *sched, cudaStream_t s) {
+    if (!bwd) return cost_dtype == 0 ? launch_one<0, 0, 2, VAR, FUSED, GATH>(d, tb, nd, tiles, err, sched, s)
+                                     : launch_one<0, 1, 2, VAR, FUSED, GATH>(d, tb, nd, tiles, err, sched, s);
     // adjoint: one tile buffer and two CTAs per SM (128 registers a thread),
     // or two buffers and one CTA per SM (no register cap below 255)
     if (nbuf == 2)
-        return cost_dtype == 0 ? launch_one<1, 0, 2, VAR, FUSED>(d, tb, nd, tiles, err, sched, cf, s)
-                               : launch_one<1, 1, 2, VAR, FUSED>(d, tb, nd, tiles, err, sched, cf, s);
-    return cost_dtype == 0 ? launch_one<1, 0, 1, VAR, FUSED>(d, tb, nd, tiles, err, sched, cf, s)
-                           : launch_one<1, 1, 1, VAR, FUSED>(d, tb, nd, tiles, err, sched, cf, s);
+        return cost_dtype == 0 ? launch_one<1, 0, 2, VAR, FUSED, GATH>(d, tb, nd, tiles, err, sched, s)
+                               : launch_one<1, 1, 2, VAR, FUSED, GATH>(d, tb, nd, tiles, err, sched, s);
+    return cost_dtype == 0 ? launch_one<1, 0, 1, VAR, FUSED, GATH>(d, tb, nd, tiles, err, sched, s)
+                           : launch_one<1, 1, 1, VAR, FUSED, GATH>(d, tb, nd, tiles, err, sched, s);
+}
+
+template <int VAR, int FUSED>
+cudaError_t launch_xpass_g(int bwd, int cost_dtype, int nbuf, int gather, const PassDesc *d, const uint32_t *tb,
+                           int nd, uint32_t tiles, int *err, uint32_t *sched, cudaStream_t s) {
+    return gather ? launch_xpass_t<VAR, FUSED, 1>(bwd, cost_dtype, nbuf, d, tb, nd, tiles, err, sched, s)
+                  : launch_xpass_t<VAR, FUSED, 0>(bwd, cost_dtype, nbuf, d, tb, nd, tiles, err, sched, s);
 }
 
 cudaError_t launch_xpass(int bwd, int cost_dtype, int nbuf, int var, const PassDesc *d, const uint32_t *tb,
-                         int nd, uint32_t tiles, int *err, uint32_t *sched, int cost_free, int fused, cudaStream_t s) {
+                         int nd, uint32_t tiles, int *err, uint32_t *sched, int gather, int fused, cudaStream_t s) {
     if (tiles == 0) return cudaSuccess;
     if (!sched) return cudaErrorInvalidValue;
     if (fused) {  // round-boundary passes: transverse field only
         if (var != 0) return cudaErrorInvalidValue;
-        return launch_xpass_t<0, 1>(bwd, cost_dtype, nbuf, d, tb, nd, tiles, err, sched, cost_free, s);
+        return launch_xpass_g<0, 1>(bwd, cost_dtype, nbuf, gather, d, tb, nd, tiles, err, sched, s);
     }
-    if (var == 1) return launch_xpass_t<1, 0>(bwd, cost_dtype, nbuf, d, tb, nd, tiles, err, sched, cost_free, s);
-    if (var == 2) return launch_xpass_t<2, 0>(bwd, cost_dtype, nbuf, d, tb, nd, tiles, err, sched, cost_free, s);
-    return launch_xpass_t<0, 0>(bwd, cost_dtype, nbuf, d, tb, nd, tiles, err, sched, cost_free, s);
+    if (var == 1) return launch_xpass_g<1, 0>(bwd, cost_dtype, nbuf, gather, d, tb, nd, tiles, err, sched, s);
+    if (var == 2) return launch_xpass_g<2, 0>(bwd, cost_dtype, nbuf, gather, d, tb, nd, tiles, err, sched, s);
+    return launch_xpass_g<0, 0>(bwd, cost_dtype, nbuf, gather, d, tb, nd, tiles, err, sched, s);
 }
 
 cudaError_t launch_small(const SmallDesc *d, int nd, int cost_dtype, int want_grad, int max_n,

@@ -100,7 +100,7 @@ struct LaunchRec {
     int tc = 0;        // tensor-core product (tensor maps below)
     CUtensorMap tm[4];  // A_hi, A_lo, B_hi, B_lo
     int sched_idx = -1;  // pass launches: tile counter slot
-    int cost_free = 0;   // pass launches: no descriptor reads the cost
+    int gather = 0;      // pass launches: gathered tiles
     int fused = 0;       // pass launches: round-boundary passes (PF_FUSED)
     double *mean_out = nullptr;  // LK_COST_MEAN: where the cost mean goes
     // Grover-mixer (rank-one) launches: mode, round and the pass grid, which
@@ -1462,13 +1462,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                 r.bytes = bytes;
                 r.sched_idx = n_sched++;
                 r.fused = (steps[s][0].flags & PF_FUSED) ? 1 : 0;
-                {
-                    const uint32_t cost_flags =
-                        bwd ? (PF_LAM_FROM_C | PF_PHASE | PF_FUSED) : (PF_PHASE | PF_E | PF_FUSED);
-                    r.cost_free = 1;
-                    for (const PassDesc &pd : steps[s])
-                        if (pd.flags & cost_flags) r.cost_free = 0;
-                }
+                r.gather = steps[s][0].c < kPassTileBits ? 1 : 0;  // the same group of every unit
                 char nm[64];
                 const int c0 = steps[s][0].c;
                 snprintf(nm, sizeof(nm), "xpass%s_%s%s_%s_%s", gk.var == 1 ? "_ma" : (gk.var == 2 ? "_gm" : ""),
@@ -2022,7 +2016,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         case LK_XPASS:
             e = launch_xpass(r.bwd, r.cost_dtype, r.nbuf, r.var, reinterpret_cast<const PassDesc *>(db + r.desc_off),
                              reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles,
-                             ctx->d_err, d_sched + r.sched_idx, r.cost_free, r.fused, ctx->stream);
+                             ctx->d_err, d_sched + r.sched_idx, r.gather, r.fused, ctx->stream);
             break;
         case LK_EIG_INIT:
             e = launch_eig_init(r.iX, r.iX_lo, r.ick0, r.ep.M, r.ep.ld, r.ep.nsets, r.ep.cost, r.ep.cost_dtype,
