@@ -1,0 +1,324 @@
+// Device helpers of the transverse-field (X) mixer kernels: phases, round
+// coefficients, packed rotations and warp sums, shared by the pass kernels
+// (xpass.cuh) and the on-chip kernels (kernels_xmix.cu).
+#pragma once
+
+#include "common.cuh"
+#include "bulk.cuh"
+
+#include <math.h>
+
+#include <algorithm>
+
+namespace qg {
+namespace {
+
+// Tile of the pass and n = 12 kernels: 2^12 amplitudes, 16 in each of 256 threads.
+constexpr int kT = kPassTileBits;
+constexpr int kTile = 1 << kT;
+constexpr int kNT = 256;
+constexpr int kNW = kNT / 32;
+
+constexpr float kTwoPiF = 6.2831853071795864769f;
+
+// XOR swizzle of a tile-local amplitude index into shared memory.  Bits 1..3
+// are flipped by a fold of bits 6..14, bit 0 is kept so that the amplitude
+// pair (l, l^1) stays one aligned 16-byte vector.  With it, every stage's
+// accesses are conflict free: 16-byte accesses vary local bits 1..3 within a
+// quarter warp; 8-byte accesses vary local bits {0,6,7,8} (stage 2) or
+// {0,1,2,3} (stage 3) within a half warp.  The map is linear over GF(2):
+// swz(a ^ b) = swz(a) ^ swz(b).
+__device__ __forceinline__ uint32_t swz(uint32_t l) {
+    return l ^ ((((l >> 6) ^ (l >> 9) ^ (l >> 12)) & 7u) << 1);
+}
+
+__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
+}
+// a * conj(b)
+__device__ __forceinline__ float2 cmul_conj(float2 a, float2 b) {
+    return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
+}
+
+// e^{-i gamma C} for a float32 cost.  gamma/(2 pi) = g_hi + g_lo; the product
+// t = (g_hi + g_lo) C is formed as a float pair (exact head product by FMA),
+// its integer part removed exactly, and the remaining turn f in [-1/2, 1/2]
+// fed to the hardware sine/cosine at 2 pi f in [-pi, pi].
+__device__ __forceinline__ float2 phase_f32(float C, float ghi, float glo) {
+    const float th = ghi * C;
+    const float te = fmaf(ghi, C, -th);
+    const float tl = fmaf(glo, C, te);
+    const float f = (th - rintf(th)) + tl;
+    float s, c;
+    __sincosf(kTwoPiF * f, &s, &c);
+    return make_float2(c, -s);
+}
+
+// (sin, cos) of 2 pi t for a float64 turn count t, without float64
+// transcendentals (slow on this part): t = q/4 + r with the nearest quarter
+// turn q/4 removed in float64, |r| <= 1/8 to the float32 sincospi, then the
+// quarter turns applied exactly.  Values near zero keep their relative accuracy.
+__device__ __forceinline__ void sincos_turns(double t, float *s, float *c) {
+    const double q = rint(4.0 * t);
+    const float r = (float)(t - 0.25 * q);
+    float sr, cr;
+    sincospif(2.f * r, &sr, &cr);
+    switch ((int)((long long)q & 3)) {
+    case 0: *s = sr; *c = cr; break;
+    case 1: *s = cr; *c = -sr; break;
+    case 2: *s = -sr; *c = -cr; break;
+    default: *s = -cr; *c = sr; break;
+    }
+}
+
+constexpr double kInvTwoPi = 0.15915494309189533577;  // 1 / (2 pi)
+
+// Round coefficients from one beta (rotation) and the round's gamma.
+__device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
+    const double bb = be * kInvTwoPi;
+    float sb, cb;
+    sincos_turns(bb, &sb, &cb);
+    RoundCoef c;
+    c.cb = cb;
+    c.sb = sb;
+    // tan form unless cos b is so small that the running 1/cos factors or
+    // the pair-term scale would leave float32 range (then: direct form)
+    if (fabsf(cb) >= 2.44140625e-4f) {
+        c.bmode = 0;
+        c.bt = sb / cb;
+    } else {
+        c.bmode = 2;
+        c.bt = 0.f;
+    }
+    c.rescale = fabsf(cb) < 0.25f ? 1 : 0;
+    const double g = ga * kInvTwoPi;
+    c.g_hi = (float)g;
+    c.g_lo = (float)(g - (double)c.g_hi);
+    c.b_hi = (float)bb;
+    c.b_lo = (float)(bb - (double)c.b_hi);
+    // cos b as the rounded tan b has it, so that the rotations keep the norm
+    // whatever t was rounded to, and its powers rounded once each
+    const double ce = c.bmode == 0 ? copysign(1.0 / sqrt(1.0 + (double)c.bt * (double)c.bt), (double)cb) : (double)cb;
+    double q = 1.0;
+    for (int k = 0; k <= kPassTileBits; k++) {
+        c.pw[k] = (float)q;
+        q *= ce;
+    }
+    c.pad[0] = c.pad[1] = 0.f;
+    return c;
+}
+
+// ----------------------------------------------------------------------------
+// Packed (f32x2) rotations in the twisted basis s_x = (-i)^{|x|} psi_x, where
+// e^{-i b X} on a qubit is the real matrix [[c, s], [-s, c]] applied to the
+// (re, im) pair of both amplitudes alike.  Register pairs (i, i | 1<<RB).
+struct Rot {
+    float2 tt, ntt;  // (t, t), (-t, -t), t = tan b   (bmode 0)
+    float c, s;      // cos b, sin b                  (bmode 2)
+    float psc;       // pair-term scale per rotation: c^2 (bmode 0) or 1
+    int mode;
+};
+
+template <int RB, int MODE>
+__device__ __forceinline__ void rot_pairs(float2 (&a)[16], const Rot &R) {
+    if (MODE == 0) {
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            if (i & (1 << RB)) continue;
+            const int j = i | (1 << RB);
+            const float2 x = a[i], y = a[j];
+            a[i] = __ffma2_rn(R.tt, y, x);   // s0 + t s1
+            a[j] = __ffma2_rn(R.ntt, x, y);  // s1 - t s0
+        }
+    } else {
+        const float2 cc = make_float2(R.c, R.c), ss = make_float2(R.s, R.s), nss = make_float2(-R.s, -R.s);
+#pragma unroll
+        for (int i = 0; i < 16; i++) {
+            if (i & (1 << RB)) continue;
+            const int j = i | (1 << RB);
+            const float2 x = a[i], y = a[j];
+            a[i] = __ffma2_rn(ss, y, __fmul2_rn(cc, x));   // c s0 + s s1
+            a[j] = __ffma2_rn(nss, x, __fmul2_rn(cc, y));  // c s1 - s s0
+        }
+    }
+}
+
+// This thread's share of Im <lambda| X_q |psi> in the twisted basis, where
+// X_q becomes [[0, i], [-i, 0]]: sum over pairs of l0.p1 - l1.p0 (real dot
+// products of (re, im) pairs), with four independent packed accumulators.
+template <int RB>
+__device__ __forceinline__ float pair_dot(const float2 (&l)[16], const float2 (&p)[16]) {
+    float2 ap[4], am[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) ap[k] = am[k] = make_float2(0.f, 0.f);
+    int k = 0;
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        if (i & (1 << RB)) continue;
+        const int j = i | (1 << RB);
+        ap[k & 3] = __ffma2_rn(l[i], p[j], ap[k & 3]);
+        am[k & 3] = __ffma2_rn(l[j], p[i], am[k & 3]);
+        k++;
+    }
+    const float2 sp = __fadd2_rn(__fadd2_rn(ap[0], ap[1]), __fadd2_rn(ap[2], ap[3]));
+    const float2 sm = __fadd2_rn(__fadd2_rn(am[0], am[1]), __fadd2_rn(am[2], am[3]));
+    return (sp.x + sp.y) - (sm.x + sm.y);
+}
+
+// The rotations of one register layout ("stage"): on bit k = register bit k
+// carries an active qubit.  The adjoint first takes the pair terms
+// <lambda|X_q|psi> of all the stage's qubits at the stage's starting point --
+// any point of the round where both vectors have had the same rotations
+// gives the same value, because all X_q commute -- and then rotates lambda,
+// and psi only when rot_psi is set (its later values are not always needed).
+template <int BWD, int MODE>
+__device__ __forceinline__ void stage_rot(float2 (&a)[16], float2 (&l)[16], uint32_t on, const Rot &R,
+                                          float &pscale, float &bacc, bool rot_psi, bool pairs = true) {
+    if (BWD) {
+        if (pairs) {
+            float s = 0.f;
+            if (on & 1u) s += pair_dot<0>(l, a);
+            if (on & 2u) s += pair_dot<1>(l, a);
+            if (on & 4u) s += pair_dot<2>(l, a);
+            if (on & 8u) s += pair_dot<3>(l, a);
+            bacc = fmaf(s, pscale, bacc);
+        }
+        for (uint32_t m = on; m; m &= m - 1u) pscale *= R.psc;
+        if (on & 1u) rot_pairs<0, MODE>(l, R);
+        if (on & 2u) rot_pairs<1, MODE>(l, R);
+        if (on & 4u) rot_pairs<2, MODE>(l, R);
+        if (on & 8u) rot_pairs<3, MODE>(l, R);
+    }
+    if (!BWD || rot_psi) {
+        if (on & 1u) rot_pairs<0, MODE>(a, R);
+        if (on & 2u) rot_pairs<1, MODE>(a, R);
+        if (on & 4u) rot_pairs<2, MODE>(a, R);
+        if (on & 8u) rot_pairs<3, MODE>(a, R);
+    }
+}
+
+// Multi-angle rotations (one angle per qubit): register bit j of the stage
+// carries local bit Lj, with rot[Lj] = (cos b, +-sin b, +-tan b, cos^2 b).
+// MODE 0 is the tan form (the cosines are applied per stage or per pass like
+// the single-angle path, pscale tracks them for the pair terms), MODE 2 the
+// direct form.  The adjoint's pair terms go to one accumulator per local bit.
+template <int BWD, int MODE, int L0, int L1, int L2, int L3, int NQ>
+__device__ __forceinline__ void stage_rot_ma(float2 (&a)[16], float2 (&l)[16], uint32_t on, const float4 *rot,
+                                             float (&bq)[NQ], float &pscale, bool rot_psi) {
+    Rot R[4];
+    const int Ls[4] = {L0, L1, L2, L3};
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+        const float4 q = rot[Ls[j]];
+        R[j].c = q.x;
+        R[j].s = q.y;
+        R[j].tt = make_float2(q.z, q.z);
+        R[j].ntt = make_float2(-q.z, -q.z);
+    }
+    if (BWD) {
+        if (on & 1u) bq[L0] = fmaf(pair_dot<0>(l, a), pscale, bq[L0]);
+        if (on & 2u) bq[L1] = fmaf(pair_dot<1>(l, a), pscale, bq[L1]);
+        if (on & 4u) bq[L2] = fmaf(pair_dot<2>(l, a), pscale, bq[L2]);
+        if (on & 8u) bq[L3] = fmaf(pair_dot<3>(l, a), pscale, bq[L3]);
+        if (MODE == 0) {
+#pragma unroll
+            for (int j = 0; j < 4; j++)
+                if (on & (1u << j)) pscale *= rot[Ls[j]].w;
+        }
+        if (on & 1u) rot_pairs<0, MODE>(l, R[0]);
+        if (on & 2u) rot_pairs<1, MODE>(l, R[1]);
+        if (on & 4u) rot_pairs<2, MODE>(l, R[2]);
+        if (on & 8u) rot_pairs<3, MODE>(l, R[3]);
+    }
+    if (!BWD || rot_psi) {
+        if (on & 1u) rot_pairs<0, MODE>(a, R[0]);
+        if (on & 2u) rot_pairs<1, MODE>(a, R[1]);
+        if (on & 4u) rot_pairs<2, MODE>(a, R[2]);
+        if (on & 8u) rot_pairs<3, MODE>(a, R[3]);
+    }
+}
+
+template <int BWD>
+__device__ __forceinline__ void scale_all(float2 (&a)[16], float2 (&l)[16], float f) {
+    const float2 ff = make_float2(f, f);
+#pragma unroll
+    for (int i = 0; i < 16; i++) {
+        a[i] = __fmul2_rn(ff, a[i]);
+        if (BWD) l[i] = __fmul2_rn(ff, l[i]);
+    }
+}
+
+// (-i)^k * v
+__device__ __forceinline__ float2 twist(float2 v, int k) {
+    switch (k & 3) {
+    case 0: return v;
+    case 1: return make_float2(v.y, -v.x);
+    case 2: return make_float2(-v.x, -v.y);
+    default: return make_float2(-v.y, v.x);
+    }
+}
+
+// Float64 arithmetic runs at a small fraction of the float32 rate on this
+// part, so the per-tile partial sums below are summed across a warp in
+// float32 (a fixed shuffle tree, so still bitwise reproducible) and only the
+// warp totals are widened to float64 for the sums over tiles and warps.
+// Each thread's share is itself a float32 sum of a few hundred terms, so the
+// warp step adds an error of the same order (~1e-7 of the sum of magnitudes).
+
+// Warp sum of one float per lane; every lane gets the total.
+__device__ __forceinline__ float warp_sum_f(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Warp sums of two floats per lane in one tree: the total of x lands in
+// lanes 0..15, the total of y in lanes 16..31.
+__device__ __forceinline__ float warp_sum2_f(float x, float y) {
+    const bool hi = (threadIdx.x & 16u) != 0;
+    float v = (hi ? y : x) + __shfl_xor_sync(0xffffffffu, hi ? x : y, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Warp sums of 16 floats per lane as a reduce-scatter: each step halves the
+// values a lane keeps and trades the other half with its partner, so value
+// j's total lands in lanes 2j and 2j + 1 after 16 shuffles (not 80).
+__device__ __forceinline__ float warp_sum16_f(const float (&v)[16]) {
+    const uint32_t lane = threadIdx.x & 31u;
+    float w8[8], w4[4], w2[2];
+    const bool h4 = lane & 16u, h3 = lane & 8u, h2 = lane & 4u, h1 = lane & 2u;
+#pragma unroll
+    for (int k = 0; k < 8; k++)
+        w8[k] = (h4 ? v[k + 8] : v[k]) + __shfl_xor_sync(0xffffffffu, h4 ? v[k] : v[k + 8], 16);
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+        w4[k] = (h3 ? w8[k + 4] : w8[k]) + __shfl_xor_sync(0xffffffffu, h3 ? w8[k] : w8[k + 4], 8);
+#pragma unroll
+    for (int k = 0; k < 2; k++)
+        w2[k] = (h2 ? w4[k + 2] : w4[k]) + __shfl_xor_sync(0xffffffffu, h2 ? w4[k] : w4[k + 2], 4);
+    float w = (h1 ? w2[1] : w2[0]) + __shfl_xor_sync(0xffffffffu, h1 ? w2[0] : w2[1], 2);
+    return w + __shfl_xor_sync(0xffffffffu, w, 1);
+}
+
+// Deterministic block sum of one float per thread: float32 within each
+// warp, float64 across warps; the result is valid in thread 0.
+template <int NW>
+__device__ __forceinline__ double block_sum(float v, double *red) {
+    double d = (double)warp_sum_f(v);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (lane == 0) red[warp] = d;
+    __syncthreads();
+    double tot = 0.0;
+    if (threadIdx.x == 0) {
+#pragma unroll
+        for (int w = 0; w < NW; w++) tot += red[w];
+    }
+    __syncthreads();
+    return tot;
+}
+
+
+}  // namespace
+}  // namespace qg
