@@ -455,9 +455,8 @@ qaoa_status qaoa_grover_batched(qaoa_ctx *ctx, const int64_t *d_counts, int n_bi
  *   d_grad      device output, 2p float64, or NULL for the expectation only
  *   cuda_stream the stream to run on (NULL = legacy default stream)
  *
- * Scratch (coefficients, phase tables, launch descriptors, an error word) is a
- * fixed 256 KiB file-scope device array that every device loading the library
- * keeps until exit; sizes beyond n = 12 or p = 96 are rejected with
+ * Scratch (a launch descriptor and an error word) is a fixed 1 KiB file-scope
+ * device array that every device loading the library keeps until exit; sizes beyond n = 12 or p = 96 are rejected with
  * QAOA_ERR_INVALID.  The first call on a device looks up the array's device
  * address (cudaGetSymbolAddress) once and keeps it; make that first call
  * before any stream capture, and do not call the entry point on a device after

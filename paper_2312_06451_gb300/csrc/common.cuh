@@ -135,7 +135,7 @@ struct SmallDesc {
     float amp0;
     int nq;                  // multi-angle: n coefficients per round (else 0)
     const double *wts;       // general X mixer: Hadamard-basis weights d_0..d_n (else nullptr)
-    const double *angles_beta;  // general X mixer: beta_1..beta_p (the unit's angles)
+    const double *angles_beta;  // beta_1..beta_p, then the gammas (the unit's angles)
 };
 
 struct PrepDesc {
@@ -345,9 +345,12 @@ cudaError_t launch_xpass(int bwd, int cost_dtype, int nbuf, int var, const PassD
                          const uint32_t *d_tile_begin, int ndesc, uint32_t total_tiles,
                          int *d_err, uint32_t *d_sched, int gather, int fused, cudaStream_t s);
 int small_max_n();
-// n = 12, transverse-field mixer: one CTA per angle set keeps the whole state
-// as one register-staged tile (descriptors as for launch_small).
-cudaError_t launch_tile12(const SmallDesc *d_descs, int ndesc, int cost_dtype, int want_grad, int *d_err,
+// n <= 12, transverse-field mixer, uniform or given initial state: one CTA per
+// angle set (kernels_onchip.cu).  Descriptors need angles_beta, not coef or
+// table.  onchip_class: the launch class of an instance (the units of a launch
+// share one), 0 when n is out of range.
+int onchip_class(int n);
+cudaError_t launch_onchip(const SmallDesc *d_descs, int ndesc, int cls, int cost_dtype, int want_grad, int *d_err,
                           cudaStream_t s);
 // Diagnostic: a bounded wait on a barrier nothing completes (sets DERR_TIMEOUT).
 cudaError_t launch_wait_probe(int *d_err, cudaStream_t s);

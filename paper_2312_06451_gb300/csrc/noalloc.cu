@@ -1,10 +1,10 @@
 // qaoa_gradient_small_noalloc: the small-n expectation / gradient without any
 // device allocation, for callers that cannot call cudaMalloc (for example code
 // running under a memory manager that forbids allocations after start-up, or a
-// host that owns all device memory itself).  The kernel's scratch -- per-round
-// rotation and phase coefficients, the phase tables of uint8 costs, the launch
-// descriptors and the device error word -- lives in one file-scope device array
-// of fixed size instead of context-owned allocations.
+// host that owns all device memory itself).  The kernel's scratch -- the launch
+// descriptor and the device error word -- lives in one file-scope device array
+// of fixed size instead of context-owned allocations; coefficients and phase
+// tables are formed on chip.
 #include "qaoa.h"
 #include "common.cuh"
 
@@ -13,7 +13,7 @@
 #include <mutex>
 
 namespace {
-constexpr size_t kNoAllocBytesDecl = 256 * 1024;
+constexpr size_t kNoAllocBytesDecl = 1024;
 }  // namespace
 
 // The scratch array (file scope, internal linkage).
@@ -21,21 +21,14 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytesDe
 
 namespace {
 
-// Fixed scratch: 256 KiB, enough for p <= kNoAllocMaxP rounds (coefficients
-// 32 B and a 2 KiB phase table per round, plus descriptors).  Every device
-// that loads the library holds this array until the process exits.
+// Fixed scratch: the error word and the descriptor (the kernel forms
+// coefficients and phase tables on chip).  Every device that loads the library
+// holds this array until the process exits.
 constexpr size_t kNoAllocBytes = kNoAllocBytesDecl;
 constexpr int kNoAllocMaxP = 96;
 constexpr size_t kOffErr = 0;
-constexpr size_t kOffPrep = 64;
-constexpr size_t kOffSmall = 192;
-constexpr size_t kOffCoef = 512;
-constexpr size_t kOffTable = kOffCoef + sizeof(qg::RoundCoef) * kNoAllocMaxP;
-static_assert(kOffTable % 256 == 0, "table offset alignment");
-static_assert(kOffTable + sizeof(float2) * qg::kPhaseTable * kNoAllocMaxP <= kNoAllocBytes,
-              "scratch too small for kNoAllocMaxP rounds");
-static_assert(sizeof(qg::PrepDesc) <= kOffSmall - kOffPrep, "descriptor layout");
-static_assert(sizeof(qg::SmallDesc) <= kOffCoef - kOffSmall, "descriptor layout");
+constexpr size_t kOffSmall = 64;
+static_assert(kOffSmall + sizeof(qg::SmallDesc) <= kNoAllocBytes, "descriptor layout");
 
 std::mutex g_mu;
 unsigned char *g_dev_ptr[qg::kMaxDevices] = {nullptr};
@@ -76,40 +69,25 @@ extern "C" qaoa_status qaoa_gradient_small_noalloc(const void *d_cost, int cost_
         return QAOA_ERR_CUDA;
     }
     int *d_err = reinterpret_cast<int *>(base + kOffErr);
-    qg::RoundCoef *coef = reinterpret_cast<qg::RoundCoef *>(base + kOffCoef);
-    float2 *table = cost_dtype == QAOA_COST_U8 ? reinterpret_cast<float2 *>(base + kOffTable) : nullptr;
 
-    // descriptors: copied into the array from this stack frame (a pageable
+    // descriptor: copied into the array from this stack frame (a pageable
     // source: the copy has consumed it when cudaMemcpyAsync returns)
-    unsigned char host[kOffCoef - kOffPrep];
-    std::memset(host, 0, sizeof(host));
-    qg::PrepDesc pd;
-    std::memset(&pd, 0, sizeof(pd));
-    pd.angles = d_angles;
-    pd.coef = coef;
-    pd.table = table;
-    pd.p = p;
-    pd.tsize = qg::kPhaseTable;
     qg::SmallDesc sd;
     std::memset(&sd, 0, sizeof(sd));
     sd.cost = d_cost;
     sd.init = nullptr;
-    sd.coef = coef;
-    sd.table = table;
+    sd.angles_beta = d_angles;
     sd.E_out = d_E;
     sd.grad_out = d_grad;
     sd.n = n;
     sd.p = p;
     sd.amp0 = (float)(1.0 / std::sqrt(std::ldexp(1.0, n)));
-    std::memcpy(host, &pd, sizeof(pd));
-    std::memcpy(host + (kOffSmall - kOffPrep), &sd, sizeof(sd));
 
     int h_err = 0;
     if (cudaMemsetAsync(d_err, 0, sizeof(int), s) != cudaSuccess ||
-        cudaMemcpyAsync(base + kOffPrep, host, sizeof(host), cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        qg::launch_prep(reinterpret_cast<const qg::PrepDesc *>(base + kOffPrep), 1, d_err, s) != cudaSuccess ||
-        qg::launch_small(reinterpret_cast<const qg::SmallDesc *>(base + kOffSmall), 1, cost_dtype,
-                         d_grad ? 1 : 0, n, d_err, s) != cudaSuccess ||
+        cudaMemcpyAsync(base + kOffSmall, &sd, sizeof(sd), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        qg::launch_onchip(reinterpret_cast<const qg::SmallDesc *>(base + kOffSmall), 1, qg::onchip_class(n), cost_dtype,
+                          d_grad ? 1 : 0, d_err, s) != cudaSuccess ||
         cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         cudaGetLastError();

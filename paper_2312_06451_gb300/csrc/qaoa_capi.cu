@@ -86,7 +86,7 @@ struct LaunchRec {
     size_t desc_off = 0, tb_off = 0;
     int ndesc = 0;
     uint32_t tiles = 0;
-    int small_maxn = 0, small_grad = 0, t12 = 0;
+    int small_maxn = 0, small_grad = 0, chip_cls = 0;
     int fam = 0;
     double bytes = 0.0;
     double flops = 0.0;
@@ -1260,11 +1260,11 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             prep[i].wtab = u.gm ? reinterpret_cast<float4 *>(mb + off_w[i]) : nullptr;
         }
         {
-            // the n = 12 tile kernel forms its coefficients itself
+            // the on-chip kernel forms its coefficients itself
             std::vector<PrepDesc> todo;
             for (int i = 0; i < nu; i++) {
                 const Unit &u = units[i];
-                if (!(u.mixer_kind == QAOA_MIXER_X && u.n == kPassTileBits && !u.ma && !u.gm)) todo.push_back(prep[i]);
+                if (!(u.mixer_kind == QAOA_MIXER_X && u.n <= smax && !u.ma && !u.gm)) todo.push_back(prep[i]);
             }
             if (!todo.empty()) {
                 LaunchRec r;
@@ -1275,17 +1275,17 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                 L.push_back(r);
             }
         }
-        // on-chip units: n = 12 with the transverse field as one register-staged
-        // tile (t12), every other n <= 12 unit in the generic kernel
-        for (int combo = 0; combo < 4; combo++) {
-            const int dt = combo & 1, t12 = combo >> 1;
+        // on-chip units (n <= 12): the transverse field by launch class, every
+        // other mixer variant in the generic kernel (class 0)
+        for (int combo = 0; combo < 2 * 5; combo++) {
+            const int dt = combo & 1, cls = combo < 2 ? 0 : 8 + (combo >> 1);
             std::vector<SmallDesc> sd;
             int maxn = 0;
             double bytes = 0;
             for (int i = 0; i < nu; i++) {
                 const Unit &u = units[i];
                 if (u.mixer_kind != QAOA_MIXER_X || u.n > smax || u.cost_dtype != dt) continue;
-                if ((u.n == kPassTileBits && !u.ma && !u.gm) != (t12 != 0)) continue;
+                if ((u.ma || u.gm ? 0 : onchip_class(u.n)) != cls) continue;
                 SmallDesc s;
                 std::memset(&s, 0, sizeof(s));
                 s.cost = u.cost;
@@ -1312,9 +1312,9 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             r.ndesc = (int)sd.size();
             r.small_maxn = maxn;
             r.small_grad = grad ? 1 : 0;
-            r.t12 = t12;
+            r.chip_cls = cls;
             r.bytes = bytes;
-            r.fam = family(ctx, std::string(t12 ? "tile12_" : "small_") + (grad ? "grad_" : "fwd_") + dtype_name(dt));
+            r.fam = family(ctx, std::string(cls ? "onchip_" : "small_") + (grad ? "grad_" : "fwd_") + dtype_name(dt));
             L.push_back(r);
         }
         std::vector<RedChunk> rchunks;
@@ -2006,9 +2006,9 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                             ctx->stream);
             break;
         case LK_SMALL:
-            if (r.t12)
-                e = launch_tile12(reinterpret_cast<const SmallDesc *>(db + r.desc_off), r.ndesc, r.cost_dtype,
-                                  r.small_grad, ctx->d_err, ctx->stream);
+            if (r.chip_cls)
+                e = launch_onchip(reinterpret_cast<const SmallDesc *>(db + r.desc_off), r.ndesc, r.chip_cls,
+                                  r.cost_dtype, r.small_grad, ctx->d_err, ctx->stream);
             else
                 e = launch_small(reinterpret_cast<const SmallDesc *>(db + r.desc_off), r.ndesc, r.cost_dtype,
                                  r.small_grad, r.small_maxn, ctx->d_err, ctx->stream);

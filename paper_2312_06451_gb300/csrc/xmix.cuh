@@ -71,6 +71,25 @@ __device__ __forceinline__ void sincos_turns(double t, float *s, float *c) {
     }
 }
 
+// e^{-i gamma c} for a small whole cost c, gamma/(2 pi) = g_hi + g_lo: the
+// quarter turns of the head product removed exactly in float32, the tail (the
+// head's rounding and g_lo c) added to the remainder, so the phase is as
+// accurate as from a float64 turn count, without float64 arithmetic (16 cycles
+// a warp instruction on this part).
+__device__ __forceinline__ float2 phase_turns(float ghi, float glo, float c) {
+    const float th = ghi * c;
+    const float tail = fmaf(glo, c, fmaf(ghi, c, -th));
+    const float q = rintf(4.f * th);
+    const float r = fmaf(-0.25f, q, th) + tail;
+    float sr, cr;
+    sincospif(2.f * r, &sr, &cr);
+    // quarter turns: q mod 4 from the float (exact: q is whole)
+    const int m = (int)(q - 4.f * floorf(0.25f * q));
+    const float sn = m == 0 ? sr : m == 1 ? cr : m == 2 ? -sr : -cr;
+    const float cs = m == 0 ? cr : m == 1 ? -sr : m == 2 ? -cr : sr;
+    return make_float2(cs, -sn);
+}
+
 constexpr double kInvTwoPi = 0.15915494309189533577;  // 1 / (2 pi)
 
 // Round coefficients from one beta (rotation) and the round's gamma.
@@ -98,12 +117,19 @@ __device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
     c.b_lo = (float)(bb - (double)c.b_hi);
     // cos b as the rounded tan b has it, so that the rotations keep the norm
     // whatever t was rounded to, and its powers rounded once each
-    const double ce = c.bmode == 0 ? copysign(1.0 / sqrt(1.0 + (double)c.bt * (double)c.bt), (double)cb) : (double)cb;
-    double q = 1.0;
-    for (int k = 0; k <= kPassTileBits; k++) {
-        c.pw[k] = (float)q;
-        q *= ce;
+    double ce = (double)cb;
+    if (c.bmode == 0) {  // 1 / sqrt(1 + t^2): a float32 start and two Newton steps
+        const double x = fma((double)c.bt, (double)c.bt, 1.0);
+        double y = (double)rsqrtf((float)x);
+        y = y * fma(-0.5 * x * y, y, 1.5);
+        y = y * fma(-0.5 * x * y, y, 1.5);
+        ce = cb < 0.f ? -y : y;
     }
+    const double c2 = ce * ce, c4 = c2 * c2, c8 = c4 * c4;
+    const double pw[13] = {1.0, ce, c2, c2 * ce, c4, c4 * ce, c4 * c2, c4 * c2 * ce, c8, c8 * ce, c8 * c2,
+                           c8 * c2 * ce, c8 * c4};
+#pragma unroll
+    for (int k = 0; k <= kPassTileBits; k++) c.pw[k] = (float)pw[k];
     c.pad[0] = c.pad[1] = 0.f;
     return c;
 }
