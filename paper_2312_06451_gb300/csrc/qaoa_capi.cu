@@ -124,7 +124,9 @@ struct LaunchRec {
 };
 
 struct Plan {
-    uint64_t key = 0;
+    std::vector<Unit> units;  // what the plan was made for, with the mode and the schedules' epoch
+    int grad = 0, ckpt = 0;
+    uint64_t epoch = 0;
     bool valid = false;
     std::vector<LaunchRec> launches;
     int n_sched = 0;  // pass launches (one tile counter each, zeroed per call)
@@ -143,17 +145,11 @@ constexpr int64_t kMaxGroverDim = 1ll << 36;  // feasible states of a Grover (ra
 constexpr int kCminDefault = 4;   // >= 16 contiguous amplitudes = one 128-byte line
 constexpr int kTmaSegBits = 8;    // shorter runs are fetched through a TMA tensor map
 constexpr size_t kAlign = 256;
+// Device block of a context: the error word, then the results and angles of
+// single calls, so that one copy brings back the word and the results.
+constexpr size_t kIoBytes = 64 * 1024;
 
 size_t align_up(size_t v, size_t a = kAlign) { return (v + a - 1) / a * a; }
-
-uint64_t fnv1a(const void *data, size_t n, uint64_t h = 1469598103934665603ull) {
-    const unsigned char *p = static_cast<const unsigned char *>(data);
-    for (size_t i = 0; i < n; i++) {
-        h ^= p[i];
-        h *= 1099511628211ull;
-    }
-    return h;
-}
 
 // Passes of one mixer round for n qubits and tile bits T: one contiguous pass
 // over qubits 0..T-1, then the remaining n-T qubits in the fewest contiguous
@@ -218,7 +214,8 @@ struct qaoa_ctx {
     int device = 0;
     cudaStream_t stream = nullptr;
     std::string err;
-    int *d_err = nullptr;
+    int *d_err = nullptr;       // device error word, at the head of the kIoBytes block below
+    int *h_err = nullptr;       // pinned copy of it
     std::map<std::string, Buf> bufs;
     void *h_stage = nullptr;
     size_t h_stage_bytes = 0;
@@ -1117,12 +1114,12 @@ const char *dtype_name(int dt) { return dt == QAOA_COST_U8 ? "u8" : "f32"; }
 
 // Build (or reuse) the launch plan for a unit list and enqueue it.
 qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, int ckpt) {
-    uint64_t key = fnv1a(units.data(), units.size() * sizeof(Unit));
-    const int flags2[2] = {grad ? 1 : 0, ckpt};
-    key = fnv1a(flags2, sizeof(flags2), key);
-    key = fnv1a(&ctx->tune_epoch, sizeof(ctx->tune_epoch), key);
-
-    if (!(ctx->plan.valid && ctx->plan.key == key)) {
+    // the plan is reused when the units are byte for byte the ones it was made
+    // for (a compare of 256 units takes 2 us; hashing them byte by byte took 35)
+    const Plan &have = ctx->plan;
+    if (!(have.valid && have.grad == (grad ? 1 : 0) && have.ckpt == ckpt && have.epoch == ctx->tune_epoch &&
+          have.units.size() == units.size() &&
+          std::memcmp(have.units.data(), units.data(), units.size() * sizeof(Unit)) == 0)) {
         if (capturing(ctx))
             return fail(ctx, QAOA_ERR_INVALID,
                         "launch plan not built; run the same call once before stream capture");
@@ -1969,7 +1966,10 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         ctx->plan.launches = L;
         ctx->plan.n_sched = n_sched;
         ctx->plan.eig_tc = any_eig_tc;
-        ctx->plan.key = key;
+        ctx->plan.units = units;
+        ctx->plan.grad = grad ? 1 : 0;
+        ctx->plan.ckpt = ckpt;
+        ctx->plan.epoch = ctx->tune_epoch;
         ctx->plan.valid = true;
     }
 
@@ -2130,11 +2130,8 @@ qaoa_status check_args(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, const 
     return QAOA_OK;
 }
 
-qaoa_status read_dev_err(qaoa_ctx *ctx) {
-    int h = 0;
-    QG_CUDA(ctx, cudaMemcpyAsync(&h, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream),
-            "error word read");
-    QG_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronize");
+// The status of the error word `h` that a call's launches left (already read).
+qaoa_status dev_err_status(qaoa_ctx *ctx, int h) {
     if (h) {
         cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream);
         if (h & DERR_BAD_ANGLE) return fail(ctx, QAOA_ERR_INVALID, "non-finite angle");
@@ -2142,6 +2139,13 @@ qaoa_status read_dev_err(qaoa_ctx *ctx) {
         return fail(ctx, QAOA_ERR_CUDA, "device error word 0x%x", h);
     }
     return QAOA_OK;
+}
+
+qaoa_status read_dev_err(qaoa_ctx *ctx) {
+    QG_CUDA(ctx, cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream),
+            "error word read");
+    QG_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronize");
+    return dev_err_status(ctx, *ctx->h_err);
 }
 
 qaoa_status scalar_run(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, const qaoa_mixer *mixer,
@@ -2155,10 +2159,17 @@ qaoa_status scalar_run(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, const 
     const int na = ma ? p * (mixer->n + 1) : 2 * p;  // angles (and partials) per set
     for (int i = 0; i < na; i++)
         if (!std::isfinite(angles[i])) return fail(ctx, QAOA_ERR_INVALID, "angle %d is not finite", i);
-    const size_t cnt = (size_t)2 * na + 1;
-    void *d_io = nullptr;
-    st = scratch(ctx, "io", cnt * sizeof(double), &d_io);
-    if (st) return st;
+    // error word, <C>, gradient, angles: in the context's block behind the error
+    // word when they fit, else in scratch of their own (the word's slot unused)
+    const size_t cnt = (size_t)2 * na + 2;
+    const bool with_err = cnt * sizeof(double) <= kIoBytes;
+    double *io = reinterpret_cast<double *>(ctx->d_err);
+    if (!with_err) {
+        void *d_io = nullptr;
+        qaoa_status st2 = scratch(ctx, "io", cnt * sizeof(double), &d_io);
+        if (st2) return st2;
+        io = static_cast<double *>(d_io);
+    }
     if (ctx->h_io_count < cnt) {
         if (ctx->h_io) {
             cudaStreamSynchronize(ctx->stream);
@@ -2170,9 +2181,9 @@ qaoa_status scalar_run(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, const 
                 "cudaMallocHost");
         ctx->h_io_count = cnt;
     }
-    std::memcpy(ctx->h_io, angles, sizeof(double) * na);
-    double *io = static_cast<double *>(d_io);
-    QG_CUDA(ctx, cudaMemcpyAsync(io, ctx->h_io, sizeof(double) * na, cudaMemcpyHostToDevice, ctx->stream),
+    double *d_ang = io + 2 + na, *h_ang = ctx->h_io + 2 + na;
+    std::memcpy(h_ang, angles, sizeof(double) * na);
+    QG_CUDA(ctx, cudaMemcpyAsync(d_ang, h_ang, sizeof(double) * na, cudaMemcpyHostToDevice, ctx->stream),
             "angle upload");
     Unit u;
     std::memset(&u, 0, sizeof(u));
@@ -2180,9 +2191,9 @@ qaoa_status scalar_run(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, const 
     u.cost_dtype = cost_dtype;
     u.n = mixer->n;
     u.p = p;
-    u.angles = io;
-    u.E = io + na;
-    u.grad = grad ? io + na + 1 : nullptr;
+    u.angles = d_ang;
+    u.E = io + 1;
+    u.grad = grad ? io + 2 : nullptr;
     u.init = static_cast<const float2 *>(d_init);
     u.tsize = kPhaseTable;
     u.mixer_kind = (ma || mixer->kind == QAOA_MIXER_X_GENERAL) ? QAOA_MIXER_X : mixer->kind;
@@ -2198,14 +2209,20 @@ qaoa_status scalar_run(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, const 
     std::vector<Unit> us(1, u);
     st = run_units(ctx, us, grad != nullptr, grad ? ckpt : 0);
     if (st) return st;
-    const size_t nout = grad ? (size_t)na + 1 : 1;
-    QG_CUDA(ctx, cudaMemcpyAsync(ctx->h_io + na, io + na, sizeof(double) * nout, cudaMemcpyDeviceToHost,
-                                 ctx->stream),
+    const size_t nout = 2 + (grad ? (size_t)na : 0);
+    QG_CUDA(ctx, cudaMemcpyAsync(ctx->h_io, io, sizeof(double) * nout, cudaMemcpyDeviceToHost, ctx->stream),
             "result download");
-    st = read_dev_err(ctx);
+    if (with_err) {
+        QG_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronize");
+        int h = 0;
+        std::memcpy(&h, ctx->h_io, sizeof(int));
+        st = dev_err_status(ctx, h);
+    } else {
+        st = read_dev_err(ctx);
+    }
     if (st) return st;
-    *E = ctx->h_io[na];
-    if (grad) std::memcpy(grad, ctx->h_io + na + 1, sizeof(double) * na);
+    *E = ctx->h_io[1];
+    if (grad) std::memcpy(grad, ctx->h_io + 2, sizeof(double) * na);
     return QAOA_OK;
 }
 
@@ -2235,10 +2252,12 @@ qaoa_status qaoa_create(qaoa_ctx **out, int device, void *cuda_stream) {
     }
     ctx->device = device;
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
-    if (cudaMalloc(&ctx->d_err, sizeof(int)) != cudaSuccess ||
-        cudaMemset(ctx->d_err, 0, sizeof(int)) != cudaSuccess || upload_binom_table() != cudaSuccess) {
+    if (cudaMalloc(&ctx->d_err, kIoBytes) != cudaSuccess ||
+        cudaMallocHost(&ctx->h_err, sizeof(int)) != cudaSuccess ||
+        cudaMemset(ctx->d_err, 0, kIoBytes) != cudaSuccess || upload_binom_table() != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_err) cudaFree(ctx->d_err);
+        if (ctx->h_err) cudaFreeHost(ctx->h_err);
         delete ctx;
         return QAOA_ERR_CUDA;
     }
@@ -2259,6 +2278,7 @@ void qaoa_destroy(qaoa_ctx *ctx) {
     for (cudaEvent_t e : ctx->ev_pool) cudaEventDestroy(e);
     if (ctx->h_stage) cudaFreeHost(ctx->h_stage);
     if (ctx->h_io) cudaFreeHost(ctx->h_io);
+    if (ctx->h_err) cudaFreeHost(ctx->h_err);
     if (ctx->d_err) cudaFree(ctx->d_err);
     delete ctx;
 }
