@@ -352,6 +352,30 @@ int small_max_n();
 int onchip_class(int n);
 cudaError_t launch_onchip(const SmallDesc *d_descs, int ndesc, int cls, int cost_dtype, int want_grad, int *d_err,
                           cudaStream_t s);
+// 13 <= n <= kGridMaxN, transverse field: every round of an angle set in one
+// launch, 2^(n-12) CTAs a set (kernels_grid.cu).
+constexpr int kGridMaxN = 20;
+struct GridDesc {
+    const void *cost;
+    const float2 *init;    // user psi_0 or nullptr
+    const double *angles;  // p betas, then p gammas
+    double *E_out;
+    double *grad_out;      // 2p, or nullptr
+    float2 *X;             // exchange buffers: p (gradients) or 2 vectors
+    float2 *lam;           // gradients: 2 vectors
+    double *part;          // [1 + 2p (1)][2^(n-12)] per-CTA sums
+    unsigned *bar;         // arrival counter, zero when the launch starts
+    int n, p;
+    float amp0;
+    int pad;
+};
+constexpr int kGridClusterN = 16;  // up to here a set is one cluster (any number of sets a launch)
+// CTAs of one launch for n-qubit sets that are resident together (0: not
+// supported here).  Cooperative launches (n > kGridClusterN) must not exceed it.
+int grid_max_ctas(int cost_dtype, int want_grad, int n);
+// The descriptors of a launch have one n up to kGridClusterN (then: any sizes above).
+cudaError_t launch_grid(const GridDesc *d_descs, const uint32_t *d_begin, int nd, uint32_t ctas, int cost_dtype,
+                        int want_grad, int n, int *d_err, cudaStream_t s);
 // Diagnostic: a bounded wait on a barrier nothing completes (sets DERR_TIMEOUT).
 cudaError_t launch_wait_probe(int *d_err, cudaStream_t s);
 

@@ -78,7 +78,7 @@ struct Unit {
 };
 
 enum LaunchKind { LK_PREP, LK_SMALL, LK_XPASS, LK_REDUCE, LK_EIG_INIT, LK_EIG_GEMM, LK_COST_MEAN, LK_ORBIT,
-                  LK_OPERANDS, LK_R1_PASS, LK_R1_SCALAR };
+                  LK_OPERANDS, LK_R1_PASS, LK_R1_SCALAR, LK_GRID };
 
 struct LaunchRec {
     int kind;
@@ -106,6 +106,7 @@ struct LaunchRec {
     // Grover-mixer (rank-one) launches: mode, round and the pass grid, which
     // fixes the slot layout the following scalar launch reads
     int r1mode = 0, r1round = 0;
+    int gn = 0;  // LK_GRID: qubits (the largest of a cooperative launch)
     uint32_t r1grid = 0;
     // grouped (block-diagonal) products and orbit kernels
     int grouped = 0, n_mtiles = 0, lda = 0, ldb = 0;
@@ -131,6 +132,7 @@ struct Plan {
     std::vector<LaunchRec> launches;
     int n_sched = 0;  // pass launches (one tile counter each, zeroed per call)
     bool eig_tc = false;  // tensor-core eigenbasis products (split-K tail workspace)
+    int n_bar = 0;        // arrival counters of the cooperative launches (zeroed per call)
 };
 
 // Global-bit layout of one pass: local bits 0..c-1 are global bits 0..c-1,
@@ -203,6 +205,12 @@ int fused_bwd_nbuf() {
     return v;
 }
 
+// A caller that picks a fusion mode wants the pass kernels.
+bool fusion_forced() {
+    static const bool v = std::getenv("QAOA_FUSE") && *std::getenv("QAOA_FUSE");
+    return v;
+}
+
 int min_contig() {
     static const int c = env_int("QAOA_MIN_CONTIG", kCminDefault, 4, 8);
     return c;
@@ -215,7 +223,7 @@ struct qaoa_ctx {
     cudaStream_t stream = nullptr;
     std::string err;
     int *d_err = nullptr;       // device error word, at the head of the kIoBytes block below
-    int *h_err = nullptr;       // pinned copy of it
+    int *h_err = nullptr;       // pinned copy of it (made at its first read)
     std::map<std::string, Buf> bufs;
     void *h_stage = nullptr;
     size_t h_stage_bytes = 0;
@@ -1112,6 +1120,82 @@ qaoa_status plan_sym_job(qaoa_ctx *ctx, const std::vector<Unit> &units, int u0, 
 
 const char *dtype_name(int dt) { return dt == QAOA_COST_U8 ? "u8" : "f32"; }
 
+// Units that run with all rounds in one launch (kernels_grid.cu): transverse
+// field, 13 <= n <= 20.  Measured against the passes (p = 6 gradients, float32
+// costs, us a call): up to n = 16, where a set is a cluster, at every batch size
+// (n = 13: 62 / 140 for one set, 172 / 351 for 256; n = 16: 67 / 155 and 1609 /
+// 1758), so always.  Above, sets that fit the chip together take 88 / 170 (n =
+// 17, 18) to 128 / 210 (n = 20), and each further launch of them as long again,
+// while the passes' time grows more slowly: even at four launches (n = 20: 500 /
+// 495), so at most kGridWaves.
+constexpr int kGridWaves = 3;
+// Not taken where the caller asks for the passes: a schedule installed for the
+// size, a fusion mode, gradients without checkpoints (two vectors; this path
+// keeps p + 2), or when the vectors do not fit the budget.
+// One launch per class and wave: each n of a cluster on its own, the larger ones together.
+constexpr int kGridClasses = kGridClusterN - kPassTileBits + 1;
+int grid_class(int n) { return std::min(n, kGridClusterN + 1) - kPassTileBits - 1; }
+struct GridPlan {
+    std::vector<char> on;
+    std::vector<size_t> off;  // state offset of each unit
+    std::vector<int> bar;     // arrival counter of each unit
+    std::vector<int> wave;    // launch of its class
+    size_t bytes = 0;
+    int n_bar = 0;
+};
+GridPlan plan_grid(const qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, int ckpt, size_t budget) {
+    GridPlan g;
+    const int nu = (int)units.size();
+    g.on.assign(nu, 0);
+    g.off.assign(nu, 0);
+    g.bar.assign(nu, 0);
+    g.wave.assign(nu, 0);
+    if (fusion_forced() || (grad && ckpt == QAOA_CKPT_NONE)) return g;
+    for (int cls = 0; cls < 2 * kGridClasses; cls++) {
+        const int dt = cls & 1, gc = cls >> 1;
+        std::vector<int> us;
+        int gn = 0;
+        size_t bytes = g.bytes;
+        std::vector<size_t> off;
+        for (int i = 0; i < nu; i++) {
+            const Unit &u = units[i];
+            if (u.mixer_kind != QAOA_MIXER_X || u.ma || u.gm || u.cost_dtype != dt || u.n <= kPassTileBits ||
+                u.n > kGridMaxN || grid_class(u.n) != gc || ctx->xtune.count({u.n, dt}))
+                continue;
+            us.push_back(i);
+            off.push_back(bytes);
+            gn = std::max(gn, u.n);
+            const size_t n_ctas = (size_t)1 << (u.n - kPassTileBits);
+            bytes = align_up(bytes + (size_t)(grad ? u.p + 2 : 2) * (sizeof(float2) << u.n) +
+                             sizeof(double) * n_ctas * (grad ? 1 + 2 * (size_t)u.p : 1));
+        }
+        if (us.empty() || bytes > budget) continue;
+        const uint64_t room = (uint64_t)grid_max_ctas(dt, grad ? 1 : 0, gn);
+        if (room < (1ull << (gn - kPassTileBits))) continue;
+        if (gn > kGridClusterN) {  // launches of sets that are resident together
+            uint64_t used = 0;
+            int wave = 0;
+            for (int i : us) {
+                const uint64_t c = 1ull << (units[i].n - kPassTileBits);
+                if (used + c > room) {
+                    wave++;
+                    used = 0;
+                }
+                g.wave[i] = wave;
+                used += c;
+            }
+            if (wave >= kGridWaves) continue;
+        }
+        for (size_t j = 0; j < us.size(); j++) {
+            g.on[us[j]] = 1;
+            g.off[us[j]] = off[j];
+            g.bar[us[j]] = g.n_bar++;
+        }
+        g.bytes = bytes;
+    }
+    return g;
+}
+
 // Build (or reuse) the launch plan for a unit list and enqueue it.
 qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, int ckpt) {
     // the plan is reused when the units are byte for byte the ones it was made
@@ -1129,6 +1213,23 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         std::vector<size_t> off_coef(nu), off_tab(nu), off_part(nu);
         std::vector<UnitLayout> lay(nu);
         size_t meta = 0;
+        size_t free_b = 0, total_b = 0;
+        cudaMemGetInfo(&free_b, &total_b);
+        const size_t held = ctx->bufs.count("state") ? ctx->bufs["state"].bytes : 0;
+        const size_t held_grid = ctx->bufs.count("gridstate") ? ctx->bufs["gridstate"].bytes : 0;
+        auto budget_of = [&](size_t avail) -> size_t {
+            const double b = (double)avail * 0.92 - 1.0 * (1ull << 30);
+            size_t v = b > 0 ? (size_t)b : 0;
+            return ctx->state_limit >= 0 ? std::min(v, (size_t)ctx->state_limit) : v;
+        };
+        GridPlan gp = plan_grid(ctx, units, grad, ckpt, budget_of(free_b + held + held_grid));
+        // what the cooperative launches take is not there for the passes
+        const size_t grid_more = gp.bytes > held_grid ? gp.bytes - held_grid : 0;
+        free_b -= std::min(free_b, grid_more);
+        size_t budget = budget_of(free_b + held);
+        if (ctx->state_limit >= 0)
+            budget = std::min(budget, (size_t)ctx->state_limit - std::min((size_t)ctx->state_limit, gp.bytes));
+        const std::vector<char> &on_grid = gp.on;
         // coefficients of all units back to back (the sets of one eigenbasis
         // job are consecutive, so their rounds form a [set][round] array)
         std::vector<size_t> off_w(nu, 0);
@@ -1146,7 +1247,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             off_tab[i] = meta;
             if (u.cost_dtype == QAOA_COST_U8) meta = align_up(meta + sizeof(float2) * kPhaseTable * u.p);
             off_part[i] = meta;
-            if (u.mixer_kind == QAOA_MIXER_X && u.n > smax) {
+            if (u.mixer_kind == QAOA_MIXER_X && u.n > smax && !on_grid[i]) {
                 lay[i] = layout_for(ctx, u, grad, ckpt);
                 // partial slots: <C>, and with gradients every beta_k and gamma_k
                 meta = align_up(meta + sizeof(double) * (grad ? 2 * u.p + 1 : 1) * lay[i].stride);
@@ -1166,17 +1267,11 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                        std::tie(o.Tf, o.Tb, o.Pf, o.Pb, o.p, o.dt, o.nbc, o.nbg, o.var, o.fused);
             }
         };
-        size_t free_b = 0, total_b = 0;
-        cudaMemGetInfo(&free_b, &total_b);
-        const size_t held = ctx->bufs.count("state") ? ctx->bufs["state"].bytes : 0;
-        const double budget_d = (double)(free_b + held) * 0.92 - 1.0 * (1ull << 30);
-        size_t budget = budget_d > 0 ? (size_t)budget_d : 0;
-        if (ctx->state_limit >= 0) budget = std::min(budget, (size_t)ctx->state_limit);
         // fused round boundaries need per-pass checkpoints: a unit whose
         // checkpoints do not fit runs the unfused schedule (and may then step
         // down to fewer checkpoints below)
         for (int i = 0; i < nu; i++) {
-            if (units[i].mixer_kind != QAOA_MIXER_X || units[i].n <= smax || !lay[i].fused || !grad) continue;
+            if (units[i].mixer_kind != QAOA_MIXER_X || units[i].n <= smax || on_grid[i] || !lay[i].fused || !grad) continue;
             if (align_up((size_t)lay[i].vecs * (sizeof(float2) << units[i].n)) > budget) {
                 lay[i].fused = false;
                 lay[i].vecs = layout_vecs(lay[i], units[i].p, grad);
@@ -1184,7 +1279,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         }
         std::map<GKey, std::vector<int>> groups;
         for (int i = 0; i < nu; i++) {
-            if (units[i].mixer_kind != QAOA_MIXER_X || units[i].n <= smax) continue;
+            if (units[i].mixer_kind != QAOA_MIXER_X || units[i].n <= smax || on_grid[i]) continue;
             const UnitLayout &L = lay[i];
             groups[{L.T_f, L.T_b, (int)L.gf.size(), (int)L.gb.size(), units[i].p, units[i].cost_dtype, L.nb_bc,
                     L.nb_bg, units[i].ma ? 1 : (units[i].gm ? 2 : 0), L.fused ? L.fuse_mask : 0}]
@@ -1257,11 +1352,12 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             prep[i].wtab = u.gm ? reinterpret_cast<float4 *>(mb + off_w[i]) : nullptr;
         }
         {
-            // the on-chip kernel forms its coefficients itself
+            // the on-chip and the cooperative kernels form their coefficients themselves
             std::vector<PrepDesc> todo;
             for (int i = 0; i < nu; i++) {
                 const Unit &u = units[i];
-                if (!(u.mixer_kind == QAOA_MIXER_X && u.n <= smax && !u.ma && !u.gm)) todo.push_back(prep[i]);
+                if (!(u.mixer_kind == QAOA_MIXER_X && u.n <= smax && !u.ma && !u.gm) && !on_grid[i])
+                    todo.push_back(prep[i]);
             }
             if (!todo.empty()) {
                 LaunchRec r;
@@ -1313,6 +1409,55 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             r.bytes = bytes;
             r.fam = family(ctx, std::string(cls ? "onchip_" : "small_") + (grad ? "grad_" : "fwd_") + dtype_name(dt));
             L.push_back(r);
+        }
+        // cooperative launches (13 <= n <= 20), one per cost type and class
+        if (gp.bytes) {
+            void *d_gs = nullptr, *d_bar = nullptr;
+            if ((st = scratch(ctx, "gridstate", gp.bytes, &d_gs))) return st;
+            if ((st = scratch(ctx, "gridbar", sizeof(unsigned) * gp.n_bar, &d_bar))) return st;
+            for (int lw = 0; lw < 2 * kGridClasses * kGridWaves; lw++) {
+                const int dt = lw & 1, wave = (lw >> 1) % kGridWaves, gc = (lw >> 1) / kGridWaves;
+                std::vector<GridDesc> gd;
+                std::vector<uint32_t> begin(1, 0);
+                double bytes = 0;
+                int gn = 0;
+                for (int i = 0; i < nu; i++) {
+                    const Unit &u = units[i];
+                    if (!on_grid[i] || u.cost_dtype != dt || grid_class(u.n) != gc || gp.wave[i] != wave) continue;
+                    gn = std::max(gn, u.n);
+                    const int64_t N = 1ll << u.n;
+                    GridDesc d;
+                    std::memset(&d, 0, sizeof(d));
+                    d.cost = u.cost;
+                    d.init = u.init;
+                    d.angles = u.angles;
+                    d.E_out = u.E;
+                    d.grad_out = grad ? u.grad : nullptr;
+                    d.X = reinterpret_cast<float2 *>(static_cast<char *>(d_gs) + gp.off[i]);
+                    d.lam = grad ? d.X + (int64_t)u.p * N : nullptr;
+                    d.part = reinterpret_cast<double *>(d.X + (int64_t)(grad ? u.p + 2 : 2) * N);
+                    d.bar = static_cast<unsigned *>(d_bar) + gp.bar[i];
+                    d.n = u.n;
+                    d.p = u.p;
+                    d.amp0 = (float)(1.0 / std::sqrt(std::ldexp(1.0, u.n)));
+                    gd.push_back(d);
+                    begin.push_back(begin.back() + (1u << (u.n - kPassTileBits)));
+                    bytes += N * (dt == QAOA_COST_U8 ? 1.0 : 4.0);
+                }
+                if (gd.empty()) continue;
+                LaunchRec r;
+                r.kind = LK_GRID;
+                r.cost_dtype = dt;
+                r.gn = gn;
+                r.small_grad = grad ? 1 : 0;
+                r.desc_off = put(gd.data(), sizeof(GridDesc) * gd.size());
+                r.tb_off = put(begin.data(), sizeof(uint32_t) * begin.size());
+                r.ndesc = (int)gd.size();
+                r.tiles = begin.back();
+                r.bytes = bytes;
+                r.fam = family(ctx, std::string(grad ? "grid_grad_" : "grid_fwd_") + dtype_name(dt));
+                L.push_back(r);
+            }
         }
         std::vector<RedChunk> rchunks;
         std::vector<RedOut> routs;
@@ -1495,7 +1640,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                 const size_t held_r1 = ctx->bufs.count("r1state") ? ctx->bufs["r1state"].bytes : 0;
                 const double rb = (double)(free_b + held + held_r1) * 0.92 - 1.0 * (1ull << 30);
                 size_t r1_budget = rb > 0 ? (size_t)rb : 0;
-                if (ctx->state_limit >= 0) r1_budget = std::min(r1_budget, (size_t)ctx->state_limit);
+                if (ctx->state_limit >= 0) r1_budget = std::min(r1_budget, (size_t)ctx->state_limit - std::min((size_t)ctx->state_limit, gp.bytes));
                 r1_budget = r1_budget > state_need ? r1_budget - state_need : 0;
                 struct RUnit {
                     int i;
@@ -1966,6 +2111,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         ctx->plan.launches = L;
         ctx->plan.n_sched = n_sched;
         ctx->plan.eig_tc = any_eig_tc;
+        ctx->plan.n_bar = gp.n_bar;
         ctx->plan.units = units;
         ctx->plan.grad = grad ? 1 : 0;
         ctx->plan.ckpt = ckpt;
@@ -1981,6 +2127,9 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         QG_CUDA(ctx, cudaMemsetAsync(d_sched, 0, sizeof(uint32_t) * ctx->plan.n_sched, ctx->stream),
                 "tile counters clear");
     }
+    if (ctx->plan.n_bar > 0)
+        QG_CUDA(ctx, cudaMemsetAsync(ctx->bufs["gridbar"].p, 0, sizeof(unsigned) * ctx->plan.n_bar, ctx->stream),
+                "arrival counters clear");
     float *d_split_ws = nullptr;
     unsigned *d_split_cnt = nullptr;
     if (ctx->plan.eig_tc) {
@@ -2012,6 +2161,11 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             else
                 e = launch_small(reinterpret_cast<const SmallDesc *>(db + r.desc_off), r.ndesc, r.cost_dtype,
                                  r.small_grad, r.small_maxn, ctx->d_err, ctx->stream);
+            break;
+        case LK_GRID:
+            e = launch_grid(reinterpret_cast<const GridDesc *>(db + r.desc_off),
+                            reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles, r.cost_dtype,
+                            r.small_grad, r.gn, ctx->d_err, ctx->stream);
             break;
         case LK_XPASS:
             e = launch_xpass(r.bwd, r.cost_dtype, r.nbuf, r.var, reinterpret_cast<const PassDesc *>(db + r.desc_off),
@@ -2142,6 +2296,7 @@ qaoa_status dev_err_status(qaoa_ctx *ctx, int h) {
 }
 
 qaoa_status read_dev_err(qaoa_ctx *ctx) {
+    if (!ctx->h_err) QG_CUDA(ctx, cudaMallocHost(&ctx->h_err, sizeof(int)), "cudaMallocHost");
     QG_CUDA(ctx, cudaMemcpyAsync(ctx->h_err, ctx->d_err, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream),
             "error word read");
     QG_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "stream synchronize");
@@ -2253,11 +2408,9 @@ qaoa_status qaoa_create(qaoa_ctx **out, int device, void *cuda_stream) {
     ctx->device = device;
     ctx->stream = static_cast<cudaStream_t>(cuda_stream);
     if (cudaMalloc(&ctx->d_err, kIoBytes) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_err, sizeof(int)) != cudaSuccess ||
         cudaMemset(ctx->d_err, 0, kIoBytes) != cudaSuccess || upload_binom_table() != cudaSuccess) {
         cudaGetLastError();
         if (ctx->d_err) cudaFree(ctx->d_err);
-        if (ctx->h_err) cudaFreeHost(ctx->h_err);
         delete ctx;
         return QAOA_ERR_CUDA;
     }
