@@ -404,7 +404,6 @@ cudaError_t launch_clique_hamiltonian(int n, int k, int64_t dim, double *d_H, cu
 
 // Grover mixer as a rank-one update on a stored state vector (kernels_rank1.cu).
 enum R1Mode { R1_FWD = 0, R1_LAST = 1, R1_BWD = 2 };
-enum R1ScalarMode { R1_SFWD = 0, R1_SLAST = 1, R1_SBWD = 2 };
 struct R1Desc {
     const void *cost;
     const float2 *init;     // user psi_0 (16-byte aligned) or nullptr: amp0 everywhere
@@ -413,27 +412,29 @@ struct R1Desc {
     const double *angles;   // beta_0..beta_{p-1}, gamma_0..gamma_{p-1}
     float2 *phi;            // ckpt: phi_0..phi_{p-1} at stride ld; else one vector
     float2 *lam;            // gradient runs: the adjoint vector
-    double *part;           // [slot][3] per-block sums (min(tiles, grid) slots)
-    double *scal;           // 4 p + 3 scalars (layout in kernels_rank1.cu)
+    double *part;           // [2][slot][3] per-block sums, halves used by passes in turn
+    double *scal;           // 4 p + 1 scalars (layout in kernels_rank1.cu)
     double *E;
     double *grad;           // 2p, or nullptr
     int64_t dim;
     int64_t ld;             // vector stride (even, >= dim)
+    double inv_dim;         // 1 / dim
     int p;
     int ckpt;
     float amp0;
-    int pad;
+    uint32_t slots;         // per half: min(tiles, largest grid)
 };
 int r1_tile_amps();
 uint32_t r1_max_grid();                       // upper bound of r1_grid over modes
 uint32_t r1_grid(int mode, int cost_dtype);   // blocks of one pass kernel (persistent: a multiple of the SMs)
-// grid: blocks of the pass (the same value for every pass and scalar launch
-// over one descriptor list: it fixes the slot layout of the partials).
+// grid: blocks of the pass (at most `tiles`); grid_in: blocks of the pass before
+// it over the same descriptor list (0: none), whose sums it reads; half: 0, 1 in
+// turn, the half of the slots it writes.
 // err: the device error word (DERR_TIMEOUT when a bounded copy wait gives up).
 cudaError_t launch_r1_pass(int mode, int cost_dtype, const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles,
-                           uint32_t grid, int round, int *err, cudaStream_t s);
-cudaError_t launch_r1_scalar(int mode, const R1Desc *d, const uint32_t *tb, int nd, uint32_t grid, int round,
-                             cudaStream_t s);
+                           uint32_t grid, uint32_t grid_in, int half, int round, int *err, cudaStream_t s);
+cudaError_t launch_r1_final(const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles, uint32_t grid_in, int half,
+                            cudaStream_t s);
 
 // Grover-mixer QAOA on cost degeneracies (kernels_grover.cu).
 struct DegLaunch {

@@ -8,7 +8,7 @@
 //     psi' = phi + d 1,   d = (e^{-i b} - 1) (sum_x phi_x) / N.
 // A round is therefore one streaming pass and one scalar: the pass applies the
 // previous round's pending d, this round's phase e^{-i g C} and sums the
-// result; a one-block kernel turns the sum into the next d.  The vector kept
+// result, which the next pass turns into its d.  The vector kept
 // in memory is phi_r = e^{-i g_r C} psi_{r-1} (with d_r beside it), which is
 // also what the adjoint sweep needs of round r.
 //
@@ -32,8 +32,8 @@
 // Sums: float32 over a thread's 8 amplitudes of a tile; across the tiles a
 // thread visits in a compensated (Kahan) float32 pair, which keeps about
 // float64 accuracy without float64 arithmetic per tile (slow on this part);
-// float64 across the block and over the blocks, in a fixed order, so results
-// are bitwise reproducible run to run.
+// float pairs within a warp and float64 across warps and blocks, in a fixed
+// order, so results are bitwise reproducible run to run.
 #include "common.cuh"
 #include "bulk.cuh"
 
@@ -55,7 +55,7 @@ constexpr int kR1BlocksPerSM = 8;                // upper bound used to size the
 constexpr uint32_t kR1RedOff = 2 * kR1MaxStages * 8;
 constexpr uint32_t kR1TabOff = 512;
 constexpr uint32_t kR1HeadB = kR1TabOff + kPhaseTable * 8;
-static_assert(kR1RedOff + 3 * (kR1Threads / 32) * 8 <= kR1TabOff, "head layout");
+static_assert(kR1RedOff + 3 * (kR1Threads / 32) * 8 + 8 * 8 <= kR1TabOff, "head layout");
 static_assert(kR1HeadB % 128 == 0, "stage area alignment");
 constexpr float kTwoPiF = 6.2831853071795864769f;
 
@@ -91,36 +91,30 @@ __device__ __forceinline__ int r1_find(const uint32_t *__restrict__ tb, int nd, 
     return lo;
 }
 
+// Tiles of a launch in contiguous runs of equal length (to one tile), one per
+// block: a block enters as few units as possible (each entry and each exit
+// costs a block a microsecond or two; dealt round-robin, 4 sets of 705432 states
+// sent every block through every set).
+struct R1Deal {
+    uint32_t q, rem;
+    __device__ __forceinline__ R1Deal(uint32_t total, uint32_t G) : q(total / G), rem(total % G) {}
+    __device__ __forceinline__ uint32_t start(uint32_t b) const { return b * q + min(b, rem); }
+    __device__ __forceinline__ uint32_t block_of(uint32_t t) const {
+        const uint32_t big = rem * (q + 1);
+        return t < big ? t / (q + 1) : rem + (t - big) / q;
+    }
+};
+
 // Barrier over the kR1Threads consumer threads only (named barrier 1; the
 // producer warp never takes part).
 __device__ __forceinline__ void r1_consumer_sync() {
     asm volatile("bar.sync 1, %0;" ::"n"(kR1Threads) : "memory");
 }
 
-// Sum of three float64 values over the kR1Threads consumer threads (or the
-// whole block of the scalar kernel, CONSUMERS false), in a fixed order; the
-// result is valid in thread 0.  Every participating thread must call it.
-template <bool CONSUMERS>
-__device__ __forceinline__ void r1_block_sum3(double (&v)[3], double (*red)[kR1Threads / 32]) {
-#pragma unroll
-    for (int q = 0; q < 3; q++)
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    if (CONSUMERS) r1_consumer_sync();  // red is free (an earlier sum has been read)
-    else __syncthreads();
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < 3; q++) red[q][w] = v[q];
-    if (CONSUMERS) r1_consumer_sync();
-    else __syncthreads();
-    if (threadIdx.x == 0)
-#pragma unroll
-        for (int q = 0; q < 3; q++) {
-            double s = 0.0;
-            for (int i = 0; i < kR1Threads / 32; i++) s += red[q][i];
-            v[q] = s;
-        }
+// Exact sum of two floats as a float pair.
+__device__ __forceinline__ float2 r1_two_sum(float a, float b) {
+    const float t = a + b, z = t - a;
+    return make_float2(t, (a - (t - z)) + (b - z));
 }
 
 // Cost values of the pair (x, x + 1); `two` false: only x is in range.
@@ -162,8 +156,36 @@ struct Kahan {
         lo = (t - hi) - y;
         hi = t;
     }
-    __device__ __forceinline__ double value() const { return (double)hi - (double)lo; }
 };
+
+// Sums of three running sums over the consumer threads, in a fixed order, as
+// float pairs within a warp (about float64 accuracy; a float64 add takes 16
+// cycles of the SM a warp) and in float64 over the warps: thread q < 3 returns
+// sum q.  Every consumer thread must call it.
+__device__ __forceinline__ double r1_block_sum3(const Kahan (&acc)[3], float2 (*red)[kR1Threads / 32]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    float2 v[3];
+#pragma unroll
+    for (int q = 0; q < 3; q++) {
+        v[q] = make_float2(acc[q].hi, -acc[q].lo);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float h = __shfl_xor_sync(0xffffffffu, v[q].x, o), l = __shfl_xor_sync(0xffffffffu, v[q].y, o);
+            const float2 t = r1_two_sum(v[q].x, h);
+            const float lo = t.y + (v[q].y + l);
+            v[q] = r1_two_sum(t.x, lo);
+        }
+    }
+    r1_consumer_sync();  // red is free (an earlier sum has been read)
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < 3; q++) red[q][w] = v[q];
+    r1_consumer_sync();
+    double s = 0.0;
+    if (threadIdx.x < 3)
+        for (int i = 0; i < kR1Threads / 32; i++) s += (double)red[threadIdx.x][i].x + (double)red[threadIdx.x][i].y;
+    return s;
+}
 
 template <int COST>
 __device__ __forceinline__ float2 r1_phase(const float2 *stab, float C, int ci, const RoundCoef &cf) {
@@ -201,29 +223,39 @@ struct R1Unit {
     bool gen, first, ckpt;
 };
 
-// One streaming pass over every tile of every unit of the launch.  Tiles go to
-// blocks round-robin (block b: tiles b, b + G, ...), so each unit's tiles form
-// one run per block.  Modes, for round r:
+// One streaming pass over every tile of every unit of the launch.  Modes, for
+// round r:
 //   R1_FWD : phi_r = (phi_{r-1} + d_{r-1}) e^{-i g_r C} (r = 0: the initial
 //            state); sums (Re, Im) of phi_r
 //   R1_LAST: psi = phi_{p-1} + d_{p-1}; sums C |psi|^2, Re and Im of C psi
 //   R1_BWD : lambda_r (stored, or (C - c0) psi_{p-1} for r = p - 1), mu,
 //            the gamma_r sum; for r > 0 lambda_{r-1} stored and summed, and
 //            without checkpoints phi_{r-1} recovered in place
-// Each block writes one (sum, sum, sum) slot per unit it visited: slot
-// (b - tile_begin[unit]) mod G.
+// Each block writes one (sum, sum, sum) slot per unit it visits: slot (block -
+// first block of the unit), in half `half` of the unit's slots.  The next
+// pass's blocks sum the slots (of the `grid_in` blocks that wrote them, the
+// other half) as they enter the unit and form the scalars they need themselves,
+// all alike; the unit's first block writes those that later passes and the
+// caller need.  (A one-block kernel between any two passes did this before, 13
+// of 5.9 us and their gaps in a 6-round gradient: 4 sets of 705432 states 459 ->
+// 301 us with the contiguous runs, 64 sets of 2^16 1205 -> 469, one of 2^28
+// 14.81 -> 14.77 ms.)
 template <int MODE, int COST>
 __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__restrict__ descs,
                                                               const uint32_t *__restrict__ tb, int nd,
-                                                              uint32_t total, int round, int nst, int *err) {
+                                                              uint32_t total, uint32_t grid_in, int half,
+                                                              int round, int nst, int *err) {
     using SG = R1Stage<MODE, COST>;
     extern __shared__ __align__(128) unsigned char r1_smem[];
     uint64_t *full_bar = reinterpret_cast<uint64_t *>(r1_smem);
     uint64_t *empty_bar = full_bar + kR1MaxStages;
-    double(*red)[kR1Threads / 32] = reinterpret_cast<double(*)[kR1Threads / 32]>(r1_smem + kR1RedOff);
+    float2(*red)[kR1Threads / 32] = reinterpret_cast<float2(*)[kR1Threads / 32]>(r1_smem + kR1RedOff);
+    double *s_in = reinterpret_cast<double *>(r1_smem + kR1RedOff + 3 * (kR1Threads / 32) * 8);
     float2 *stab = reinterpret_cast<float2 *>(r1_smem + kR1TabOff);
     unsigned char *stages = r1_smem + kR1HeadB;
     const uint32_t G = gridDim.x;
+    const R1Deal deal(total, G);
+    const uint32_t t0 = deal.start(blockIdx.x), t1 = deal.start(blockIdx.x + 1);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         for (int k = 0; k < nst; k++) {
@@ -241,7 +273,7 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
         int64_t N = 0;
         const void *src_v = nullptr, *src_l = nullptr, *src_c = nullptr;
         uint32_t i = 0;
-        for (uint32_t t = blockIdx.x; t < total; t += G, i++) {
+        for (uint32_t t = t0; t < t1; t++, i++) {
             const uint32_t s = i % (uint32_t)nst;
             const uint32_t fb = smem_u32(&full_bar[s]);
             if (i >= (uint32_t)nst && !fail && !mbar_wait(smem_u32(&empty_bar[s]), ((i / nst) - 1) & 1u)) {
@@ -290,18 +322,80 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
     Kahan acc[3];
     bool fail = false;
     auto flush = [&]() {
-        double v[3] = {acc[0].value(), acc[1].value(), acc[2].value()};
-        r1_block_sum3<true>(v, red);
-        if (tid == 0) {
-            double *pp = D->part + (size_t)U.slot * 3;
-            pp[0] = v[0];
-            pp[1] = v[1];
-            pp[2] = v[2];
-        }
+        const double v = r1_block_sum3(acc, red);
+        if (tid < 3) D->part[((size_t)half * D->slots + U.slot) * 3 + tid] = v;
         acc[0] = acc[1] = acc[2] = Kahan();
     };
+    // The scalars of the previous pass (see the top of the file), for every
+    // thread in s_in: FWD, LAST: d of the round before; BWD: c0 and m.
+    const bool has_in = !(MODE == R1_FWD && round == 0);
+    auto scalars = [&]() {
+        const int p = D->p;
+        const double inv = D->inv_dim;
+        double *sc = D->scal;
+        if (warp == 0) {
+            const R1Deal prev(total, grid_in);
+            const uint32_t b0 = prev.block_of(U.t_lo), ns = prev.block_of(U.t_hi - 1) - b0 + 1;
+            const double *pp = D->part + (size_t)(half ^ 1) * D->slots * 3;
+            double v[3] = {0.0, 0.0, 0.0};
+            for (uint32_t j = lane; j < ns; j += 32)
+#pragma unroll
+                for (int q = 0; q < 3; q++) v[q] += pp[3 * j + q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int q = 0; q < 3; q++) v[q] += __shfl_xor_sync(0xffffffffu, v[q], o);
+            if (lane < 3) s_in[lane] = lane == 0 ? v[0] : lane == 1 ? v[1] : v[2];
+        } else if (warp == 1 && lane == 0) {
+            // e^{s i b} - 1 = 2 i s sin(b/2) e^{s i b/2}: (re, im) without cancellation at small b
+            constexpr double kInv2Pi = 0.15915494309189533577;
+            double sh, ch;
+            sincospi(D->angles[MODE == R1_FWD ? round - 1 : MODE == R1_LAST ? p - 1 : round] * kInv2Pi, &sh, &ch);
+            s_in[3] = -2.0 * sh * sh;
+            s_in[4] = (MODE == R1_BWD ? 2.0 : -2.0) * sh * ch;
+        }
+        r1_consumer_sync();
+        if (tid == 0) {
+            const double A = s_in[0], B = s_in[1], Cs = s_in[2], fr = s_in[3], fi = s_in[4];
+            const bool first = U.slot == 0;  // the block that keeps the unit's scalars
+            if (MODE != R1_BWD) {
+                const int r = MODE == R1_FWD ? round - 1 : p - 1;
+                const double dr = (fr * A - fi * B) * inv, dim = (fr * B + fi * A) * inv;
+                if (first) {
+                    sc[4 * r] = dr;
+                    sc[4 * r + 1] = dim;
+                    sc[4 * r + 2] = A;
+                    sc[4 * r + 3] = B;
+                }
+                s_in[5] = dr;
+                s_in[6] = dim;
+            } else {
+                const double N = (double)D->dim;
+                // sum psi_r = S_r + N d_r
+                const double Pr = sc[4 * round + 2] + N * sc[4 * round], Pi = sc[4 * round + 3] + N * sc[4 * round + 1];
+                double Lr = B, Li = Cs, c0;  // L = sum lambda_r
+                if (round == p - 1) {
+                    c0 = A;
+                    Lr = B - A * Pr;
+                    Li = Cs - A * Pi;
+                    if (first) {
+                        *D->E = A;
+                        sc[4 * p] = A;
+                    }
+                } else {
+                    c0 = sc[4 * p];
+                    if (first) D->grad[p + round + 1] = 2.0 * A;
+                }
+                if (first) D->grad[round] = 2.0 * (Lr * Pi - Li * Pr) * inv;
+                s_in[5] = (fr * Lr - fi * Li) * inv;
+                s_in[6] = (fr * Li + fi * Lr) * inv;
+                s_in[7] = c0;
+            }
+        }
+        r1_consumer_sync();
+    };
     uint32_t i = 0;
-    for (uint32_t t = blockIdx.x; t < total; t += G, i++) {
+    for (uint32_t t = t0; t < t1; t++, i++) {
         const uint32_t s = i % (uint32_t)nst;
         if (!D || t >= U.t_hi) {  // entering a unit (uniform over the consumers)
             if (D) flush();
@@ -309,7 +403,7 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
             D = descs + di;
             U.t_lo = tb[di];
             U.t_hi = tb[di + 1];
-            U.slot = (blockIdx.x + G - U.t_lo % G) % G;
+            U.slot = blockIdx.x - deal.block_of(U.t_lo);
             U.N = D->dim;
             const int64_t ld = D->ld;
             const int p = D->p;
@@ -318,27 +412,26 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
             U.ckpt = D->ckpt != 0;
             U.gen = MODE == R1_FWD && round == 0 && !D->init;
             U.first = MODE == R1_BWD && round == p - 1;
+            if (COST == 1 && MODE != R1_LAST) {  // (the previous unit's last readers passed flush's barriers)
+                for (int k = tid; k < kPhaseTable; k += kR1Threads) stab[k] = D->table[round * kPhaseTable + k];
+                if (!has_in) r1_consumer_sync();
+            }
+            if (has_in) scalars();
             if (MODE == R1_FWD) {
                 U.in = round == 0 ? D->init : D->phi + (U.ckpt ? (int64_t)(round - 1) * ld : 0);
                 U.out = D->phi + (U.ckpt ? (int64_t)round * ld : 0);
-                U.dp = round == 0 ? make_float2(0.f, 0.f)
-                                  : make_float2((float)sc[4 * (round - 1)], (float)sc[4 * (round - 1) + 1]);
+                U.dp = has_in ? make_float2((float)s_in[5], (float)s_in[6]) : make_float2(0.f, 0.f);
             } else if (MODE == R1_LAST) {
                 U.in = D->phi + (U.ckpt ? (int64_t)(p - 1) * ld : 0);
-                U.dp = make_float2((float)sc[4 * (p - 1)], (float)sc[4 * (p - 1) + 1]);
+                U.dp = make_float2((float)s_in[5], (float)s_in[6]);
             } else {
                 U.out = D->phi + (U.ckpt ? (int64_t)round * ld : 0);
                 U.in = U.out;
-                U.c0 = (float)sc[4 * p];
-                U.m = make_float2((float)sc[4 * p + 1], (float)sc[4 * p + 2]);
+                U.c0 = (float)s_in[7];
+                U.m = make_float2((float)s_in[5], (float)s_in[6]);
                 U.dp = make_float2((float)sc[4 * round], (float)sc[4 * round + 1]);
                 U.dq = round > 0 ? make_float2((float)sc[4 * (round - 1)], (float)sc[4 * (round - 1) + 1])
                                  : make_float2(0.f, 0.f);
-            }
-            if (COST == 1 && MODE != R1_LAST) {
-                r1_consumer_sync();  // the previous unit's table is no longer read
-                for (int k = tid; k < kPhaseTable; k += kR1Threads) stab[k] = D->table[round * kPhaseTable + k];
-                r1_consumer_sync();
             }
         }
         bool ok = !fail && mbar_wait(smem_u32(&full_bar[s]), (i / nst) & 1u);
@@ -464,73 +557,24 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
         for (int k = 0; k < nst; k++) mbar_wait(smem_u32(&full_bar[k]), 0u), mbar_wait(smem_u32(&full_bar[k]), 1u);
 }
 
-// Scalars between passes, one block per unit: the unit's block slots summed
-// in slot order, then the round's scalar formulas in float64.
-//   R1_SFWD (round r): S_r = sum phi_r, d_r = (e^{-i b_r} - 1) S_r / N
-//   R1_SLAST: <C> to E; with gradients c0 = <C>, sum lambda_{p-1} =
-//             sum C psi - c0 sum psi, the beta_{p-1} partial and
-//             m = (e^{+i b_{p-1}} - 1) sum lambda_{p-1} / N
-//   R1_SBWD (round r): the gamma_r partial; for r > 0 the beta_{r-1} partial
-//             and m for round r - 1
+// After the last pass, one warp per unit: its slots' first sums, <C> (an
+// expectation run's R1_LAST) or the gamma_0 partial.
 // Scalar layout per unit: [4 r + 0, 1] = d_r, [4 r + 2, 3] = S_r (r < p),
-// [4 p] = c0, [4 p + 1, 2] = m of the round the adjoint is at.
-__global__ void __launch_bounds__(kR1Threads) r1_scalar_kernel(const R1Desc *__restrict__ descs,
-                                                              const uint32_t *__restrict__ tb, uint32_t grid,
-                                                              int mode, int round) {
-    __shared__ double red[3][kR1Threads / 32];
-    const R1Desc D = descs[blockIdx.x];
-    const uint32_t nt = tb[blockIdx.x + 1] - tb[blockIdx.x];
-    const uint32_t ns = nt < grid ? nt : grid;
-    double v[3] = {0.0, 0.0, 0.0};
-    for (uint32_t i = threadIdx.x; i < ns; i += kR1Threads) {
-        v[0] += D.part[3 * i];
-        v[1] += D.part[3 * i + 1];
-        v[2] += D.part[3 * i + 2];
+// [4 p] = c0.
+__global__ void __launch_bounds__(32) r1_final_kernel(const R1Desc *__restrict__ descs, const uint32_t *__restrict__ tb,
+                                                      uint32_t total, uint32_t grid_in, int half) {
+    const R1Desc &D = descs[blockIdx.x];
+    const R1Deal prev(total, grid_in);
+    const uint32_t b0 = prev.block_of(tb[blockIdx.x]), ns = prev.block_of(tb[blockIdx.x + 1] - 1) - b0 + 1;
+    const double *pp = D.part + (size_t)half * D.slots * 3;
+    double v = 0.0;
+    for (uint32_t j = threadIdx.x; j < ns; j += 32) v += pp[3 * j];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (threadIdx.x == 0) {
+        if (D.grad) D.grad[D.p] = 2.0 * v;
+        else *D.E = v;
     }
-    r1_block_sum3<false>(v, red);
-    if (threadIdx.x != 0) return;
-    const double A = v[0], B = v[1], Cs = v[2];
-    double *sc = D.scal;
-    const double N = (double)D.dim;
-    const int p = D.p;
-    constexpr double kInv2Pi = 0.15915494309189533577;
-    // e^{s i b} - 1 = 2 i s sin(b/2) e^{s i b/2}: (re, im) without cancellation at small b
-    auto mixer_factor = [&](double beta, double sgn, double &re, double &im) {
-        double sh, ch;
-        sincospi(beta * kInv2Pi, &sh, &ch);  // sin(b/2), cos(b/2)
-        re = -2.0 * sh * sh;
-        im = sgn * 2.0 * sh * ch;
-    };
-    if (mode == R1_SFWD) {
-        double fr, fi;
-        mixer_factor(D.angles[round], -1.0, fr, fi);
-        sc[4 * round + 2] = A;
-        sc[4 * round + 3] = B;
-        sc[4 * round] = (fr * A - fi * B) / N;
-        sc[4 * round + 1] = (fr * B + fi * A) / N;
-        return;
-    }
-    // beta_r partial and m for round r from L = sum lambda_r
-    auto adjoint_round = [&](int r, double Lr, double Li) {
-        const double Pr = sc[4 * r + 2] + N * sc[4 * r];  // sum psi_r = S_r + N d_r
-        const double Pi = sc[4 * r + 3] + N * sc[4 * r + 1];
-        D.grad[r] = 2.0 * (Lr * Pi - Li * Pr) / N;
-        double fr, fi;
-        mixer_factor(D.angles[r], 1.0, fr, fi);
-        sc[4 * p + 1] = (fr * Lr - fi * Li) / N;
-        sc[4 * p + 2] = (fr * Li + fi * Lr) / N;
-    };
-    if (mode == R1_SLAST) {
-        *D.E = A;
-        if (!D.grad) return;
-        sc[4 * p] = A;
-        const double Pr = sc[4 * (p - 1) + 2] + N * sc[4 * (p - 1)];
-        const double Pi = sc[4 * (p - 1) + 3] + N * sc[4 * (p - 1) + 1];
-        adjoint_round(p - 1, B - A * Pr, Cs - A * Pi);
-        return;
-    }
-    D.grad[p + round] = 2.0 * A;
-    if (round > 0) adjoint_round(round - 1, B, Cs);
 }
 
 }  // namespace
@@ -583,33 +627,33 @@ uint32_t r1_grid(int mode, int cost_dtype) {
 }
 
 template <int MODE, int COST>
-cudaError_t r1_go(const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles, uint32_t grid, int round, int *err,
-                  cudaStream_t s) {
+cudaError_t r1_go(const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles, uint32_t grid, uint32_t grid_in, int half,
+                  int round, int *err, cudaStream_t s) {
     static int attr_done[kMaxDevices] = {0};
     const R1Config c = r1_config<MODE, COST>();
     cudaError_t e = smem_attr_once(r1_pass_kernel<MODE, COST>, (int)c.smem, attr_done);
     if (e != cudaSuccess) return e;
-    r1_pass_kernel<MODE, COST><<<grid, kR1Block, c.smem, s>>>(d, tb, nd, tiles, round, c.nst, err);
+    r1_pass_kernel<MODE, COST><<<grid, kR1Block, c.smem, s>>>(d, tb, nd, tiles, grid_in, half, round, c.nst, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_r1_pass(int mode, int cost_dtype, const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles,
-                           uint32_t grid, int round, int *err, cudaStream_t s) {
+                           uint32_t grid, uint32_t grid_in, int half, int round, int *err, cudaStream_t s) {
     if (tiles == 0 || grid == 0) return cudaSuccess;
     if (cost_dtype == 0) {
-        if (mode == R1_FWD) return r1_go<R1_FWD, 0>(d, tb, nd, tiles, grid, round, err, s);
-        if (mode == R1_LAST) return r1_go<R1_LAST, 0>(d, tb, nd, tiles, grid, round, err, s);
-        return r1_go<R1_BWD, 0>(d, tb, nd, tiles, grid, round, err, s);
+        if (mode == R1_FWD) return r1_go<R1_FWD, 0>(d, tb, nd, tiles, grid, grid_in, half, round, err, s);
+        if (mode == R1_LAST) return r1_go<R1_LAST, 0>(d, tb, nd, tiles, grid, grid_in, half, round, err, s);
+        return r1_go<R1_BWD, 0>(d, tb, nd, tiles, grid, grid_in, half, round, err, s);
     }
-    if (mode == R1_FWD) return r1_go<R1_FWD, 1>(d, tb, nd, tiles, grid, round, err, s);
-    if (mode == R1_LAST) return r1_go<R1_LAST, 1>(d, tb, nd, tiles, grid, round, err, s);
-    return r1_go<R1_BWD, 1>(d, tb, nd, tiles, grid, round, err, s);
+    if (mode == R1_FWD) return r1_go<R1_FWD, 1>(d, tb, nd, tiles, grid, grid_in, half, round, err, s);
+    if (mode == R1_LAST) return r1_go<R1_LAST, 1>(d, tb, nd, tiles, grid, grid_in, half, round, err, s);
+    return r1_go<R1_BWD, 1>(d, tb, nd, tiles, grid, grid_in, half, round, err, s);
 }
 
-cudaError_t launch_r1_scalar(int mode, const R1Desc *d, const uint32_t *tb, int nd, uint32_t grid, int round,
-                             cudaStream_t s) {
+cudaError_t launch_r1_final(const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles, uint32_t grid_in, int half,
+                            cudaStream_t s) {
     if (nd <= 0) return cudaSuccess;
-    r1_scalar_kernel<<<nd, kR1Threads, 0, s>>>(d, tb, grid, mode, round);
+    r1_final_kernel<<<nd, 32, 0, s>>>(d, tb, tiles, grid_in, half);
     return cudaGetLastError();
 }
 

@@ -78,7 +78,7 @@ struct Unit {
 };
 
 enum LaunchKind { LK_PREP, LK_SMALL, LK_XPASS, LK_REDUCE, LK_EIG_INIT, LK_EIG_GEMM, LK_COST_MEAN, LK_ORBIT,
-                  LK_OPERANDS, LK_R1_PASS, LK_R1_SCALAR, LK_GRID };
+                  LK_OPERANDS, LK_R1_PASS, LK_R1_FINAL, LK_GRID };
 
 struct LaunchRec {
     int kind;
@@ -103,11 +103,11 @@ struct LaunchRec {
     int gather = 0;      // pass launches: gathered tiles
     int fused = 0;       // pass launches: round-boundary passes (PF_FUSED)
     double *mean_out = nullptr;  // LK_COST_MEAN: where the cost mean goes
-    // Grover-mixer (rank-one) launches: mode, round and the pass grid, which
-    // fixes the slot layout the following scalar launch reads
-    int r1mode = 0, r1round = 0;
+    // Grover-mixer (rank-one) launches: mode, round, the pass grid and that of
+    // the pass before it (which fixes the slot layout it reads), half of the slots
+    int r1mode = 0, r1round = 0, r1half = 0;
     int gn = 0;  // LK_GRID: qubits (the largest of a cooperative launch)
-    uint32_t r1grid = 0;
+    uint32_t r1grid = 0, r1in = 0;
     // grouped (block-diagonal) products and orbit kernels
     int grouped = 0, n_mtiles = 0, lda = 0, ldb = 0;
     const GroupTile *gtiles = nullptr;
@@ -1691,9 +1691,9 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         used += need;
                         wtiles += ru.nt;
                         ru.part_off = r1_meta;
-                        r1_meta = align_up(r1_meta + sizeof(double) * 3 * std::min<uint32_t>(ru.nt, gmax));
+                        r1_meta = align_up(r1_meta + sizeof(double) * 2 * 3 * std::min<uint32_t>(ru.nt, gmax));
                         ru.scal_off = r1_meta;
-                        r1_meta = align_up(r1_meta + sizeof(double) * (4 * u.p + 3));
+                        r1_meta = align_up(r1_meta + sizeof(double) * (4 * u.p + 1));
                         w.us.push_back(ru);
                         r1_need = std::max(r1_need, used);
                     }
@@ -1725,6 +1725,8 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         d.grad = grad ? u.grad : nullptr;
                         d.dim = u.dim;
                         d.ld = ru.ld;
+                        d.inv_dim = 1.0 / (double)u.dim;
+                        d.slots = std::min<uint32_t>(ru.nt, gmax);
                         d.p = u.p;
                         d.ckpt = ru.ck;
                         d.amp0 = (float)(1.0 / std::sqrt((double)u.dim));
@@ -1752,6 +1754,8 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         return b;
                     };
                     const char *mname[3] = {"fwd", "last", "bwd"};
+                    uint32_t grid_in = 0;
+                    int half = 0;
                     auto add = [&](int mode, int round) {
                         LaunchRec r;
                         r.kind = LK_R1_PASS;
@@ -1763,26 +1767,30 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         r.r1mode = mode;
                         r.r1round = round;
                         r.r1grid = std::min<uint32_t>(tb.back(), r1_grid(mode, w.dt));
+                        r.r1in = grid_in;
+                        r.r1half = half;
                         r.bytes = pass_bytes_r1(mode, round);
                         char nm[48];
                         snprintf(nm, sizeof(nm), "grover_r1_%s_%s", mname[mode], dtype_name(w.dt));
                         r.fam = family(ctx, nm);
                         L.push_back(r);
-                        LaunchRec q;
-                        q.kind = LK_R1_SCALAR;
-                        q.desc_off = doff;
-                        q.tb_off = toff;
-                        q.ndesc = (int)ds.size();
-                        q.r1mode = mode == R1_FWD ? R1_SFWD : (mode == R1_LAST ? R1_SLAST : R1_SBWD);
-                        q.r1round = round;
-                        q.r1grid = r.r1grid;
-                        q.fam = family(ctx, "grover_r1_scalar");
-                        L.push_back(q);
+                        grid_in = r.r1grid;
+                        half ^= 1;
                     };
                     for (int k = 0; k < w.p; k++) add(R1_FWD, k);
                     add(R1_LAST, w.p - 1);
                     if (grad)
                         for (int k = w.p - 1; k >= 0; k--) add(R1_BWD, k);
+                    LaunchRec q;  // <C>, or the last gamma partial
+                    q.kind = LK_R1_FINAL;
+                    q.desc_off = doff;
+                    q.tb_off = toff;
+                    q.ndesc = (int)ds.size();
+                    q.tiles = tb.back();
+                    q.r1in = grid_in;
+                    q.r1half = half ^ 1;
+                    q.fam = family(ctx, "grover_r1_final");
+                    L.push_back(q);
                 }
             }
         }
@@ -2195,13 +2203,13 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             break;
         case LK_R1_PASS:
             e = launch_r1_pass(r.r1mode, r.cost_dtype, reinterpret_cast<const R1Desc *>(db + r.desc_off),
-                               reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles, r.r1grid,
-                               r.r1round, ctx->d_err, ctx->stream);
+                               reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles, r.r1grid, r.r1in,
+                               r.r1half, r.r1round, ctx->d_err, ctx->stream);
             break;
-        case LK_R1_SCALAR:
-            e = launch_r1_scalar(r.r1mode, reinterpret_cast<const R1Desc *>(db + r.desc_off),
-                                 reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.r1grid, r.r1round,
-                                 ctx->stream);
+        case LK_R1_FINAL:
+            e = launch_r1_final(reinterpret_cast<const R1Desc *>(db + r.desc_off),
+                                reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles, r.r1in, r.r1half,
+                                ctx->stream);
             break;
         case LK_COST_MEAN:
             e = launch_cost_mean(r.ep.cost, r.ep.cost_dtype, r.ep.M, r.mean_out, ctx->stream);
