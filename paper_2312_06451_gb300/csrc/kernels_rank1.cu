@@ -265,6 +265,7 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
         fence_mbar_init();
     }
     __syncthreads();
+    chain_begin();
 
     if (warp == kR1Threads / 32) {  // ---------------------------- producer
         if (lane != 0) return;
@@ -563,6 +564,7 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
 // [4 p] = c0.
 __global__ void __launch_bounds__(32) r1_final_kernel(const R1Desc *__restrict__ descs, const uint32_t *__restrict__ tb,
                                                       uint32_t total, uint32_t grid_in, int half) {
+    chain_begin();
     const R1Desc &D = descs[blockIdx.x];
     const R1Deal prev(total, grid_in);
     const uint32_t b0 = prev.block_of(tb[blockIdx.x]), ns = prev.block_of(tb[blockIdx.x + 1] - 1) - b0 + 1;
@@ -633,8 +635,8 @@ cudaError_t r1_go(const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles, u
     const R1Config c = r1_config<MODE, COST>();
     cudaError_t e = smem_attr_once(r1_pass_kernel<MODE, COST>, (int)c.smem, attr_done);
     if (e != cudaSuccess) return e;
-    r1_pass_kernel<MODE, COST><<<grid, kR1Block, c.smem, s>>>(d, tb, nd, tiles, grid_in, half, round, c.nst, err);
-    return cudaGetLastError();
+    return launch_chained(r1_pass_kernel<MODE, COST>, grid, kR1Block, c.smem, s, d, tb, nd, tiles, grid_in, half, round,
+                          c.nst, err);
 }
 
 cudaError_t launch_r1_pass(int mode, int cost_dtype, const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles,
@@ -653,8 +655,7 @@ cudaError_t launch_r1_pass(int mode, int cost_dtype, const R1Desc *d, const uint
 cudaError_t launch_r1_final(const R1Desc *d, const uint32_t *tb, int nd, uint32_t tiles, uint32_t grid_in, int half,
                             cudaStream_t s) {
     if (nd <= 0) return cudaSuccess;
-    r1_final_kernel<<<nd, 32, 0, s>>>(d, tb, tiles, grid_in, half);
-    return cudaGetLastError();
+    return launch_chained(r1_final_kernel, nd, 32, 0, s, d, tb, tiles, grid_in, half);
 }
 
 }  // namespace qg

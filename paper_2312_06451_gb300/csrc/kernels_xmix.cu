@@ -217,8 +217,11 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
     const PrepDesc D = descs[blockIdx.x];
     // nb angles per round's mixer (nq qubits for multi-angle, else 1):
     // beta_{k,q} = angles[k nb + q], gamma_k = angles[p nb + k]
+    // The coefficients' float64 chain is long: with a table to fill, one warp
+    // forms them while the others fill it.
     const int nb = D.nq ? D.nq : 1;
-    for (int e = threadIdx.x; e < (D.gm_n ? 0 : D.p * nb); e += blockDim.x) {
+    const int tid = threadIdx.x, nt = blockDim.x, tab0 = D.table ? 32 : nt;  // table threads from tab0
+    for (int e = tid; !D.gm_n && tid < tab0 && e < D.p * nb; e += tab0) {
         const int k = e / nb;
         const double be = D.angles[e], ga = D.angles[D.p * nb + k];
         if (!isfinite(be) || !isfinite(ga)) atomicOr(err, DERR_BAD_ANGLE);
@@ -244,7 +247,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
             const double g = ga * kInvTwoPi;
             c.g_hi = (float)g;
             c.g_lo = (float)(g - (double)c.g_hi);
-            c.b_hi = c.b_lo = c.pad[0] = c.pad[1] = 0.f;
+            c.b_hi = c.b_lo = c.c_lo = c.pad = 0.f;
             for (int j = 0; j <= kPassTileBits; j++) c.pw[j] = 1.f;  // direct form: no cosine factors
             D.coef[e] = c;
         }
@@ -256,9 +259,9 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
             D.wtab[e] = make_float4(cs, -sn, (float)G, 0.f);
         }
     }
-    if (D.table) {
+    if (D.table && tid >= tab0) {
         const int tot = D.p * D.tsize;
-        for (int e = threadIdx.x; e < tot; e += blockDim.x) {
+        for (int e = tid - tab0; e < tot; e += nt - tab0) {
             const int k = e / D.tsize, cst = e - k * D.tsize;
             // e^{-i gamma c} from the turn count gamma c / (2 pi)
             const double g = D.angles[D.p * nb + k] * kInvTwoPi;
@@ -271,6 +274,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
 // Fixed-order two-level reduction of the per-(tile, warp) partial sums.
 __global__ void __launch_bounds__(256) reduce1_kernel(const RedChunk *__restrict__ chunks, double *level2) {
     __shared__ double red[8];
+    chain_begin();
     const RedChunk C = chunks[blockIdx.x];
     double acc = 0.0;
     for (int i = threadIdx.x; i < C.cnt; i += 256) acc += C.src[i];
@@ -286,6 +290,7 @@ __global__ void __launch_bounds__(256) reduce1_kernel(const RedChunk *__restrict
 }
 
 __global__ void __launch_bounds__(32) reduce2_kernel(const RedOut *__restrict__ outs, const double *level2) {
+    chain_begin();
     const RedOut O = outs[blockIdx.x];
     double acc = 0.0;
     for (int i = threadIdx.x; i < O.n; i += 32) acc += level2[O.first + i];
@@ -358,11 +363,9 @@ cudaError_t launch_prep(const PrepDesc *d, int nd, int *err, cudaStream_t s) {
 
 cudaError_t launch_reduce(const RedChunk *chunks, int nchunks, double *level2, const RedOut *outs, int nouts,
                           cudaStream_t s) {
-    reduce1_kernel<<<nchunks, 256, 0, s>>>(chunks, level2);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_chained(reduce1_kernel, nchunks, 256, 0, s, chunks, level2);
     if (e != cudaSuccess) return e;
-    reduce2_kernel<<<nouts, 32, 0, s>>>(outs, level2);
-    return cudaGetLastError();
+    return launch_chained(reduce2_kernel, nouts, 32, 0, s, outs, static_cast<const double *>(level2));
 }
 
 }  // namespace qg

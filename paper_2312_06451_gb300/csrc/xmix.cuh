@@ -92,6 +92,14 @@ __device__ __forceinline__ float2 phase_turns(float ghi, float glo, float c) {
 
 constexpr double kInvTwoPi = 0.15915494309189533577;  // 1 / (2 pi)
 
+// Product of two float pairs (value x + y, |y| at most half an ulp of x).
+__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
+    const float p = a.x * b.x;
+    const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x);
+    const float t = p + e;
+    return make_float2(t, e - (t - p));
+}
+
 // Round coefficients from one beta (rotation) and the round's gamma.
 __device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
     const double bb = be * kInvTwoPi;
@@ -130,7 +138,8 @@ __device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
                            c8 * c2 * ce, c8 * c4};
 #pragma unroll
     for (int k = 0; k <= kPassTileBits; k++) c.pw[k] = (float)pw[k];
-    c.pad[0] = c.pad[1] = 0.f;
+    c.c_lo = (float)(ce - (double)c.pw[1]);
+    c.pad = 0.f;
     return c;
 }
 

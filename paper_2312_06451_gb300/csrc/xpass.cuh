@@ -698,6 +698,7 @@ xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ ti
     unsigned char *bufs = smem_raw + G::kHead;
     __shared__ PassDesc D;
     __shared__ float4 s_rot[12];  // multi-angle: (cos, +-sin, +-tan, cos^2) per local bit
+    __shared__ float2 s_cc[12];   // multi-angle: cosines as float pairs (1 where not rotated)
     __shared__ float4 s_w[33];    // general X mixer: weight phases and G(w)
     __shared__ uint32_t s_tr[3];  // D's first tile, end tile and index
     __shared__ PassConst s_k[2];  // the round's constants (round-boundary launches: rounds k and k+1)
@@ -708,6 +709,7 @@ xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ ti
         fence_mbar_init();
     }
     __syncthreads();
+    chain_begin();
     const uint32_t stride = gridDim.x;
     int cursor = 0;  // loader's descriptor search position (warp 0)
     if (warp == 0) {
@@ -780,25 +782,29 @@ xpass_kernel(const PassDesc *__restrict__ descs, const uint32_t *__restrict__ ti
                     const float c = q.bmode == 0 ? q.pw[1] : q.cb;
                     s_rot[tid] = make_float4(q.cb, sgn * q.sb, sgn * q.bt, c * c);
                     const bool on = (D.active >> tid) & 1u;
+                    s_cc[tid] = on ? make_float2(q.pw[1], q.c_lo) : make_float2(1.f, 0.f);
                     tan_ok = !on || q.bmode == 0;
                     resc = on && q.rescale;
                 }
                 tan_ok = __syncthreads_and(tan_ok);
                 resc = __syncthreads_or(resc) && tan_ok;
                 if (tid == 0) {
-                    auto prod = [&](int b0) {
-                        float f = 1.f;
-                        for (int j = b0; j < b0 + 4; j++)
-                            if ((D.active >> j) & 1u) f *= D.coef[D.gpos[j]].pw[1];
-                        return tan_ok ? f : 1.f;
+                    // products of the rotated qubits' cosines as float pairs (a
+                    // rounding here would scale every amplitude of the pass alike)
+                    auto prod = [&](int b0) -> float2 {
+                        float2 f = make_float2(1.f, 0.f);
+#pragma unroll
+                        for (int j = b0; j < b0 + 4; j++) f = pair_mul(f, s_cc[j]);
+                        return f;
                     };
+                    const float2 fq = prod(4), fr = prod(0), fp = prod(8);
                     PassConst &K = s_k[0];
                     K.R.mode = tan_ok ? 0 : 2;
                     K.rescale = resc ? 1 : 0;
-                    K.fsq = prod(4);
-                    K.fsr = prod(0);
-                    K.fsp = prod(8);
-                    K.fse = resc ? 1.f : K.fsq * K.fsr * K.fsp;
+                    K.fsq = tan_ok ? fq.x : 1.f;
+                    K.fsr = tan_ok ? fr.x : 1.f;
+                    K.fsp = tan_ok ? fp.x : 1.f;
+                    K.fse = tan_ok && !resc ? pair_mul(pair_mul(fq, fr), fp).x : 1.f;
                 }
             }
             __syncthreads();
@@ -876,8 +882,8 @@ cudaError_t launch_one(const PassDesc *d, const uint32_t *tb, int nd, uint32_t t
         __atomic_store_n(&grid_caps[dev], grid_cap, __ATOMIC_RELEASE);
     }
     const uint32_t grid = std::min<uint32_t>(tiles, (uint32_t)grid_cap);
-    xpass_kernel<BWD, COST, NBUF, VAR, FUSED, GATH><<<grid, kNT, smem, s>>>(d, tb, nd, tiles, err, sched);
-    return cudaGetLastError();
+    return launch_chained(xpass_kernel<BWD, COST, NBUF, VAR, FUSED, GATH>, grid, kNT, smem, s, d, tb, nd, tiles, err,
+                          sched);
 }
 
 template <int VAR, int FUSED, int GATH>
