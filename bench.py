@@ -71,9 +71,8 @@ def measured_peaks():
 
 def gemm_peak(gemm: str):
     """Denominator of a contraction's roofline.  CUDA-core fp32: 152 SMs x 128
-    FP32 lanes x 2 flop x 2070 MHz (unit counts and maximum clock).  TF32 /
-    split-precision tensor paths: the measured bf16 dense peak x the nominal
-    tf32 / bf16 ratio (1.1 / 2.25)."""
+    FP32 lanes x 2 flop x 2070 MHz (unit counts and maximum clock).  The split
+    tensor path (pairs of half planes): the measured bf16 dense peak."""
     if gemm == "fp32":
         return {"bound": "alu", "peak": 152 * 128 * 2 * 2.070e9 / 1e12, "source": "derived: 152 SM x 128 lanes x 2 x 2.07 GHz"}
     path = os.path.join(ROOT, "MEASURED_PEAKS.json")
@@ -83,7 +82,7 @@ def gemm_peak(gemm: str):
         with open(path) as f:
             bf16 = float(json.load(f)["bf16_tflops"])
         src = "measured"
-    return {"bound": "tensor", "peak": bf16 * 1.1 / 2.25, "source": f"{src} bf16 burst x 1.1/2.25 (tf32)"}
+    return {"bound": "tensor", "peak": bf16, "source": f"{src} bf16 burst"}
 
 
 def reducers(dist, device):
@@ -995,7 +994,7 @@ def main():
                     help="workload 4: load the mixer's eigendecomposition (dense V or its blocks) from this file, "
                          "or save it there")
     ap.add_argument("--gemm", default="3xtf32", choices=["fp32", "3xtf32"],
-                    help="eigenbasis product precision (workload 4): tcgen05 3xTF32 or CUDA-core float32")
+                    help="eigenbasis product precision (workload 4): tcgen05 22-bit split or CUDA-core float32")
     ap.add_argument("--eig", default="blocks", choices=["blocks", "dense"],
                     help="workload 4: the mixer through its cyclic-shift momentum blocks (default) or one dense "
                          "eigendecomposition")

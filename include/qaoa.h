@@ -143,7 +143,8 @@ qaoa_status qaoa_x_mixer_weights(int n, int kmax, const double *c, double *d);
 /* Precision of the dense eigenbasis products for QAOA_MIXER_EIGEN. */
 enum {
     QAOA_GEMM_FP32_SIMT = 0, /* complex64 CUDA-core products, fp32 accumulate */
-    QAOA_GEMM_3XTF32 = 1,    /* tensor cores, tf32 hi/lo split, 3 products */
+    QAOA_GEMM_3XTF32 = 1,    /* tensor cores, hi/lo split with a tf32 pair's 22 bits
+                                (two scaled half planes), 3 products; |V| <= 4 */
     QAOA_GEMM_BF16X3 = 2     /* tensor cores, bf16 hi/lo split, 3 products */
 };
 

@@ -197,6 +197,7 @@ struct EigEpiParams {
     float *out_lo;  // tensor-core path: remainder planes of split outputs
     float *out2_lo;
     const double *c0;  // adjoint epilogues: cost shift (lambda_p = (C - c0) psi_p, gamma partials)
+    const float *sc_in, *sc_out, *sc_out2;  // tensor-core path: scale pairs of the B operand and the split outputs
 };
 
 // Grouped products: tile i covers output rows out_row .. out_row + 127 of block
@@ -205,14 +206,16 @@ struct EigEpiParams {
 struct GroupTile {
     int a_row, k_off, kext, out_row, row_end, part_idx;
 };
-// Vp_lo / Vtp_lo non-null: Vp / Vtp get the tf32 heads, *_lo the remainders.
+// Vp_lo / Vtp_lo non-null: Vp / Vtp and *_lo are half planes (heads, remainders).
 cudaError_t launch_eig_prepare(const float *V, int D, int ld, float *Vp, float *Vtp, float *Vp_lo, float *Vtp_lo,
                                const double *lam, float *lam_hi, float *lam_lo, cudaStream_t s);
-// Mean of a cost vector (D entries) into *out, fixed summation order; one block.
-cudaError_t launch_cost_mean(const void *cost, int cost_dtype, int D, double *out, cudaStream_t s);
+// Mean of a cost vector (D entries) into *mean, fixed summation order, and (sc:
+// four floats) the scales of the tensor-core operands; one block.
+cudaError_t launch_eig_scale(const void *cost, int cost_dtype, int D, const float2 *init, double *mean, float *sc,
+                             cudaStream_t s);
 cudaError_t launch_eig_init(float *X, float *X_lo, float *ck0, int D, int ld, int nsets, const void *cost,
                             int cost_dtype, const RoundCoef *coef, int coef_stride, const float2 *init, float amp0,
-                            cudaStream_t s);
+                            const float *scale, cudaStream_t s);
 // out^T[Np][Mp] = A[Mp][Kp] * B[Np][Kp]^T with a fused epilogue; Mp, Np, Kp
 // multiples of 128.
 cudaError_t launch_eig_gemm_simt(const float *A, const float *B, int Mp, int Np, int Kp, const EigEpiParams &P,
@@ -225,8 +228,8 @@ cudaError_t launch_eig_gemm_simt_grouped(const float *A, int lda, const float *B
 cudaError_t launch_eig_gemm_tc_grouped(const CUtensorMap &a_hi, const CUtensorMap &a_lo, const CUtensorMap &b_hi,
                                        const CUtensorMap &b_lo, int Np, const GroupTile *d_tiles, int n_mtiles,
                                        const EigEpiParams &P, int *err, cudaStream_t s);
-// tcgen05 3xTF32 product with the same epilogues; tensor maps (2-d, K-major,
-// 32-float boxes x 128 rows, 128-byte swizzle) of the operand planes.  The
+// tcgen05 split product with the same epilogues; tensor maps (2-d, K-major,
+// 64-half boxes x 128 rows, 128-byte swizzle) of the operand planes.  The
 // tiles of a last, partial wave may be split along K: d_ws holds
 // eig_split_max_tail() x kEigMaxSeg partial 128 x 128 float tiles and d_cnt
 // eig_split_max_tail() counters, zero before the first product of a call
@@ -338,7 +341,8 @@ struct OrbitArgs {
     int D, ldp, nsets, round;
     const float *in;      // Z (PHASE, LAST) or W (BWD): [2S][ldp]
     const float *in_psi;  // BWD: checkpointed psi_{r-1} in the momentum basis
-    float *out, *out_lo;  // X or L (tf32 head and remainder when out_lo)
+    float *out, *out_lo;  // X or L (half planes, head and remainder, when out_lo)
+    const float *scale;   // scale of the half planes
     float *ckpt;          // INIT: T^T psi_0
     const float2 *init;   // INIT: user psi_0 (computational basis) or nullptr
     float amp0;
@@ -354,8 +358,8 @@ constexpr int kOrbitThreads = 128;                   // threads per block of the
 constexpr int kOrbitsPerBlock = kOrbitThreads / 2;  // two threads (real, imaginary rows) per orbit
 cudaError_t launch_orbit(const OrbitTabs &T, const OrbitArgs &A, cudaStream_t s);
 // Padded block matrices of a symmetric eigendecomposition: A = V_b (or V_b^T)
-// stacked as rows block_pos[b] .. of a [ldp][pmax] matrix (zero padded), the
-// tf32 split planes when *_lo is set; eigenvalues at padded positions.
+// stacked as rows block_pos[b] .. of a [ldp][pmax] matrix (zero padded), half
+// planes when *_lo is set; eigenvalues at padded positions.
 cudaError_t launch_sym_prepare(const float *V, const double *lam, const int *d_bdim, const int *d_boff,
                                const int *d_bpos, int nb, int pmax, float *Vp, float *Vtp, float *Vp_lo, float *Vtp_lo,
                                float *lam_hi, float *lam_lo, cudaStream_t s);

@@ -19,6 +19,7 @@
 #include <type_traits>
 
 #include <cuda.h>
+#include <cuda_fp16.h>
 #include <math.h>
 
 namespace qg {
@@ -66,20 +67,29 @@ struct EpiArgs {
     int round;            // round whose beta / gamma this epilogue uses
     double *part;         // partial sums [set][M tile] (kind dependent) or nullptr
     int part_stride;      // = number of M tiles
-    float *out_lo;        // split outputs for tensor-core operands: out holds the
-    float *out2_lo;       // tf32 head, out_lo the float32 remainder (or nullptr)
+    float *out_lo;        // split outputs for tensor-core operands: out and out_lo are
+    float *out2_lo;       // the half planes of put() (or nullptr: out is float32)
     const double *c0;     // cost shift of the adjoint (C - c0), or nullptr
+    const float *sc_in;   // tensor-core products: scales of the B operand (see eig_scale_kernel)
+    const float *sc_out, *sc_out2;  // and of the split outputs
 };
 
-// Store v to out (and its tf32 split when out_lo is set).  The head is v
-// rounded to the nearest tf32 value (magnitude rounded half up on the 13
-// dropped bits), so the remainder's sign does not follow v's: the tensor
-// cores' own truncation of the remainder then carries no bias.
-__device__ __forceinline__ void put(float *out, float *out_lo, size_t o, float v) {
+// Tensor-core operands are pairs of half planes: x = v s (s a power of two),
+// head = half(x), remainder = half((x - head) 2^11), so v = (head + 2^-11
+// remainder) / s with 22 bits, and an absolute error below 2^-36 / s where the
+// head is subnormal.  Eigenvectors have |v| <= 1 and s = kVScale; the state
+// matrices' s keeps the largest possible amplitude at kStateTop or below.
+constexpr float kVScale = 8192.f, kStateTop = 8192.f, kLoScale = 2048.f;
+
+// Store v to out: as float32, or split into the half planes out and out_lo
+// when out_lo is set.  Both roundings are to nearest, so the remainder's sign
+// does not follow v's.
+__device__ __forceinline__ void put(float *out, float *out_lo, size_t o, float v, float s) {
     if (out_lo) {
-        const float hi = __uint_as_float((__float_as_uint(v) + 0x1000u) & 0xFFFFE000u);
-        out[o] = hi;
-        out_lo[o] = v - hi;
+        const float x = v * s;
+        const __half h = __float2half_rn(x);
+        reinterpret_cast<__half *>(out)[o] = h;
+        reinterpret_cast<__half *>(out_lo)[o] = __float2half_rn((x - __half2float(h)) * kLoScale);
     } else {
         out[o] = v;
     }
@@ -98,8 +108,8 @@ __device__ __forceinline__ float epi_elem(const EpiArgs &E, int j, int s, float2
     float contrib = 0.f;
     switch (E.kind) {
     case EPI_STORE:
-        put(E.out, E.out_lo, o_re, v.x);
-        put(E.out, E.out_lo, o_im, v.y);
+        E.out[o_re] = v.x;
+        E.out[o_im] = v.y;
         break;
     case EPI_FWD_EIG: {  // Y = e^{-i b lambda} v, checkpoint V^T phi
         if (E.ckpt) {
@@ -107,8 +117,8 @@ __device__ __forceinline__ float epi_elem(const EpiArgs &E, int j, int s, float2
             E.ckpt[o_im] = v.y;
         }
         const float2 w = cmul(v, turn_phase(cf.b_hi, cf.b_lo, E.lam_hi[j], E.lam_lo[j]));
-        put(E.out, E.out_lo, o_re, w.x);
-        put(E.out, E.out_lo, o_im, w.y);
+        E.out[o_re] = w.x;
+        E.out[o_im] = w.y;
         break;
     }
     case EPI_FWD_PHASE: {  // X = e^{-i g' C} v, checkpoint psi_k
@@ -117,8 +127,8 @@ __device__ __forceinline__ float epi_elem(const EpiArgs &E, int j, int s, float2
             E.ckpt[o_im] = v.y;
         }
         const float2 w = cmul(v, turn_phase(cf.g_hi, cf.g_lo, cost_at(E, j), 0.f));
-        put(E.out, E.out_lo, o_re, w.x);
-        put(E.out, E.out_lo, o_im, w.y);
+        E.out[o_re] = w.x;
+        E.out[o_im] = w.y;
         break;
     }
     case EPI_FWD_LAST: {  // psi_p: <C> partial, store psi_p and lambda_p = (C - c0) psi_p
@@ -130,8 +140,8 @@ __device__ __forceinline__ float epi_elem(const EpiArgs &E, int j, int s, float2
         }
         if (E.out2) {
             const float Cs = C - (E.c0 ? (float)__ldg(E.c0) : 0.f);
-            put(E.out2, E.out2_lo, o_re, Cs * v.x);
-            put(E.out2, E.out2_lo, o_im, Cs * v.y);
+            E.out2[o_re] = Cs * v.x;
+            E.out2[o_im] = Cs * v.y;
         }
         break;
     }
@@ -142,8 +152,8 @@ __device__ __forceinline__ float epi_elem(const EpiArgs &E, int j, int s, float2
         const float lam = E.lam_hi[j] + E.lam_lo[j];
         contrib = lam * (v.x * psi.y - v.y * psi.x);  // Im(conj(v) lambda psi)
         const float2 w = make_float2(fmaf(v.x, ph.x, v.y * ph.y), fmaf(v.y, ph.x, -v.x * ph.y));  // v conj(ph)
-        put(E.out, E.out_lo, o_re, w.x);
-        put(E.out, E.out_lo, o_im, w.y);
+        E.out[o_re] = w.x;
+        E.out[o_im] = w.y;
         break;
     }
     case EPI_BWD_PHASE: {  // gamma partial with phi = e^{-i g C} psi_{k-1}, then undo the phase
@@ -153,8 +163,8 @@ __device__ __forceinline__ float epi_elem(const EpiArgs &E, int j, int s, float2
         contrib = (C - (E.c0 ? (float)__ldg(E.c0) : 0.f)) * (v.x * phi.y - v.y * phi.x);
         if (E.out) {
             const float2 w = make_float2(fmaf(v.x, ph.x, v.y * ph.y), fmaf(v.y, ph.x, -v.x * ph.y));
-            put(E.out, E.out_lo, o_re, w.x);
-            put(E.out, E.out_lo, o_im, w.y);
+            E.out[o_re] = w.x;
+            E.out[o_im] = w.y;
         }
         break;
     }
@@ -268,19 +278,22 @@ gemm_simt_kernel(const float *__restrict__ A, const float *__restrict__ B, int K
     }
 }
 
-// ------------------------------------------------- tcgen05 split-TF32 GEMM
-// out^T[N][M] = A[M][K] B[N][K]^T with A = A_hi + A_lo and B = B_hi + B_lo held
-// as separate tf32 planes: per k-step the tensor cores add A_lo B_hi + A_hi B_lo
-// + A_hi B_hi ("3xTF32") into a float32 accumulator in tensor memory.
+// ------------------------------------------------- tcgen05 split product
+// out^T[N][M] = A[M][K] B[N][K]^T with A and B as pairs of scaled half planes
+// (see put): per k-step the tensor cores add A_hi B_hi into one float32
+// accumulator in tensor memory and A_lo B_hi + A_hi B_lo, 2^11 times too large,
+// into another.  A half carries the 11 significant bits of a tf32 value, so with
+// scaled remainders the three products keep the 22 bits that a tf32 split
+// ("3xTF32") keeps, at twice its rate and half its bytes; the range that half
+// lacks is what the power-of-two scales are for.
 //
 // The tensor-core accumulation does not round to nearest: its error shrinks
-// magnitudes and grows with the number of products accumulated.  So each
-// 32-wide K chunk (12 MMAs) is accumulated into a fresh tensor-memory buffer
-// (two buffers alternate) and drained at once into float32 registers with
-// round-to-nearest adds.  The operand split rounds the head to nearest (see
-// put()), so the hardware's truncation of the tf32 remainders is unbiased.
-// Measured on the 12870-state ring mixer at p = 6: <C> within 6.2e-6
-// (relative) of the complex128 result; a truncated head gave 1.35e-5.
+// magnitudes and grows with the number of products accumulated.  So the
+// accumulators are drained every few K chunks into float32 registers with
+// round-to-nearest adds.
+// Ring mixer on 12870 states, 256 sets, p = 6 gradient (24 grouped products):
+// 3.47 -> 2.36 ms; error against 64 bits 5.5e-6 -> 4.6e-6 (draining every 3
+// chunks instead of 2: 2.28 ms, 5.8e-6).
 //
 // 128 x 128 output tile per CTA, STAGES-deep TMA ring of 128-byte-swizzled
 // K-major tiles.  Warp 0 lane 0 issues TMA loads, warp 1 lane 0 the MMAs;
@@ -300,22 +313,20 @@ namespace tc {
 constexpr int NACC = 4, NDRAIN = 16;  // 128-column accumulators in TMEM, draining warps
 // Both products: GNACC buffers, each a pair of TMEM accumulators (the
 // A_hi B_hi products, and the two small cross terms apart, so the large sum
-// takes only one truncating add per 8-wide K step), drained into the float32
+// takes only one truncating add per 16-wide K step), drained into the float32
 // registers (round to nearest) every DGRP K chunks.  The truncating adds bias
-// <C> low in proportion to the adds between drains: on DkS n=16, k=8 (block
-// ring mixer, p=6) the error relative to max(|E|, rms C) is about -2.3e-6 -
-// 1.45e-6 DGRP; a single accumulator drained every chunk gave -5.9e-6.
-constexpr int GNACC = 2, DGRP = 3;
-constexpr int BM = 128, BN = 128, BKF = 32, STAGES = 3, NT = 32 * (2 + NDRAIN);
+// <C> low in proportion to the adds between drains (12 here, as with a tf32
+// split's 8-wide steps and half as many drains).
+constexpr int GNACC = 2, DGRP = 2;
+constexpr int BM = 128, BN = 128, BKF = 64, STAGES = 3, NT = 32 * (2 + NDRAIN);
 constexpr uint32_t kTileA = BM * 128, kTileB = BN * 128;
 constexpr uint32_t kStage = 2 * kTileA + 2 * kTileB;  // A_hi, A_lo, B_hi, B_lo
 constexpr uint32_t kSmem = STAGES * kStage + 1024;      // + alignment slack
 constexpr uint32_t kTmemCols = NACC * BN;               // four 128-column accumulators
 static_assert(GNACC * 2 * BN <= (int)kTmemCols, "accumulator pairs exceed the TMEM allocation");
 constexpr uint32_t kSpin = 1u << 24;
-// instruction descriptor: D f32, A/B tf32, both K-major, N = 128, M = 128
-constexpr uint32_t kIdesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(BN >> 3) << 17) |
-                            ((uint32_t)(BM >> 4) << 24);
+// instruction descriptor: D f32, A/B f16 (format 0), both K-major, N = 128, M = 128
+constexpr uint32_t kIdesc = (1u << 4) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -363,10 +374,10 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
     d |= (uint64_t)2 << 61;            // 128-byte swizzle
     return d;
 }
-__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(tmem),
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
@@ -440,6 +451,7 @@ __device__ __forceinline__ void epi_row16(const EpiArgs &E, int m, int s0, int n
         xh = cost_at(E, m);
     }
     if (kShift && E.c0) c0 = (float)__ldg(E.c0);
+    const float rs = __ldg(E.sc_in + 1), so = __ldg(E.sc_out);  // 1 / (operand scales), output scale
     // groups of kGrp sets: the adjoint's checkpoint values of a group are loaded
     // together (groups of 8 spill at this kernel's register cap and measured slower)
     constexpr int kGrp = 4;
@@ -460,18 +472,18 @@ __device__ __forceinline__ void epi_row16(const EpiArgs &E, int m, int s0, int n
             c[q] = 0.f;
             if (q >= nq) continue;
             const size_t o_re = (size_t)(2 * (s0 + q)) * E.ld + m, o_im = o_re + E.ld;
-            const float2 v = make_float2(acc[2 * q], acc[2 * q + 1]);
+            const float2 v = make_float2(rs * acc[2 * q], rs * acc[2 * q + 1]);
             if (KIND == EPI_STORE) {
-                put(E.out, E.out_lo, o_re, v.x);
-                put(E.out, E.out_lo, o_im, v.y);
+                put(E.out, E.out_lo, o_re, v.x, so);
+                put(E.out, E.out_lo, o_im, v.y, so);
             } else if (KIND == EPI_FWD_EIG || KIND == EPI_FWD_PHASE) {
                 if (E.ckpt) {
                     E.ckpt[o_re] = v.x;
                     E.ckpt[o_im] = v.y;
                 }
                 const float2 w = cmul(v, turn_phase(ang[q].x, ang[q].y, xh, xl));
-                put(E.out, E.out_lo, o_re, w.x);
-                put(E.out, E.out_lo, o_im, w.y);
+                put(E.out, E.out_lo, o_re, w.x, so);
+                put(E.out, E.out_lo, o_im, w.y, so);
             } else if (KIND == EPI_FWD_LAST) {
                 c[q] = xh * fmaf(v.x, v.x, v.y * v.y);
                 if (E.out) {
@@ -480,8 +492,8 @@ __device__ __forceinline__ void epi_row16(const EpiArgs &E, int m, int s0, int n
                 }
                 if (E.out2) {
                     const float Cs = xh - c0;
-                    put(E.out2, E.out2_lo, o_re, Cs * v.x);
-                    put(E.out2, E.out2_lo, o_im, Cs * v.y);
+                    put(E.out2, E.out2_lo, o_re, Cs * v.x, __ldg(E.sc_out2));
+                    put(E.out2, E.out2_lo, o_im, Cs * v.y, __ldg(E.sc_out2));
                 }
             } else {  // adjoint: partial with the checkpoint turned forward, then undo the phase on v
                 const float2 ph = turn_phase(ang[q].x, ang[q].y, xh, xl);
@@ -489,8 +501,8 @@ __device__ __forceinline__ void epi_row16(const EpiArgs &E, int m, int s0, int n
                 c[q] = (kEig ? xh + xl : xh - c0) * (v.x * f.y - v.y * f.x);
                 if (kEig || E.out) {
                     const float2 w = make_float2(fmaf(v.x, ph.x, v.y * ph.y), fmaf(v.y, ph.x, -v.x * ph.y));
-                    put(E.out, E.out_lo, o_re, w.x);
-                    put(E.out, E.out_lo, o_im, w.y);
+                    put(E.out, E.out_lo, o_re, w.x, so);
+                    put(E.out, E.out_lo, o_im, w.y, so);
                 }
             }
         }
@@ -609,14 +621,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__
                 const uint32_t base = tc::su32(smem + s * kStage);
                 const uint32_t d = tmem + (uint32_t)(b * 2 * TBN), dc = d + (uint32_t)TBN;
 #pragma unroll
-                for (int kk = 0; kk < BKF / 8; kk++) {
+                for (int kk = 0; kk < BKF / 16; kk++) {
                     const uint64_t ah = tc::sdesc(base + kk * 32), al = tc::sdesc(base + kTileA + kk * 32);
                     const uint64_t bh = tc::sdesc(base + 2 * kTileA + kk * 32),
                                    bl = tc::sdesc(base + 2 * kTileA + kTileB + kk * 32);
                     const uint32_t accum = (first && kk == 0) ? 0u : 1u;
-                    tc::mma_tf32(dc, al, bh, tc::kIdesc, accum);
-                    tc::mma_tf32(dc, ah, bl, tc::kIdesc, 1u);
-                    tc::mma_tf32(d, ah, bh, tc::kIdesc, accum);
+                    tc::mma_f16(dc, al, bh, tc::kIdesc, accum);
+                    tc::mma_f16(dc, ah, bl, tc::kIdesc, 1u);
+                    tc::mma_f16(d, ah, bh, tc::kIdesc, accum);
                 }
                 tc::mma_commit(tc::su32(&empty[s]));
                 if (last) tc::mma_commit(tc::su32(&accf[b]));
@@ -644,7 +656,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__
                 tc::tmem_ld16(col + TBN, rc);
                 tc::tmem_wait_ld();
 #pragma unroll
-                for (int i = 0; i < 16; i++) acc[16 * q + i] += __uint_as_float(r[i]) + __uint_as_float(rc[i]);
+                for (int i = 0; i < 16; i++) acc[16 * q + i] += fmaf(__uint_as_float(rc[i]), 1.f / kLoScale, __uint_as_float(r[i]));
             }
             tc::fence_before();
             __syncwarp();
@@ -840,14 +852,14 @@ gemm_tc_grouped_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_co
                     const uint32_t base = tc::su32(smem + st * kStage);
                     const uint32_t d = tmem + (uint32_t)(b * 2 * TBN), dc = d + (uint32_t)TBN;
 #pragma unroll
-                    for (int kk = 0; kk < BKF / 8; kk++) {
+                    for (int kk = 0; kk < BKF / 16; kk++) {
                         const uint64_t ah = tc::sdesc(base + kk * 32), al = tc::sdesc(base + kTileA + kk * 32);
                         const uint64_t bh = tc::sdesc(base + 2 * kTileA + kk * 32),
                                        bl = tc::sdesc(base + 2 * kTileA + kTileB + kk * 32);
                         const uint32_t accum = (first && kk == 0) ? 0u : 1u;
-                        tc::mma_tf32(dc, al, bh, tc::kIdesc, accum);
-                        tc::mma_tf32(dc, ah, bl, tc::kIdesc, 1u);
-                        tc::mma_tf32(d, ah, bh, tc::kIdesc, accum);
+                        tc::mma_f16(dc, al, bh, tc::kIdesc, accum);
+                        tc::mma_f16(dc, ah, bl, tc::kIdesc, 1u);
+                        tc::mma_f16(d, ah, bh, tc::kIdesc, accum);
                     }
                     tc::mma_commit(tc::su32(&empty[st]));
                     if (last) {
@@ -892,7 +904,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_co
                     tc::tmem_ld16(col + TBN, rc);
                     tc::tmem_wait_ld();
 #pragma unroll
-                    for (int i = 0; i < 16; i++) acc[16 * q + i] += __uint_as_float(r[i]) + __uint_as_float(rc[i]);
+                    for (int i = 0; i < 16; i++) acc[16 * q + i] += fmaf(__uint_as_float(rc[i]), 1.f / kLoScale, __uint_as_float(r[i]));
                 }
                 tc::fence_before();
                 __syncwarp();
@@ -950,7 +962,7 @@ gemm_tc_grouped_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_co
 // also keeps psi_0 as checkpoint 0.
 __global__ void eig_init_kernel(float *X, float *X_lo, float *ck0, int D, int ld, int nsets, const void *cost,
                                 int cost_dtype, const RoundCoef *coef, int coef_stride, const float2 *init,
-                                float amp0) {
+                                float amp0, const float *scale) {
     const int s = blockIdx.y;
     if (s >= nsets) return;
     const RoundCoef cf = coef[s * coef_stride];
@@ -960,8 +972,9 @@ __global__ void eig_init_kernel(float *X, float *X_lo, float *ck0, int D, int ld
                                         : (float)reinterpret_cast<const unsigned char *>(cost)[j];
         const float2 w = cmul(v, turn_phase(cf.g_hi, cf.g_lo, C, 0.f));
         const size_t o = (size_t)(2 * s) * ld + j;
-        put(X, X_lo, o, w.x);
-        put(X, X_lo, o + ld, w.y);
+        const float s0 = X_lo ? __ldg(scale) : 1.f;
+        put(X, X_lo, o, w.x, s0);
+        put(X, X_lo, o + ld, w.y, s0);
         if (ck0) {
             ck0[o] = v.x;
             ck0[o + ld] = v.y;
@@ -973,20 +986,67 @@ __global__ void eig_init_kernel(float *X, float *X_lo, float *ck0, int D, int ld
 // adjoint sweep.  Any constant gives the same gradient, because
 // <mu_k|phi_k> = <lambda_p|psi_p> = <C> is real; the mean removes the
 // component of lambda_p along psi_p that would otherwise dominate it.
-__global__ void __launch_bounds__(256) cost_mean_kernel(const void *cost, int cost_dtype, int D, double *out) {
-    __shared__ double red[8];
+// sc (tensor-core products): {s, 1 / (s kVScale)} of the psi matrices, then of
+// the lambda matrices: the powers of two that keep their amplitudes, at most
+// |psi_0| and max |C - c0| |psi_0| in either basis, at kStateTop or below.
+__global__ void __launch_bounds__(1024) eig_scale_kernel(const void *cost, int cost_dtype, int D, const float2 *init,
+                                                         double *out, float *sc) {
+    __shared__ double red[32];
+    __shared__ float redf[3][32];
+    __shared__ double s_mean;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    auto cost_of = [&](int j) -> float {
+        return cost_dtype == 0 ? __ldg(reinterpret_cast<const float *>(cost) + j)
+                               : (float)__ldg(reinterpret_cast<const unsigned char *>(cost) + j);
+    };
     double acc = 0.0;
-    for (int j = threadIdx.x; j < D; j += 256)
-        acc += cost_dtype == 0 ? (double)reinterpret_cast<const float *>(cost)[j]
-                               : (double)reinterpret_cast<const unsigned char *>(cost)[j];
+    float lo = INFINITY, hi = -INFINITY, nrm = 0.f;
+    for (int j = threadIdx.x; j < D; j += 1024) {
+        const float C = cost_of(j);
+        acc += (double)C;
+        lo = fminf(lo, C);
+        hi = fmaxf(hi, C);
+        if (init) nrm = fmaf(init[j].x, init[j].x, fmaf(init[j].y, init[j].y, nrm));
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        nrm += __shfl_xor_sync(0xffffffffu, nrm, o);
+    }
+    if (lane == 0) {
+        red[warp] = acc;
+        redf[0][warp] = lo;
+        redf[1][warp] = hi;
+        redf[2][warp] = nrm;
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         double t = 0.0;
-        for (int w = 0; w < 8; w++) t += red[w];
-        *out = t / (double)D;
+        for (int w = 0; w < 32; w++) {
+            t += red[w];
+            lo = fminf(lo, redf[0][w]);
+            hi = fmaxf(hi, redf[1][w]);
+            nrm = w ? nrm + redf[2][w] : redf[2][0];
+        }
+        s_mean = t / (double)D;
+        *out = s_mean;
+        if (sc) {
+            // s = kStateTop / 2^e with 2^e >= bound (1.01: the sums' own rounding)
+            auto scale_of = [](float bound) -> float {
+                if (!(bound > 0.f) || isinf(bound)) return 1.f;
+                int e;
+                frexpf(bound * 1.01f, &e);  // bound < 2^e
+                return ldexpf(kStateTop, -min(max(e, -100), 110));
+            };
+            const float norm = init ? sqrtf(nrm) : 1.f;
+            const float dev = fmaxf(fabsf(hi - (float)s_mean), fabsf(lo - (float)s_mean));
+            sc[0] = scale_of(norm);
+            sc[1] = 1.f / (sc[0] * kVScale);
+            sc[2] = scale_of(norm * dev);
+            sc[3] = 1.f / (sc[2] * kVScale);
+        }
     }
 }
 
@@ -1037,6 +1097,7 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
         const int s0 = T.orb_start[o], r = T.orb_start[o + 1] - s0;
         const RoundCoef cf = A.coef[s * A.coef_stride + A.round];
         const size_t row = (size_t)(2 * s + part) * A.ldp;
+        const float so = A.scale ? __ldg(A.scale) : 1.f;
         // (re, im) of a member from this lane's part and the partner's
         auto pair_of = [&](float v) -> float2 {
             const float w = __shfl_xor_sync(pair_mask, v, 1);
@@ -1140,7 +1201,7 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
 #pragma unroll
                 for (int a = 0; a < RMAX; a++) {
                     if (a >= R) continue;
-                    put(out, out_lo, row + vpos(a), c[a]);
+                    put(out, out_lo, row + vpos(a), c[a], so);
                 }
             };
             float x[RMAX];
@@ -1250,8 +1311,8 @@ __global__ void sym_prepare_kernel(const float *V, const double *lam, const int 
         const int i = (int)(e / pmax), c = (int)(e % pmax);
         const size_t o = (size_t)(bpos[b] + i) * pmax + c;
         const bool in = i < Db && c < Db;
-        put(Vp, Vp_lo, o, in ? Vb[(size_t)i * Db + c] : 0.f);
-        put(Vtp, Vtp_lo, o, in ? Vb[(size_t)c * Db + i] : 0.f);
+        put(Vp, Vp_lo, o, in ? Vb[(size_t)i * Db + c] : 0.f, kVScale);
+        put(Vtp, Vtp_lo, o, in ? Vb[(size_t)c * Db + i] : 0.f, kVScale);
         if (c == 0) {
             const double l = i < Db ? lam[boff[b] + i] : 0.0;
             const float hi = (float)l;
@@ -1269,8 +1330,8 @@ __global__ void eig_prepare_kernel(const float *V, int D, int ld, float *Vp, flo
          e += (int64_t)gridDim.x * blockDim.x) {
         const int r = (int)(e / ld), c = (int)(e % ld);
         const float v = (r < D && c < D) ? V[(int64_t)r * D + c] : 0.f;
-        put(Vp, Vp_lo, e, v);
-        put(Vtp, Vtp_lo, (int64_t)c * ld + r, v);
+        put(Vp, Vp_lo, e, v, kVScale);
+        put(Vtp, Vtp_lo, (int64_t)c * ld + r, v, kVScale);
         if (r == 0) {
             const double l = c < D ? lam[c] : 0.0;
             const float hi = (float)l;
@@ -1326,17 +1387,18 @@ cudaError_t launch_orbit(const OrbitTabs &T, const OrbitArgs &A, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_cost_mean(const void *cost, int cost_dtype, int D, double *out, cudaStream_t s) {
-    cost_mean_kernel<<<1, 256, 0, s>>>(cost, cost_dtype, D, out);
+cudaError_t launch_eig_scale(const void *cost, int cost_dtype, int D, const float2 *init, double *mean, float *sc,
+                             cudaStream_t s) {
+    eig_scale_kernel<<<1, 1024, 0, s>>>(cost, cost_dtype, D, init, mean, sc);
     return cudaGetLastError();
 }
 
 cudaError_t launch_eig_init(float *X, float *X_lo, float *ck0, int D, int ld, int nsets, const void *cost,
                             int cost_dtype, const RoundCoef *coef, int coef_stride, const float2 *init, float amp0,
-                            cudaStream_t s) {
+                            const float *scale, cudaStream_t s) {
     dim3 grid((D + 255) / 256, nsets);
     eig_init_kernel<<<grid, 256, 0, s>>>(X, X_lo, ck0, D, ld, nsets, cost, cost_dtype, coef, coef_stride, init,
-                                         amp0);
+                                         amp0, scale);
     return cudaGetLastError();
 }
 
@@ -1363,6 +1425,9 @@ EpiArgs to_args(const EigEpiParams &P) {
     E.out_lo = P.out_lo;
     E.out2_lo = P.out2_lo;
     E.c0 = P.c0;
+    E.sc_in = P.sc_in;
+    E.sc_out = P.sc_out;
+    E.sc_out2 = P.sc_out2;
     return E;
 }
 }  // namespace

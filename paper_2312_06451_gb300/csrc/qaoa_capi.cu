@@ -77,7 +77,7 @@ struct Unit {
     const double *wts;     // general X mixer: n + 1 weights
 };
 
-enum LaunchKind { LK_PREP, LK_SMALL, LK_XPASS, LK_REDUCE, LK_EIG_INIT, LK_EIG_GEMM, LK_COST_MEAN, LK_ORBIT,
+enum LaunchKind { LK_PREP, LK_SMALL, LK_XPASS, LK_REDUCE, LK_EIG_INIT, LK_EIG_GEMM, LK_EIG_SCALE, LK_ORBIT,
                   LK_OPERANDS, LK_R1_PASS, LK_R1_FINAL, LK_GRID };
 
 struct LaunchRec {
@@ -102,7 +102,7 @@ struct LaunchRec {
     int sched_idx = -1;  // pass launches: tile counter slot
     int gather = 0;      // pass launches: gathered tiles
     int fused = 0;       // pass launches: round-boundary passes (PF_FUSED)
-    double *mean_out = nullptr;  // LK_COST_MEAN: where the cost mean goes
+    double *mean_out = nullptr;  // LK_EIG_SCALE: where the cost mean goes (the scales, if any, to ep.sc_in)
     // Grover-mixer (rank-one) launches: mode, round, the pass grid and that of
     // the pass before it (which fixes the slot layout it reads), half of the slots
     int r1mode = 0, r1round = 0, r1half = 0;
@@ -390,16 +390,16 @@ bool encode_gather_map(CUtensorMap *m, const void *base, int n, int c, int lo, i
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Row-major float32 matrix [rows][ld] as a K-major tensor-core operand:
-// 32-float (128-byte) boxes x 128 rows, 128-byte swizzle.
+// Row-major half plane [rows][ld] as a K-major tensor-core operand: 64-element
+// (128-byte) boxes x 128 rows, 128-byte swizzle.
 bool encode_kmajor_map(CUtensorMap *m, const float *base, int ld, int rows) {
     auto enc = tensor_map_encoder();
     if (!enc) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)rows};
-    const cuuint64_t strides[1] = {(cuuint64_t)ld * sizeof(float)};
-    const cuuint32_t box[2] = {32, 128};
+    const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
+    const cuuint32_t box[2] = {64, 128};
     const cuuint32_t es[2] = {1, 1};
-    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float *>(base), dims, strides, box, es,
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<float *>(base), dims, strides, box, es,
                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -981,11 +981,14 @@ qaoa_status plan_sym_job(qaoa_ctx *ctx, const std::vector<Unit> &units, int u0, 
     ep.coef = coef;
     ep.coef_stride = p;
     ep.part_stride = nmt;
+    // scale pairs of the psi and the lambda matrices (tensor-core products)
+    const float *sc_psi = tcp ? reinterpret_cast<const float *>(c0 + 1) : nullptr;
+    const float *sc_lam = tcp ? sc_psi + 2 : nullptr;
     double useful = 0.0;  // useful flops of one grouped product
     for (int b = 0; b < NB; b++) useful += 2.0 * SL.block_dim[b] * (double)SL.block_dim[b] * 2.0 * S;
     const int fam_g = family(ctx, tcp ? "eig_gemm_tc_3xtf32_blocks" : "eig_gemm_simt_blocks");
     const int fam_o = family(ctx, "orbit_transform");
-    bool map_ok = true;
+    bool map_ok = true, adjoint = false;
     auto lo_of = [&](const float *B) -> const float * { return B == X ? Xl : B == Y ? Yl : B == Lm ? Ll : nullptr; };
     auto gemm = [&](const float *A, const float *B, EigEpiParams q) {
         LaunchRec r;
@@ -1008,6 +1011,7 @@ qaoa_status plan_sym_job(qaoa_ctx *ctx, const std::vector<Unit> &units, int u0, 
                      encode_kmajor_map(&r.tm[2], B, ldp, 2 * Spad) &&
                      encode_kmajor_map(&r.tm[3], lo_of(B), ldp, 2 * Spad);
             q.out_lo = q.out == Y ? Yl : nullptr;  // only Y feeds another product
+            q.sc_in = q.sc_out = adjoint ? sc_lam : sc_psi;
         }
         r.ep = q;
         Lr.push_back(r);
@@ -1033,12 +1037,15 @@ qaoa_status plan_sym_job(qaoa_ctx *ctx, const std::vector<Unit> &units, int u0, 
     oa.coef = coef;
     oa.coef_stride = p;
     oa.part_stride = nob;
-    if (grad) {
+    oa.scale = sc_psi;
+    if (grad || tcp) {
         LaunchRec r;
-        r.kind = LK_COST_MEAN;
+        r.kind = LK_EIG_SCALE;
         r.ep = ep;
+        r.ep.sc_in = sc_psi;
+        r.iinit = u.init;
         r.mean_out = c0;
-        r.fam = family(ctx, "cost_mean");
+        r.fam = family(ctx, "eig_scale");
         Lr.push_back(r);
     }
     {
@@ -1075,12 +1082,14 @@ qaoa_status plan_sym_job(qaoa_ctx *ctx, const std::vector<Unit> &units, int u0, 
             a.round = r;
             a.out = grad ? Lm : nullptr;
             a.out_lo = grad ? Ll : nullptr;
+            a.scale = sc_lam;
             a.c0 = grad ? c0 : nullptr;
             a.part = part;
         }
         orbit(a);
     }
     if (grad) {
+        adjoint = true;
         for (int r = p - 1; r >= 0; r--) {
             EigEpiParams q = ep;
             q.kind = EPI_BWD_EIG;
@@ -1100,6 +1109,7 @@ qaoa_status plan_sym_job(qaoa_ctx *ctx, const std::vector<Unit> &units, int u0, 
             a.in_psi = CKP(r);
             a.out = r > 0 ? Lm : nullptr;
             a.out_lo = r > 0 ? Ll : nullptr;
+            a.scale = sc_lam;
             a.c0 = c0;
             a.part = part + (1 + p + r) * pq;
             orbit(a);
@@ -1852,7 +1862,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                 g.part_off = part_bytes;
                 part_bytes += align_up(sizeof(double) * (1 + 2 * u.p) * g.Spad * std::max(g.nmt, g.nob));
                 g.c0_off = part_bytes;  // the job's cost mean (shift of the adjoint)
-                part_bytes += align_up(sizeof(double));
+                part_bytes += align_up(sizeof(double) + 4 * sizeof(float));  // then the operand scales
                 eg.push_back(g);
                 i = j;
             }
@@ -1930,6 +1940,11 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                     const float *lam_hi = static_cast<const float *>(dL), *lam_lo = lam_hi + ld;
                     const size_t mat = (size_t)2 * g.Spad * ld;
                     float *base = reinterpret_cast<float *>(static_cast<char *>(d_est) + g.st_off);
+                    // padding entries are never written: clear the operand planes once per plan (a stale
+                    // half could be an infinity, which zero padding of V does not cancel)
+                    if (tcp)
+                        QG_CUDA(ctx, cudaMemsetAsync(base, 0, mat * (grad ? 6 + 2 * p : 4) * sizeof(float), ctx->stream),
+                                "state clear");
                     float *X = base, *Y = base + mat, *Lm = grad ? base + 2 * mat : nullptr;
                     auto CKX = [&](int k) { return base + (3 + k) * mat; };
                     auto CKY = [&](int k) { return base + (3 + p + k) * mat; };
@@ -1955,12 +1970,18 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                     ep.part_stride = g.nmt;
                     double *c0 = reinterpret_cast<double *>(static_cast<char *>(d_epart) + g.c0_off);
                     ep.c0 = grad ? c0 : nullptr;
-                    if (grad) {
+                    // scale pairs of the psi and the lambda matrices (tensor-core products)
+                    const float *sc_psi = tcp ? reinterpret_cast<const float *>(c0 + 1) : nullptr;
+                    const float *sc_lam = tcp ? sc_psi + 2 : nullptr;
+                    bool adjoint = false;
+                    if (grad || tcp) {
                         LaunchRec r;
-                        r.kind = LK_COST_MEAN;
+                        r.kind = LK_EIG_SCALE;
                         r.ep = ep;
+                        r.ep.sc_in = sc_psi;
+                        r.iinit = u.init;
                         r.mean_out = c0;
-                        r.fam = family(ctx, "cost_mean");
+                        r.fam = family(ctx, "eig_scale");
                         L.push_back(r);
                     }
                     const double gflops = 2.0 * D * (double)D * 2.0 * g.S;
@@ -1992,6 +2013,8 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                             q.out_lo = q.out == X ? Xl : q.out == Y ? Yl : q.out == Lm ? Ll : nullptr;
                             q.out2_lo = q.out2 == Lm ? Ll : nullptr;
                             if (q.kind == EPI_FWD_LAST) q.out_lo = nullptr;  // psi_p is not a product operand
+                            q.sc_in = q.sc_out = adjoint ? sc_lam : sc_psi;
+                            q.sc_out2 = sc_lam;
                         }
                         r.ep = q;
                         L.push_back(r);
@@ -2002,6 +2025,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         r.ep = ep;
                         r.iX = X;
                         r.iX_lo = Xl;
+                        r.ep.sc_in = sc_psi;
                         r.ick0 = grad ? CKX(0) : nullptr;
                         r.iinit = u.init;
                         r.iamp0 = (float)(1.0 / std::sqrt((double)D));
@@ -2024,13 +2048,14 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         } else {
                             q.kind = EPI_FWD_LAST;
                             q.round = k;
-                            q.out = grad ? X : nullptr;
+                            q.out = nullptr;  // psi_p itself is not needed again
                             q.out2 = Lm;
                             q.part = part;
                         }
                         gemm(Vp, Y, q);
                     }
                     if (grad) {
+                        adjoint = true;
                         for (int k = p - 1; k >= 0; k--) {
                             EigEpiParams q = ep;
                             q.kind = EPI_BWD_EIG;
@@ -2182,7 +2207,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             break;
         case LK_EIG_INIT:
             e = launch_eig_init(r.iX, r.iX_lo, r.ick0, r.ep.M, r.ep.ld, r.ep.nsets, r.ep.cost, r.ep.cost_dtype,
-                                r.ep.coef, r.ep.coef_stride, r.iinit, r.iamp0, ctx->stream);
+                                r.ep.coef, r.ep.coef_stride, r.iinit, r.iamp0, r.ep.sc_in, ctx->stream);
             break;
         case LK_EIG_GEMM:
             if (r.grouped)
@@ -2211,8 +2236,9 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                                 reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles, r.r1in, r.r1half,
                                 ctx->stream);
             break;
-        case LK_COST_MEAN:
-            e = launch_cost_mean(r.ep.cost, r.ep.cost_dtype, r.ep.M, r.mean_out, ctx->stream);
+        case LK_EIG_SCALE:
+            e = launch_eig_scale(r.ep.cost, r.ep.cost_dtype, r.ep.M, r.iinit, r.mean_out,
+                                 const_cast<float *>(r.ep.sc_in), ctx->stream);
             break;
         case LK_REDUCE:
             e = launch_reduce(reinterpret_cast<const RedChunk *>(db + r.desc_off), r.ndesc,
