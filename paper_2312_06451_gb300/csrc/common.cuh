@@ -276,6 +276,12 @@ __device__ __forceinline__ void chain_begin() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
+// Launches that depend on nothing a neighbour does (the on-chip and grid kernels
+// of one call, a launch per size class) run side by side: each calls
+// beside_begin, so that the next may start at once, and beside_end before it
+// exits, so that its completion still implies that of all before it.
+__device__ __forceinline__ void beside_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void beside_end() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <typename... P, typename... A>
 cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...args) {
     cudaLaunchConfig_t c = {};
@@ -385,8 +391,10 @@ int small_max_n();
 // table.  onchip_class: the launch class of an instance (the units of a launch
 // share one), 0 when n is out of range.
 int onchip_class(int n);
+// beside: the launch before this one on the stream is of this kind too (see
+// beside_begin); the same for launch_grid.
 cudaError_t launch_onchip(const SmallDesc *d_descs, int ndesc, int cls, int cost_dtype, int want_grad, int *d_err,
-                          cudaStream_t s);
+                          bool beside, cudaStream_t s);
 // 13 <= n <= kGridMaxN, transverse field: every round of an angle set in one
 // launch, 2^(n-12) CTAs a set (kernels_grid.cu).
 constexpr int kGridMaxN = 20;
@@ -410,7 +418,7 @@ constexpr int kGridClusterN = 16;  // up to here a set is one cluster (any numbe
 int grid_max_ctas(int cost_dtype, int want_grad, int n);
 // The descriptors of a launch have one n up to kGridClusterN (then: any sizes above).
 cudaError_t launch_grid(const GridDesc *d_descs, const uint32_t *d_begin, int nd, uint32_t ctas, int cost_dtype,
-                        int want_grad, int n, int *d_err, cudaStream_t s);
+                        int want_grad, int n, int *d_err, bool beside, cudaStream_t s);
 // Diagnostic: a bounded wait on a barrier nothing completes (sets DERR_TIMEOUT).
 cudaError_t launch_wait_probe(int *d_err, cudaStream_t s);
 

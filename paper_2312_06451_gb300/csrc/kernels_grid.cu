@@ -93,6 +93,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
     __shared__ double s_E;
     __shared__ int s_fail, s_top;
     __shared__ GridDesc D;
+    beside_begin();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int di = grid_desc(begin, nd, blockIdx.x);
     for (int i = tid; i < (int)(sizeof(GridDesc) / 4); i += kNT)
@@ -215,6 +216,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
         }
         if (!set_wait<HI>(D.bar, target += ncta, &s_fail)) {
             if (tid == 0) atomicOr(err, DERR_TIMEOUT);
+            beside_end();
             return;
         }
         load_from(X, g ^ 1, true, a);
@@ -250,6 +252,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
     set_arrive<HI>(D.bar);
     if (!set_wait<HI>(D.bar, target += ncta, &s_fail)) {
         if (tid == 0) atomicOr(err, DERR_TIMEOUT);
+        beside_end();
         return;
     }
     // sum over the set's CTAs of quantity q (warp-wide, a fixed order)
@@ -313,6 +316,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
             load_table(k, C);
             if (!set_wait<HI>(D.bar, target += ncta, &s_fail)) {
                 if (tid == 0) atomicOr(err, DERR_TIMEOUT);
+                beside_end();
                 return;
             }
             if (k < p - 1) flush(k + 1);
@@ -335,6 +339,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
         set_arrive<HI>(D.bar);
         if (!set_wait<HI>(D.bar, target += ncta, &s_fail)) {
             if (tid == 0) atomicOr(err, DERR_TIMEOUT);
+            beside_end();
             return;
         }
         // the set's derivatives: output o by warp o of the set
@@ -343,6 +348,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
             if (lane == 0) D.grad_out[o] = 2.0 * s;
         }
     }
+    beside_end();
 }
 
 template <int COST, int GRAD, int HI>
@@ -361,21 +367,27 @@ struct GridLaunch {
         if (e == cudaSuccess) __atomic_store_n(&wide_done[dev], 1, __ATOMIC_RELEASE);
         return e;
     }
-    static void config(cudaLaunchConfig_t &c, cudaLaunchAttribute &at, uint32_t ctas, int n, cudaStream_t s) {
+    static void config(cudaLaunchConfig_t &c, cudaLaunchAttribute (&at)[2], uint32_t ctas, int n, bool beside,
+                       cudaStream_t s) {
         c = {};
         c.gridDim = dim3(ctas);
         c.blockDim = dim3(kNT);
         c.dynamicSmemBytes = smem;
         c.stream = s;
-        c.attrs = &at;
+        c.attrs = at;
         c.numAttrs = 1;
-        if (HI) {
-            at.id = cudaLaunchAttributeCooperative;
-            at.val.cooperative = 1;
-        } else {
-            at.id = cudaLaunchAttributeClusterDimension;
-            at.val.clusterDim.x = 1u << (n - kNB);
-            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        if (HI) {  // (cooperative launches stay in stream order)
+            at[0].id = cudaLaunchAttributeCooperative;
+            at[0].val.cooperative = 1;
+            return;
+        }
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = 1u << (n - kNB);
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        if (beside) {
+            at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[1].val.programmaticStreamSerializationAllowed = 1;
+            c.numAttrs = 2;
         }
     }
     static int room(int n) {
@@ -392,8 +404,8 @@ struct GridLaunch {
             return nsm * per;
         }
         cudaLaunchConfig_t c;
-        cudaLaunchAttribute at;
-        config(c, at, 1u << (n - kNB), n, nullptr);
+        cudaLaunchAttribute at[2];
+        config(c, at, 1u << (n - kNB), n, false, nullptr);
         if (cudaOccupancyMaxActiveClusters(&per, kern, &c) != cudaSuccess) {
             cudaGetLastError();
             per = 0;
@@ -401,12 +413,12 @@ struct GridLaunch {
         return per << (n - kNB);
     }
     static cudaError_t go(const GridDesc *d, const uint32_t *begin, int nd, uint32_t ctas, int n, int *err,
-                          cudaStream_t s) {
+                          bool beside, cudaStream_t s) {
         cudaError_t e = attrs();
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t c;
-        cudaLaunchAttribute at;
-        config(c, at, ctas, n, s);
+        cudaLaunchAttribute at[2];
+        config(c, at, ctas, n, beside, s);
         return cudaLaunchKernelEx(&c, kern, d, begin, nd, err);
     }
 };
@@ -432,9 +444,9 @@ int grid_max_ctas(int cost_dtype, int want_grad, int n) {
 }
 
 cudaError_t launch_grid(const GridDesc *d, const uint32_t *begin, int nd, uint32_t ctas, int cost_dtype,
-                        int want_grad, int n, int *err, cudaStream_t s) {
+                        int want_grad, int n, int *err, bool beside, cudaStream_t s) {
     return grid_pick(cost_dtype, want_grad, n > kGridClusterN,
-                     [&](auto g) { return decltype(g)::go(d, begin, nd, ctas, n, err, s); });
+                     [&](auto g) { return decltype(g)::go(d, begin, nd, ctas, n, err, beside, s); });
 }
 
 }  // namespace qg

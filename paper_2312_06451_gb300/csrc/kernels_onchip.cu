@@ -36,6 +36,7 @@ __global__ void __launch_bounds__(Chip<NB>::NT) onchip_kernel(const SmallDesc *_
     __shared__ float2 stab[kPhaseTable];
     __shared__ double s_red[2][2][NW];  // [round parity][beta, gamma][warp]
     __shared__ int s_top;               // largest uint8 cost
+    beside_begin();
     const SmallDesc D = descs[blockIdx.x];
     const int p = D.p, n = D.n, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const double *ang = D.angles_beta;
@@ -182,15 +183,18 @@ __global__ void __launch_bounds__(Chip<NB>::NT) onchip_kernel(const SmallDesc *_
         __syncthreads();
         flush(0);
     }
+    beside_end();
 }
 
 template <int NB>
-cudaError_t go_onchip(const SmallDesc *d, int nd, int cost_dtype, int want_grad, int *err, cudaStream_t s) {
+cudaError_t go_onchip(const SmallDesc *d, int nd, int cost_dtype, int want_grad, int *err, bool beside,
+                      cudaStream_t s) {
     const size_t smem = (size_t)Chip<NB>::N * ((want_grad ? 16 : 8) + (cost_dtype == 0 ? 4 : 1));
     auto go = [&](auto kern, int slot) -> cudaError_t {
         static int attr_done[4][kMaxDevices];
         cudaError_t e = smem_attr_once(kern, (int)smem, attr_done[slot]);
         if (e != cudaSuccess) return e;
+        if (beside) return launch_chained(kern, nd, Chip<NB>::NT, smem, s, d, err);
         kern<<<nd, Chip<NB>::NT, smem, s>>>(d, err);
         return cudaGetLastError();
     };
@@ -203,12 +207,12 @@ cudaError_t go_onchip(const SmallDesc *d, int nd, int cost_dtype, int want_grad,
 int onchip_class(int n) { return n < 1 || n > kPassTileBits ? 0 : (n < 9 ? 9 : n); }
 
 cudaError_t launch_onchip(const SmallDesc *d, int nd, int cls, int cost_dtype, int want_grad, int *err,
-                          cudaStream_t s) {
+                          bool beside, cudaStream_t s) {
     switch (cls) {
-    case 9: return go_onchip<9>(d, nd, cost_dtype, want_grad, err, s);
-    case 10: return go_onchip<10>(d, nd, cost_dtype, want_grad, err, s);
-    case 11: return go_onchip<11>(d, nd, cost_dtype, want_grad, err, s);
-    case 12: return go_onchip<12>(d, nd, cost_dtype, want_grad, err, s);
+    case 9: return go_onchip<9>(d, nd, cost_dtype, want_grad, err, beside, s);
+    case 10: return go_onchip<10>(d, nd, cost_dtype, want_grad, err, beside, s);
+    case 11: return go_onchip<11>(d, nd, cost_dtype, want_grad, err, beside, s);
+    case 12: return go_onchip<12>(d, nd, cost_dtype, want_grad, err, beside, s);
     default: return cudaErrorInvalidValue;
     }
 }

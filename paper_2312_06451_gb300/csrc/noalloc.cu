@@ -87,7 +87,7 @@ extern "C" qaoa_status qaoa_gradient_small_noalloc(const void *d_cost, int cost_
     if (cudaMemsetAsync(d_err, 0, sizeof(int), s) != cudaSuccess ||
         cudaMemcpyAsync(base + kOffSmall, &sd, sizeof(sd), cudaMemcpyHostToDevice, s) != cudaSuccess ||
         qg::launch_onchip(reinterpret_cast<const qg::SmallDesc *>(base + kOffSmall), 1, qg::onchip_class(n), cost_dtype,
-                          d_grad ? 1 : 0, d_err, s) != cudaSuccess ||
+                          d_grad ? 1 : 0, d_err, false, s) != cudaSuccess ||
         cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) {
         cudaGetLastError();

@@ -1426,7 +1426,8 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             if ((st = scratch(ctx, "gridstate", gp.bytes, &d_gs))) return st;
             if ((st = scratch(ctx, "gridbar", sizeof(unsigned) * gp.n_bar, &d_bar))) return st;
             for (int lw = 0; lw < 2 * kGridClasses * kGridWaves; lw++) {
-                const int dt = lw & 1, wave = (lw >> 1) % kGridWaves, gc = (lw >> 1) / kGridWaves;
+                // the cooperative launches first: the clusters fill what their last one leaves
+                const int dt = lw & 1, wave = (lw >> 1) % kGridWaves, gc = kGridClasses - 1 - (lw >> 1) / kGridWaves;
                 std::vector<GridDesc> gd;
                 std::vector<uint32_t> begin(1, 0);
                 double bytes = 0;
@@ -2172,6 +2173,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         QG_CUDA(ctx, cudaMemsetAsync(d_split_cnt, 0, eig_split_cnt_bytes(), ctx->stream), "split counters clear");
     }
     const bool prof = ctx->profiling && !capturing(ctx);
+    bool beside = false;  // the launch before was an on-chip or grid one: the next of them runs beside it
     for (const LaunchRec &r : ctx->plan.launches) {
         NvtxRange nvtx_launch(r.fam >= 0 && r.fam < (int)ctx->fam_names.size() ? ctx->fam_names[r.fam].c_str()
                                                                               : "qaoa_launch");
@@ -2190,7 +2192,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         case LK_SMALL:
             if (r.chip_cls)
                 e = launch_onchip(reinterpret_cast<const SmallDesc *>(db + r.desc_off), r.ndesc, r.chip_cls,
-                                  r.cost_dtype, r.small_grad, ctx->d_err, ctx->stream);
+                                  r.cost_dtype, r.small_grad, ctx->d_err, beside, ctx->stream);
             else
                 e = launch_small(reinterpret_cast<const SmallDesc *>(db + r.desc_off), r.ndesc, r.cost_dtype,
                                  r.small_grad, r.small_maxn, ctx->d_err, ctx->stream);
@@ -2198,7 +2200,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         case LK_GRID:
             e = launch_grid(reinterpret_cast<const GridDesc *>(db + r.desc_off),
                             reinterpret_cast<const uint32_t *>(db + r.tb_off), r.ndesc, r.tiles, r.cost_dtype,
-                            r.small_grad, r.gn, ctx->d_err, ctx->stream);
+                            r.small_grad, r.gn, ctx->d_err, beside, ctx->stream);
             break;
         case LK_XPASS:
             e = launch_xpass(r.bwd, r.cost_dtype, r.nbuf, r.var, reinterpret_cast<const PassDesc *>(db + r.desc_off),
@@ -2248,6 +2250,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         }
         if (e != cudaSuccess) return cuda_fail(ctx, e, "kernel launch");
         ctx->launches++;
+        beside = r.kind == LK_GRID || (r.kind == LK_SMALL && r.chip_cls);
         if (prof) {
             cudaEventRecord(eb, ctx->stream);
             ctx->pending.push_back({r.fam, ea, eb});
