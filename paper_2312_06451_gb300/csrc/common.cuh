@@ -494,6 +494,11 @@ int degeneracy_sliced_kk(const DegLaunch &L);
 // colex ranks [t_start, t_start + t_count).
 cudaError_t launch_degeneracy_sliced(const DegLaunch &L, const uint64_t *d_binom, uint64_t t_start,
                                      uint64_t t_count, unsigned long long *d_counts, int *d_err, cudaStream_t s);
+// The whole count for enumerated sets of kDegRunsMin..8, through a task counter
+// *d_next (zero when the launch starts).
+constexpr int kDegRunsMin = 5;
+cudaError_t launch_degeneracy_runs(const DegLaunch &L, const uint64_t *d_binom, unsigned long long *d_counts,
+                                   unsigned long long *d_next, int *d_err, cudaStream_t s);
 cudaError_t launch_degeneracy(const DegLaunch &L, const uint64_t *d_binom, uint64_t start, uint64_t count,
                               unsigned long long *d_counts, int *d_err, cudaStream_t s);
 cudaError_t launch_grover_eval(const int64_t *d_counts, int nb, int p, int n_sets, const double *d_angles,

@@ -32,6 +32,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 namespace qg {
 namespace {
@@ -224,7 +225,7 @@ degeneracy_kernel(const DegParams P, const uint64_t *__restrict__ binom, uint64_
 // ------------------------------------------------- bit-sliced weight-k count
 // Weight-k problems whose cost is a function of I = |edges inside y| alone
 // (densest k-subgraph with y = x, k-vertex cover with y = the complement),
-// |y| = KK in 2..8.  The sets y = {v} u T with v < min(T) are counted per
+// |y| = KK in 2..8 (many sets of 5 and more: the next section).  The sets y = {v} u T with v < min(T) are counted per
 // (KK-1)-set T at once: I = inside(T) + a(v) with a(v) = |N(v) & T|, and
 // a(v) for all 128 vertices is the bitwise sum of the neighbour masks of T's
 // members, held as three bit planes (a <= 7).  The histogram of a over
@@ -424,6 +425,208 @@ degeneracy_sliced_kernel(const DegParams P, const uint64_t *__restrict__ binom, 
     }
 }
 
+// ------------------------------------- bit-sliced count by runs, set size 5..8
+// The same sets y = {v, w} u T2, v < w < a = min(T2), counted per (KK-2)-set T2
+// instead of per T.  With x(v) = |N(v) & T2| in 0..KK-2 and its class masks C_j,
+//     I(y) = inside(T2) + x(v) + x(w) + [v adjacent to w],
+// so the histogram over all pairs follows from the class sizes below a (products,
+// once per T2) and only adjacent pairs have to be looked at:
+//     E[i + j] += |N(w) & C_j & {v < w}| for every w of class i,
+//     H[inside + s] += pairs[s] - E[s] + E[s - 1].
+// That takes KK - 2 masked popcounts a step (w, T2) -- of one 32-bit word while
+// w < 32 -- where counting per T takes KK - 1 of two, besides forming T's planes.
+//
+// A warp's lanes take 32 sets U of T2 = {a, b} u U with one b, and sweep a and w
+// together, so every lane is at the same step (threads that walked T in order
+// met their changes of T2 at different times, and with 32 lanes some lane met one
+// at nearly every step), rows of the adjacency are read once a warp, and a step
+// adds its KK - 1 counts, 16 bits each, to the class of w in shared memory with
+// one 16-byte read and write.  Tasks (b, 32 sets U, a range of a of about
+// kRunSteps steps) are claimed from a counter.
+// The instruction rate bounds it.  C(100, 6) sets and 1024 reduced gradients, a
+// call: 654 -> 271 us.
+constexpr int kRunSteps = 256;
+struct RunPlan {
+    uint64_t first[129];    // first task of b (first[n] = number of tasks)
+    uint32_t pieces[128];   // ranges of a for b
+};
+
+template <int KK>
+struct RunGeom {
+    static constexpr int kNb = KK * (KK - 1) / 2 + 1;  // I = 0 .. C(KK, 2)
+    static constexpr int kNC = KK - 1;                 // classes 0 .. KK - 2
+    static constexpr size_t smem = (size_t)kDegThreads * (kNC * 16 + kNb * 4);
+};
+
+template <int KK>
+__global__ void __launch_bounds__(kDegThreads)
+degeneracy_runs_kernel(const __grid_constant__ DegParams P, const __grid_constant__ RunPlan R,
+                       const uint64_t *__restrict__ binom, int n_bins, unsigned long long *__restrict__ counts,
+                       unsigned long long *next, int *err) {
+    using G = RunGeom<KK>;
+    constexpr int kNC = G::kNC, kNb = G::kNb, kU = KK - 4;
+    extern __shared__ __align__(16) unsigned char rsm[];
+    uint4 *acc = reinterpret_cast<uint4 *>(rsm) + threadIdx.x;                              // [class][thread]
+    uint32_t *h = reinterpret_cast<uint32_t *>(rsm + (size_t)kNC * kDegThreads * 16) + threadIdx.x;  // [I][thread]
+    __shared__ uint4 s_low[128];       // neighbours below w
+    __shared__ int s_deg[128];         // how many
+    __shared__ ulonglong2 s_up[128];   // all neighbours
+    const int tid = threadIdx.x, lane = tid & 31, n = P.n;
+    for (int w = tid; w < 128; w += kDegThreads) {
+        const uint64_t lo = P.up_lo[w], hi = P.up_hi[w];
+        s_up[w] = make_ulonglong2(lo, hi);
+        const uint64_t ml = lo & (w < 64 ? (1ull << w) - 1ull : ~0ull), mh = hi & (w < 64 ? 0ull : (1ull << (w - 64)) - 1ull);
+        s_low[w] = make_uint4((uint32_t)ml, (uint32_t)(ml >> 32), (uint32_t)mh, (uint32_t)(mh >> 32));
+        s_deg[w] = __popcll(ml) + __popcll(mh);
+    }
+    for (int i = 0; i < kNb; i++) h[i * kDegThreads] = 0u;
+    for (int i = 0; i < kNC; i++) acc[i * kDegThreads] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    uint64_t bound = 0;  // no counter of this thread exceeds it
+    auto flush = [&]() {
+        for (int I = 0; I < kNb; I++) {
+            unsigned long long s = h[I * kDegThreads];
+            h[I * kDegThreads] = 0u;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0 && s) {
+                const int cost = P.kind == 1 ? I : P.m - I;
+                if ((unsigned)cost < (unsigned)n_bins) atomicAdd(&counts[cost], s);
+                else atomicOr(err, DERR_BAD_DESC);
+            }
+        }
+        bound = 0;
+    };
+    for (;;) {
+        unsigned long long task = 0;
+        if (lane == 0) task = atomicAdd(next, 1ull);
+        task = __shfl_sync(0xffffffffu, task, 0);
+        if (task >= R.first[n]) break;
+        int b = 0;  // the last b with first[b] <= task
+        for (int step = 64; step > 0; step >>= 1)
+            if (b + step < n && R.first[b + step] <= task) b += step;
+        const uint32_t pieces = R.pieces[b];
+        const uint64_t rem = task - R.first[b], chunk = rem / pieces;
+        const uint32_t piece = (uint32_t)(rem - chunk * pieces);
+        // U: the (KK-4)-set of {b+1, ..} of rank 32 chunk + lane (colex)
+        const uint64_t u = chunk * 32 + lane;
+        const bool valid = u < binom[(n - 1 - b) * 129 + kU];
+        uint64_t r = valid ? u : 0ull;
+        Planes B;
+        B.b0l = s_up[b].x;
+        B.b0h = s_up[b].y;
+        B.b1l = B.b1h = B.b2l = B.b2h = 0ull;
+        Set2 T3 = {b < 64 ? 1ull << b : 0ull, b < 64 ? 0ull : 1ull << (b - 64)};
+        int tin3 = 0;
+        {
+            int c = n - 2 - b;
+#pragma unroll
+            for (int i = kU; i >= 1; i--) {
+                while (binom[c * 129 + i] > r) c--;
+                r -= binom[c * 129 + i];
+                const int x = b + 1 + c;
+                c--;
+                const ulonglong2 m = s_up[x];
+                tin3 += __popcll(m.x & T3.lo) + __popcll(m.y & T3.hi);
+                B = planes_add(B, m.x, m.y);
+                if (x < 64) T3.lo |= 1ull << x;
+                else T3.hi |= 1ull << (x - 64);
+            }
+        }
+        // a from 1 to b - 1 in ranges of about equally many steps (a(a-1)/2 below a)
+        auto cut = [&](uint32_t j) -> int {
+            if (j == 0) return 1;
+            if (j >= pieces) return b;
+            const float x = 0.5f * (float)(b * (b - 1)) * ((float)j / (float)pieces);
+            return max(1, min(b, (int)ceilf(0.5f * (1.f + sqrtf(1.f + 8.f * x)))));
+        };
+        const int a1 = cut(piece + 1);
+        for (int a = cut(piece); a < a1; a++) {
+            const ulonglong2 ma = s_up[a];
+            const Planes B2 = planes_add(B, ma.x, ma.y);
+            auto bit = [&](uint64_t lo, uint64_t hi) -> int { return (int)((a < 64 ? lo >> a : hi >> (a - 64)) & 1ull); };
+            const int tin2 = tin3 + bit(B.b0l, B.b0h) + 2 * bit(B.b1l, B.b1h) + 4 * bit(B.b2l, B.b2h);
+            const uint32_t x0[4] = {(uint32_t)B2.b0l, (uint32_t)(B2.b0l >> 32), (uint32_t)B2.b0h, (uint32_t)(B2.b0h >> 32)};
+            const uint32_t x1[4] = {(uint32_t)B2.b1l, (uint32_t)(B2.b1l >> 32), (uint32_t)B2.b1h, (uint32_t)(B2.b1h >> 32)};
+            const uint32_t x2[4] = {(uint32_t)B2.b2l, (uint32_t)(B2.b2l >> 32), (uint32_t)B2.b2h, (uint32_t)(B2.b2h >> 32)};
+            uint32_t C[kNC][4];  // class masks (1 .. KK - 2)
+#pragma unroll
+            for (int j = 1; j < kNC; j++)
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    C[j][q] = ((j & 1) ? x0[q] : ~x0[q]) & ((j & 2) ? x1[q] : ~x1[q]) & ((j & 4) ? x2[q] : ~x2[q]);
+            // steps w of words 0 .. NW - 1 (the neighbours below w lie there)
+            auto sweep = [&](auto nw_tag) {
+                constexpr int NW = decltype(nw_tag)::value, q0 = NW - 1;
+                uint32_t r0 = x0[q0], r1 = x1[q0], r2 = x2[q0];  // w's class in bit 0
+                const int w1 = min(a, 32 * NW);
+                for (int w = 32 * q0; w < w1; w++) {
+                    const uint4 row4 = s_low[w];
+                    const uint32_t row[4] = {row4.x, row4.y, row4.z, row4.w};
+                    uint32_t e[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u}, sum = 0;
+#pragma unroll
+                    for (int j = 1; j < kNC; j++) {
+#pragma unroll
+                        for (int q = 0; q < NW; q++) e[j] += __popc(row[q] & C[j][q]);
+                        sum += e[j];
+                    }
+                    e[0] = (uint32_t)s_deg[w] - sum;
+                    const uint32_t cls = (r0 & 1u) | ((r1 & 1u) << 1) | ((r2 & 1u) << 2);
+                    r0 >>= 1;
+                    r1 >>= 1;
+                    r2 >>= 1;
+                    uint4 *p = acc + cls * kDegThreads;
+                    uint4 v = *p;
+                    v.x += e[0] + (e[1] << 16);
+                    v.y += e[2] + (e[3] << 16);
+                    if (kNC > 4) v.z += e[4] + (e[5] << 16);
+                    if (kNC > 6) v.w += e[6];
+                    *p = v;
+                }
+            };
+            sweep(std::integral_constant<int, 1>());
+            if (a > 32) sweep(std::integral_constant<int, 2>());
+            if (a > 64) sweep(std::integral_constant<int, 3>());
+            if (a > 96) sweep(std::integral_constant<int, 4>());
+            // all pairs below a by their classes, adjacent ones moved up by one
+            int nj[kNC], E[2 * kNC], H[2 * kNC];
+            nj[0] = a;
+#pragma unroll
+            for (int j = 1; j < kNC; j++) {
+                nj[j] = 0;
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    const int left = a - 32 * q;
+                    const uint32_t m = left >= 32 ? 0xffffffffu : left > 0 ? (1u << left) - 1u : 0u;
+                    nj[j] += __popc(C[j][q] & m);
+                }
+                nj[0] -= nj[j];
+            }
+#pragma unroll
+            for (int s = 0; s < 2 * kNC; s++) E[s] = H[s] = 0;
+#pragma unroll
+            for (int i = 0; i < kNC; i++) {
+                H[2 * i] += nj[i] * (nj[i] - 1) / 2;
+#pragma unroll
+                for (int j = i + 1; j < kNC; j++) H[i + j] += nj[i] * nj[j];
+                const uint4 v = acc[i * kDegThreads];
+                acc[i * kDegThreads] = make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int j = 0; j < kNC; j++) E[i + j] += (int)((j & 1) ? vw[j >> 1] >> 16 : vw[j >> 1] & 0xffffu);
+            }
+            if (valid) {
+#pragma unroll
+                for (int s = 0; s < 2 * kNC; s++)
+                    if (s < 2 * kNC) h[(tin2 + s) * kDegThreads] += (uint32_t)(H[s] - E[s] + (s ? E[s - 1] : 0));
+            }
+            bound += (uint64_t)(a * (a - 1) / 2);
+        }
+        if (bound > (1ull << 31)) flush();
+    }
+    flush();
+}
+
 // ------------------------------------------------------- reduced simulation
 // One CTA per angle set, as many threads as values (a warp at least, 512 at
 // most).  Float64 runs at a small fraction of the float32 rate here, so the
@@ -460,10 +663,11 @@ __device__ __forceinline__ double2 cmuld(double2 a, double2 b) {
 
 __global__ void __launch_bounds__(kGrMaxThreads)
 grover_eval_kernel(const int64_t *__restrict__ counts, int nb, int p, const double *__restrict__ angles,
-                   double *__restrict__ E, double *__restrict__ grad) {
+                   double *__restrict__ E, double *__restrict__ grad, int keep) {
     extern __shared__ double2 gsm[];
     double2 *psi = gsm, *lam = gsm + nb, *red = gsm + 2 * nb, *trig = red + kGrMaxWarps;
-    double *u = reinterpret_cast<double *>(trig + p);
+    double2 *tab = trig + p;  // keep: (cos, sin)(gamma_k j) of every round and value
+    double *u = reinterpret_cast<double *>(tab + (keep ? p * nb : 0));
     const int set = blockIdx.x;
     const double *a = angles + (size_t)set * 2 * p;
     // N = sum of the degeneracies (exact in float64 below 2^53)
@@ -479,14 +683,24 @@ grover_eval_kernel(const int64_t *__restrict__ counts, int nb, int p, const doub
         sincos(a[k], &sb, &cb);
         trig[k] = make_double2(cb, sb);
     }
+    if (keep)
+        for (int e = threadIdx.x; e < p * nb; e += blockDim.x) {
+            double sn, cs;
+            sincos(a[p + e / nb] * (double)(e % nb), &sn, &cs);
+            tab[e] = make_double2(cs, sn);
+        }
     __syncthreads();
+    auto phase = [&](int k, int j) -> double2 {
+        if (keep) return tab[k * nb + j];
+        double sn, cs;
+        sincos(a[p + k] * (double)j, &sn, &cs);
+        return make_double2(cs, sn);
+    };
     for (int k = 0; k < p; k++) {
-        const double g = a[p + k];
         double2 s = make_double2(0.0, 0.0);
         for (int j = threadIdx.x; j < nb; j += blockDim.x) {
-            double sn, cs;
-            sincos(g * (double)j, &sn, &cs);
-            psi[j] = cmuld(psi[j], make_double2(cs, -sn));
+            const double2 ph = phase(k, j);
+            psi[j] = cmuld(psi[j], make_double2(ph.x, -ph.y));
             s.x += u[j] * psi[j].x;
             s.y += u[j] * psi[j].y;
         }
@@ -505,7 +719,6 @@ grover_eval_kernel(const int64_t *__restrict__ counts, int nb, int p, const doub
     double *g_out = grad + (size_t)set * 2 * p;
     for (int j = threadIdx.x; j < nb; j += blockDim.x) lam[j] = make_double2((double)j * psi[j].x, (double)j * psi[j].y);
     for (int k = p - 1; k >= 0; k--) {
-        const double g = a[p + k];
         double2 sl = make_double2(0.0, 0.0), sp = make_double2(0.0, 0.0);
         for (int j = threadIdx.x; j < nb; j += blockDim.x) {
             sl.x += u[j] * lam[j].x;
@@ -527,9 +740,7 @@ grover_eval_kernel(const int64_t *__restrict__ counts, int nb, int p, const doub
             psi[j].y += dp.y * u[j];
             // Im( conj(lam_j) c_j psi_j )
             gg.x += (double)j * (lam[j].x * psi[j].y - lam[j].y * psi[j].x);
-            double sn, cs;
-            sincos(g * (double)j, &sn, &cs);
-            const double2 ph = make_double2(cs, sn);
+            const double2 ph = phase(k, j);
             lam[j] = cmuld(lam[j], ph);
             psi[j] = cmuld(psi[j], ph);
         }
@@ -601,6 +812,51 @@ cudaError_t launch_degeneracy_sliced(const DegLaunch &L, const uint64_t *d_binom
     }
 }
 
+template <int KK>
+static cudaError_t go_runs(const DegParams &P, const RunPlan &R, const uint64_t *d_binom, int n_bins,
+                           unsigned long long *d_counts, unsigned long long *d_next, int *d_err, cudaStream_t s) {
+    static int attr_done[kMaxDevices];
+    cudaError_t e = smem_attr_once(degeneracy_runs_kernel<KK>, (int)RunGeom<KK>::smem, attr_done);
+    if (e != cudaSuccess) return e;
+    int dev = 0, nsm = 0, occ = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, degeneracy_runs_kernel<KK>, kDegThreads, RunGeom<KK>::smem);
+    if (e != cudaSuccess) return e;
+    const uint64_t want = (R.first[P.n] + kDegWarps - 1) / kDegWarps;
+    const unsigned grid = (unsigned)std::max<uint64_t>(1, std::min<uint64_t>(want, (uint64_t)nsm * std::max(1, occ)));
+    degeneracy_runs_kernel<KK><<<grid, kDegThreads, RunGeom<KK>::smem, s>>>(P, R, d_binom, n_bins, d_counts, d_next,
+                                                                           d_err);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_degeneracy_runs(const DegLaunch &L, const uint64_t *d_binom, unsigned long long *d_counts,
+                                   unsigned long long *d_next, int *d_err, cudaStream_t s) {
+    const int kk = degeneracy_sliced_kk(L), n = L.n;
+    if (kk < kDegRunsMin) return cudaErrorInvalidValue;
+    RunPlan R;
+    uint64_t total = 0;
+    for (int b = 0; b < 128; b++) {
+        R.first[b] = total;
+        const uint64_t steps = (uint64_t)b * (b > 0 ? b - 1 : 0) / 2;
+        R.pieces[b] = (uint32_t)std::max<uint64_t>(1, (steps + kRunSteps - 1) / kRunSteps);
+        // U: (kk-4)-sets of the n - 1 - b vertices above b; v < w < a < b need b >= 3
+        uint64_t nu = 1;
+        for (int i = 0; i < kk - 4; i++) nu = nu * (uint64_t)std::max(0, n - 1 - b - i) / (uint64_t)(i + 1);
+        if (b < n && b >= 3) total += (nu + 31) / 32 * R.pieces[b];
+    }
+    R.first[128] = total;
+    for (int b = n; b < 128; b++) R.first[b] = total;
+    const DegParams P = deg_params(L);
+    switch (kk) {
+    case 5: return go_runs<5>(P, R, d_binom, L.n_bins, d_counts, d_next, d_err, s);
+    case 6: return go_runs<6>(P, R, d_binom, L.n_bins, d_counts, d_next, d_err, s);
+    case 7: return go_runs<7>(P, R, d_binom, L.n_bins, d_counts, d_next, d_err, s);
+    case 8: return go_runs<8>(P, R, d_binom, L.n_bins, d_counts, d_next, d_err, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 cudaError_t launch_degeneracy(const DegLaunch &L, const uint64_t *d_binom, uint64_t start, uint64_t count,
                               unsigned long long *d_counts, int *d_err, cudaStream_t s) {
     DegParams P = deg_params(L);
@@ -623,15 +879,22 @@ cudaError_t launch_degeneracy(const DegLaunch &L, const uint64_t *d_binom, uint6
 
 cudaError_t launch_grover_eval(const int64_t *d_counts, int nb, int p, int n_sets, const double *d_angles,
                                double *d_E, double *d_grad, cudaStream_t s) {
-    const size_t smem = (size_t)(2 * nb + kGrMaxWarps + p) * sizeof(double2) + (size_t)nb * sizeof(double);
+    size_t smem = (size_t)(2 * nb + kGrMaxWarps + p) * sizeof(double2) + (size_t)nb * sizeof(double);
     if (smem > 200 * 1024) return cudaErrorInvalidValue;
+    // the phases of all rounds kept on chip when that leaves room for several
+    // sets on an SM: the adjoint sweep needs them again, and (round, value) pairs
+    // fill the lanes that the values alone do not (16 values, p = 10, 1024
+    // sets: 89 us before)
+    const size_t tab = (size_t)p * nb * sizeof(double2);
+    const int keep = smem + tab <= 24 * 1024 ? 1 : 0;
+    if (keep) smem += tab;
     static int attr_done[kMaxDevices];
     {
         cudaError_t e = smem_attr_once(grover_eval_kernel, 200 * 1024, attr_done);
         if (e != cudaSuccess) return e;
     }
     const int threads = std::min(kGrMaxThreads, std::max(32, (nb + 31) / 32 * 32));
-    grover_eval_kernel<<<n_sets, threads, smem, s>>>(d_counts, nb, p, d_angles, d_E, d_grad);
+    grover_eval_kernel<<<n_sets, threads, smem, s>>>(d_counts, nb, p, d_angles, d_E, d_grad, keep);
     return cudaGetLastError();
 }
 

@@ -2874,10 +2874,28 @@ qaoa_status qaoa_cost_degeneracy(qaoa_ctx *ctx, const qaoa_problem *prob, int64_
             QG_CUDA(ctx, cudaStreamSynchronize(ctx->stream), "binomial table upload");
         }
         QG_CUDA(ctx, cudaMemsetAsync(d_counts, 0, sizeof(int64_t) * n_bins, ctx->stream), "counts clear");
-        if (const int kk = degeneracy_sliced_kk(L)) {
+        const int kk = degeneracy_sliced_kk(L);
+        // (kk-1)-sets the sliced kernel would walk
+        uint64_t NT = 1;
+        for (int i = 0; i < kk - 1; i++) NT = NT * (uint64_t)(n - i) / (uint64_t)(i + 1);
+        // many: counted per (kk-2)-set.  A call with few of them is all latency, where
+        // the runs' longer tasks cost 10 us more (n = 42, k = 6, 850668: 70 / 60 us; n =
+        // 84, k = 5, 1929501: 76 / 76; n = 60, k = 6, 5461512: 112 / 143 with 64 reduced
+        // gradients)
+        if (kk >= kDegRunsMin && NT >= (1ull << 21)) {
+            void *d_next = nullptr;
+            st = scratch(ctx, "degtask", sizeof(unsigned long long), &d_next);
+            if (st) return st;
+            QG_CUDA(ctx, cudaMemsetAsync(d_next, 0, sizeof(unsigned long long), ctx->stream), "task counter clear");
+            cudaError_t e = launch_degeneracy_runs(L, static_cast<const uint64_t *>(d_binom),
+                                                   reinterpret_cast<unsigned long long *>(d_counts),
+                                                   static_cast<unsigned long long *>(d_next), ctx->d_err, ctx->stream);
+            if (e != cudaSuccess) return cuda_fail(ctx, e, "degeneracy kernel launch");
+            ctx->launches++;
+            return read_dev_err(ctx);
+        }
+        if (kk) {
             // bit-sliced count: all (kk-1)-sets T, each with the v < min(T)
-            uint64_t NT = 1;
-            for (int i = 0; i < kk - 1; i++) NT = NT * (uint64_t)(n - i) / (uint64_t)(i + 1);
             // each T adds at most 127 to one thread's 32-bit counter per value
             const uint64_t tslab = 1ull << 34;
             for (uint64_t t0 = 0; t0 < NT; t0 += tslab) {
