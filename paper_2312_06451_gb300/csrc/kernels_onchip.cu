@@ -19,7 +19,9 @@
 // later, behind a barrier that is there anyway.
 // 256 gradients at n = 10, p = 8, uint8 costs: 95.5 us (a shared-memory sweep
 // and two barriers per qubit and vector) and 11.5 us of coefficient preparation
-// before, 30.3 us now.
+// before, 30.3 us in these registers.  Costs fetched 16 bytes at a time, with the
+// first coefficients formed meanwhile by one warp, took a further 10% (between
+// event pairs 37.0 -> 33.3 us; one <C> at n = 12, p = 3: 16.5 -> 13.4).
 #include "onchip.cuh"
 
 namespace qg {
@@ -46,40 +48,56 @@ __global__ void __launch_bounds__(Chip<NB>::NT) onchip_kernel(const SmallDesc *_
                      NB > 9 || n >= 4 ? 0xFu : (1u << n) - 1u,
                      NB > 9 ? (0xFu << (12 - NB)) & 0xFu : (n == 9 ? 8u : 0u)};
 
-    // cost vector to shared memory (zero beyond 2^n), its largest value
+    // coefficients of the kChunk rounds that hold round k; the first chunk by one
+    // warp while the others fetch the costs
+    int chunk = 0;
+    auto form = [&](int first, int j) {
+        if (first + j < p)
+            s_rc[j] = round_consts(make_coef(ang[first + j], ang[p + first + j]), M, 0u, 0u);
+    };
+    auto load_chunk = [&](int k) {
+        if (k / kChunk == chunk) return;
+        chunk = k / kChunk;
+        __syncthreads();
+        if (tid < kChunk) form(chunk * kChunk, tid);
+        __syncthreads();
+    };
     if (tid == 0) s_top = 0;
     __syncthreads();
+    if (warp == NW - 1) form(0, lane);
+    // cost vector to shared memory (zero beyond 2^n), its largest value
     {
-        int top = 0;
+        constexpr int kPer = COST == 0 ? 4 : 16;  // values in 16 bytes
+        unsigned top = 0;
         const int have = 1 << n;
-        for (int x = tid; x < N; x += NT) {
-            if (COST == 0) {
-                reinterpret_cast<float *>(scost)[x] = x < have ? __ldg(reinterpret_cast<const float *>(D.cost) + x) : 0.f;
-            } else {
-                const int c = x < have ? (int)__ldg(reinterpret_cast<const unsigned char *>(D.cost) + x) : 0;
-                scost[x] = (unsigned char)c;
-                top = max(top, c);
+        if (have >= kPer) {
+#pragma unroll 4
+            for (int i = tid; i < N / kPer; i += NT) {
+                const uint4 v = i < have / kPer ? __ldg(reinterpret_cast<const uint4 *>(D.cost) + i) : make_uint4(0u, 0u, 0u, 0u);
+                reinterpret_cast<uint4 *>(scost)[i] = v;
+                if (COST == 1) top = __vmaxu4(top, __vmaxu4(__vmaxu4(v.x, v.y), __vmaxu4(v.z, v.w)));
+            }
+            top = max(max(top & 255u, (top >> 8) & 255u), max((top >> 16) & 255u, top >> 24));
+        } else {
+            for (int x = tid; x < N; x += NT) {
+                if (COST == 0) {
+                    reinterpret_cast<float *>(scost)[x] = x < have ? __ldg(reinterpret_cast<const float *>(D.cost) + x) : 0.f;
+                } else {
+                    const unsigned c = x < have ? (unsigned)__ldg(reinterpret_cast<const unsigned char *>(D.cost) + x) : 0u;
+                    scost[x] = (unsigned char)c;
+                    top = max(top, c);
+                }
             }
         }
         if (COST == 1) {
             top = __reduce_max_sync(0xffffffffu, top);
-            if (lane == 0) atomicMax(&s_top, top);
+            if (lane == 0) atomicMax(&s_top, (int)top);
         }
     }
     bool bad = false;
     for (int k = tid; k < 2 * p; k += NT) bad = bad || !isfinite(ang[k]);
     if (bad) atomicOr(err, DERR_BAD_ANGLE);
 
-    // coefficients of the kChunk rounds that hold round k
-    int chunk = -1;
-    auto load_chunk = [&](int k) {
-        if (k / kChunk == chunk) return;
-        chunk = k / kChunk;
-        __syncthreads();
-        const int r = chunk * kChunk + tid;
-        if (tid < kChunk && r < p) s_rc[tid] = round_consts(make_coef(ang[r], ang[p + r]), M, 0u, 0u);
-        __syncthreads();
-    };
     auto coef = [&](int k, float sgn) -> RoundC { return signed_round(s_rc[k % kChunk], sgn); };
     auto load_table = [&](const RoundC &C) {
         if (COST == 1) {  // its last readers passed a barrier since
@@ -102,7 +120,7 @@ __global__ void __launch_bounds__(Chip<NB>::NT) onchip_kernel(const SmallDesc *_
 
     // ---------------- initial state in layout Q, twisted basis
     float2 a[16], l[16];
-    __syncthreads();
+    __syncthreads();  // costs, their maximum and the first coefficients are there
 #pragma unroll
     for (int i = 0; i < 16; i++) {
         const uint32_t x = at(false, i);
