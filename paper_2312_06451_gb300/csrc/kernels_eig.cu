@@ -1065,25 +1065,115 @@ __global__ void __launch_bounds__(1024) eig_scale_kernel(const void *cost, int c
 //   BWD  : mu = T W, phi = e^{-i g C} T P; gamma partial
 //          sum_j (C_j - c0) Im(conj(mu_j) phi_j); L = T^T (e^{+i g C} mu)
 // Partial sums: fixed-order block sums, float64 across warps.
+// Full-period orbits (all but a few) of the lengths below have M_r as
+// compile-time constants: vectors 0 (t = 0), 2t - 1 and 2t (cos and sin of
+// momentum t) and, for even r, r - 1 (t = r/2), folded over members j and
+// r - j, so a transform is about r^2/2 multiply-adds with immediate operands
+// and reads no matrix.  The forms that read M_r from shared memory issue r^2
+// multiply-adds and kept the shared-memory pipe 61% busy (r = 16, four entries
+// a load), or read one entry per multiply-add (the other lengths).  256
+// gradients, a launch, before -> now: n = 11, k = 5 17.0 -> 8.3 us; 13, 6
+// 28.8 -> 11.2; 14, 7 40.2 -> 17.8; 15, 7 58.9 -> 19.3; 16, 8 50.6 -> 38.2
+// (the planes of all sets no longer fit L2); 18, 5 165 -> 26; 20, 4 102 -> 30.
+// n <= 9 has at most 126 states and other lengths no known use: they read M_r.
+constexpr bool orbit_folds(int r) { return (r >= 10 && r <= 16) || r == 18 || r == 20; }
+constexpr double cx_cos(double x) {  // |x| <= pi
+    double t = 1.0, s = 1.0;
+    for (int k = 1; k <= 24; k++) {
+        t *= -x * x / ((2.0 * k - 1.0) * (2.0 * k));
+        s += t;
+    }
+    return s;
+}
+constexpr double cx_sqrt(double x) {
+    double y = x > 1.0 ? x : 1.0;
+    for (int k = 0; k < 60; k++) y = 0.5 * (y + x / y);
+    return y;
+}
+template <int R>
+struct OrbitTab {
+    float k0 = 0.f, cs[R / 2 + 1][R / 2 + 1] = {}, sn[R / 2 + 1][R / 2 + 1] = {};  // [t][j]
+    constexpr OrbitTab() {
+        const double pi = 3.14159265358979323846, w = cx_sqrt(2.0 / R);
+        k0 = (float)(1.0 / cx_sqrt((double)R));
+        for (int t = 0; t <= R / 2; t++)
+            for (int j = 0; j <= R / 2; j++) {
+                const int q = (t * j) % R;
+                const double a = 2.0 * pi * (2 * q > R ? q - R : q) / R;
+                cs[t][j] = (float)(w * cx_cos(a));
+                const double b = a - 0.5 * pi;
+                sn[t][j] = (float)(w * cx_cos(b < -pi ? b + 2.0 * pi : b));
+            }
+    }
+};
+// x = M c
+template <int R>
+__device__ __forceinline__ void orbit_to_members(const float *c, float *x) {
+    constexpr OrbitTab<R> T;
+    constexpr int P = (R - 1) / 2;  // momenta with a cos and a sin, and pairs (j, R - j)
+    constexpr bool EVEN = R % 2 == 0;
+#pragma unroll
+    for (int j = 0; j <= R / 2; j++) {
+        float e = T.k0 * c[0];
+        if (EVEN) e = fmaf((j & 1) ? -T.k0 : T.k0, c[R - 1], e);
+#pragma unroll
+        for (int t = 1; t <= P; t++) e = fmaf(T.cs[t][j], c[2 * t - 1], e);
+        if (j == 0 || j > P) {
+            x[j] = e;
+            continue;
+        }
+        float o = T.sn[1][j] * c[2];
+#pragma unroll
+        for (int t = 2; t <= P; t++) o = fmaf(T.sn[t][j], c[2 * t], o);
+        x[j] = e + o;
+        x[R - j] = e - o;
+    }
+}
+// c = M^T x
+template <int R>
+__device__ __forceinline__ void orbit_from_members(const float *x, float *c) {
+    constexpr OrbitTab<R> T;
+    constexpr int P = (R - 1) / 2, H = R / 2;
+    constexpr bool EVEN = R % 2 == 0;
+    float s[P + 1], d[P + 1];
+#pragma unroll
+    for (int j = 1; j <= P; j++) {
+        s[j] = x[j] + x[R - j];
+        d[j] = x[j] - x[R - j];
+    }
+    float a = x[0], b = x[0];
+    if (EVEN) {
+        a += x[H];
+        b += (H & 1) ? -x[H] : x[H];
+    }
+#pragma unroll
+    for (int j = 1; j <= P; j++) {
+        a += s[j];
+        b += (j & 1) ? -s[j] : s[j];
+    }
+    c[0] = T.k0 * a;
+    if (EVEN) c[R - 1] = T.k0 * b;
+#pragma unroll
+    for (int t = 1; t <= P; t++) {
+        float e = T.cs[t][0] * x[0];
+        if (EVEN) e = fmaf(T.cs[t][H], x[H], e);
+        float o = T.sn[t][1] * d[1];
+#pragma unroll
+        for (int j = 1; j <= P; j++) e = fmaf(T.cs[t][j], s[j], e);
+#pragma unroll
+        for (int j = 2; j <= P; j++) o = fmaf(T.sn[t][j], d[j], o);
+        c[2 * t - 1] = e;
+        c[2 * t] = o;
+    }
+}
+
 template <int MODE, int RMAX>
 __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, OrbitArgs A) {
     __shared__ double red[kOrbitThreads / 32];
     // every M_r of the layout (sum of r^2 over the periods, at most
     // kOrbitSmem floats), read by all threads at once: shared-memory broadcasts
     __shared__ __align__(16) float s_mr[kOrbitSmem];
-    // the full-period matrix M_RMAX and its transpose, 16-byte aligned, so
-    // that both transforms read four consecutive entries at once
-    constexpr int kF = RMAX <= 16 ? RMAX : 1;
-    __shared__ __align__(16) float s_mf[kF * kF];
-    __shared__ __align__(16) float s_mft[kF * kF];
     for (int i = threadIdx.x; i < T.mr_len; i += kOrbitThreads) s_mr[i] = T.mr[i];
-    const int off_full = RMAX <= 16 ? T.mr_off[RMAX] : -1;
-    if (off_full >= 0)
-        for (int i = threadIdx.x; i < kF * kF; i += kOrbitThreads) {
-            const float m = T.mr[off_full + i];
-            s_mf[i] = m;
-            s_mft[(i % kF) * kF + i / kF] = m;
-        }
     __syncthreads();
     // Two adjacent lanes per (orbit, set): part 0 holds the real rows, part 1
     // the imaginary ones.  M_r is real, so each row transforms on its own;
@@ -1104,19 +1194,17 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
             return part ? make_float2(w, v) : make_float2(v, w);
         };
         auto take = [&](float2 z) -> float { return part ? z.y : z.x; };
-        // Full-period orbits (all but a few; they come first in orbit order)
-        // take a copy of the body with the period known at compile time: no
-        // bound tests, M_r rows read as float4.  The sums run over the same
-        // index order in both copies, so the results agree bit for bit.
+        // Full-period orbits take a copy of the body with the period and M_r known at
+        // compile time: no bound tests, no matrix reads.
         auto body = [&](auto full_tag) {
             constexpr bool FULL = decltype(full_tag)::value;
             const int R = FULL ? RMAX : r;
-            const float *M = FULL ? s_mf : s_mr + T.mr_off[r];
+            const float *M = FULL ? nullptr : s_mr + T.mr_off[r];
             float c[RMAX];
-            // full-period orbits start on a multiple of 16 members: their vector
-            // positions and member indices are read once, 16 bytes at a time
+            // vector positions and member indices, read once (16 bytes at a time
+            // where the period keeps every orbit aligned)
             int pos[FULL ? RMAX : 1], mem[FULL ? RMAX : 1];
-            if constexpr (FULL) {
+            if constexpr (FULL && RMAX % 4 == 0) {
                 const int4 *vp = reinterpret_cast<const int4 *>(T.vec_pos + s0);
                 const int4 *mp = reinterpret_cast<const int4 *>(T.members + s0);
 #pragma unroll
@@ -1130,6 +1218,12 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
                     mem[4 * q + 1] = w.y;
                     mem[4 * q + 2] = w.z;
                     mem[4 * q + 3] = w.w;
+                }
+            } else if constexpr (FULL) {
+#pragma unroll
+                for (int q = 0; q < RMAX; q++) {
+                    pos[q] = __ldg(T.vec_pos + s0 + q);
+                    mem[q] = __ldg(T.members + s0 + q);
                 }
             }
             auto vpos = [&](int a) -> int {
@@ -1148,23 +1242,15 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
 #pragma unroll
                 for (int a = 0; a < RMAX; a++)
                     if (a < R) c[a] = in[row + vpos(a)];
-                // member sums accumulated side by side (independent FMA chains)
+                if constexpr (FULL) {
+                    orbit_to_members<RMAX>(c, x);
+                } else {
+                    // member sums accumulated side by side (independent FMA chains)
 #pragma unroll
-                for (int j = 0; j < RMAX; j++) x[j] = 0.f;
+                    for (int j = 0; j < RMAX; j++) x[j] = 0.f;
 #pragma unroll
-                for (int a = 0; a < RMAX; a++) {
-                    if (a >= R) continue;
-                    if constexpr (FULL) {  // row a of M^T: M[j][a], j = 4q .. 4q + 3
-                        const float4 *MT4 = reinterpret_cast<const float4 *>(s_mft) + a * (RMAX / 4);
-#pragma unroll
-                        for (int q = 0; q < RMAX / 4; q++) {
-                            const float4 m = MT4[q];
-                            x[4 * q] = fmaf(m.x, c[a], x[4 * q]);
-                            x[4 * q + 1] = fmaf(m.y, c[a], x[4 * q + 1]);
-                            x[4 * q + 2] = fmaf(m.z, c[a], x[4 * q + 2]);
-                            x[4 * q + 3] = fmaf(m.w, c[a], x[4 * q + 3]);
-                        }
-                    } else {
+                    for (int a = 0; a < RMAX; a++) {
+                        if (a >= R) continue;
 #pragma unroll
                         for (int j = 0; j < RMAX; j++) {
                             if (j >= R) continue;
@@ -1175,22 +1261,14 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
             };
             // c = T^T x written to this lane's row of `out` (tf32 split when out_lo)
             auto from_amp = [&](const float (&x)[RMAX], float *out, float *out_lo) {
+if constexpr (FULL) {
+                    orbit_from_members<RMAX>(x, c);
+                } else {
 #pragma unroll
-                for (int a = 0; a < RMAX; a++) c[a] = 0.f;
+                    for (int a = 0; a < RMAX; a++) c[a] = 0.f;
 #pragma unroll
-                for (int j = 0; j < RMAX; j++) {
-                    if (j >= R) continue;
-                    if constexpr (FULL) {
-                        const float4 *M4 = reinterpret_cast<const float4 *>(M) + j * (RMAX / 4);
-#pragma unroll
-                        for (int q = 0; q < RMAX / 4; q++) {
-                            const float4 m = M4[q];
-                            c[4 * q] = fmaf(m.x, x[j], c[4 * q]);
-                            c[4 * q + 1] = fmaf(m.y, x[j], c[4 * q + 1]);
-                            c[4 * q + 2] = fmaf(m.z, x[j], c[4 * q + 2]);
-                            c[4 * q + 3] = fmaf(m.w, x[j], c[4 * q + 3]);
-                        }
-                    } else {
+                    for (int j = 0; j < RMAX; j++) {
+                        if (j >= R) continue;
 #pragma unroll
                         for (int a = 0; a < RMAX; a++) {
                             if (a >= R) continue;
@@ -1267,9 +1345,8 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
                 if (A.out) from_amp(x, A.out, A.out_lo);
             }
         };
-        // (the 32-wide copy would not fit the registers next to the generic one)
-        if constexpr (RMAX <= 16) {
-            if (r == RMAX && off_full >= 0 && (s0 & 3) == 0) body(std::integral_constant<bool, true>());
+        if constexpr (orbit_folds(RMAX)) {
+            if (r == RMAX && (RMAX % 4 != 0 || (s0 & 3) == 0)) body(std::integral_constant<bool, true>());
             else body(std::integral_constant<bool, false>());
         } else {
             body(std::integral_constant<bool, false>());
@@ -1358,33 +1435,35 @@ cudaError_t launch_eig_prepare(const float *V, int D, int ld, float *Vp, float *
     return cudaGetLastError();
 }
 
+template <int RMAX>
+static cudaError_t go_orbit(const OrbitTabs &T, const OrbitArgs &A, dim3 grid, cudaStream_t s) {
+    switch (A.mode) {
+    case ORB_INIT: orbit_kernel<ORB_INIT, RMAX><<<grid, kOrbitThreads, 0, s>>>(T, A); break;
+    case ORB_PHASE: orbit_kernel<ORB_PHASE, RMAX><<<grid, kOrbitThreads, 0, s>>>(T, A); break;
+    case ORB_LAST: orbit_kernel<ORB_LAST, RMAX><<<grid, kOrbitThreads, 0, s>>>(T, A); break;
+    case ORB_BWD: orbit_kernel<ORB_BWD, RMAX><<<grid, kOrbitThreads, 0, s>>>(T, A); break;
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 cudaError_t launch_orbit(const OrbitTabs &T, const OrbitArgs &A, cudaStream_t s) {
     if (T.max_r < 1 || T.max_r > kSymMaxN || T.mr_len < 1 || T.mr_len > kOrbitSmem) return cudaErrorInvalidValue;
     dim3 grid((T.n_orbits + kOrbitsPerBlock - 1) / kOrbitsPerBlock, A.nsets);
     if (grid.x == 0 || grid.y == 0) return cudaSuccess;
-    // the longest orbit sets the register arrays: 16 or 32 members
-    const bool r16 = T.max_r <= 16;
-    switch (A.mode) {
-    case ORB_INIT:
-        if (r16) orbit_kernel<ORB_INIT, 16><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        else orbit_kernel<ORB_INIT, 32><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        break;
-    case ORB_PHASE:
-        if (r16) orbit_kernel<ORB_PHASE, 16><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        else orbit_kernel<ORB_PHASE, 32><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        break;
-    case ORB_LAST:
-        if (r16) orbit_kernel<ORB_LAST, 16><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        else orbit_kernel<ORB_LAST, 32><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        break;
-    case ORB_BWD:
-        if (r16) orbit_kernel<ORB_BWD, 16><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        else orbit_kernel<ORB_BWD, 32><<<grid, kOrbitThreads, 0, s>>>(T, A);
-        break;
-    default:
-        return cudaErrorInvalidValue;
+    // the longest orbit sets the register arrays: its length where that has
+    // constants of its own, else 16 or 32
+    switch (T.max_r) {
+    case 10: return go_orbit<10>(T, A, grid, s);
+    case 11: return go_orbit<11>(T, A, grid, s);
+    case 12: return go_orbit<12>(T, A, grid, s);
+    case 13: return go_orbit<13>(T, A, grid, s);
+    case 14: return go_orbit<14>(T, A, grid, s);
+    case 15: return go_orbit<15>(T, A, grid, s);
+    case 18: return go_orbit<18>(T, A, grid, s);
+    case 20: return go_orbit<20>(T, A, grid, s);
+    default: return T.max_r <= 16 ? go_orbit<16>(T, A, grid, s) : go_orbit<32>(T, A, grid, s);
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_eig_scale(const void *cost, int cost_dtype, int D, const float2 *init, double *mean, float *sc,
