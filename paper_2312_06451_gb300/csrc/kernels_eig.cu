@@ -293,14 +293,15 @@ gemm_simt_kernel(const float *__restrict__ A, const float *__restrict__ B, int K
 // round-to-nearest adds.
 // Ring mixer on 12870 states, 256 sets, p = 6 gradient (24 grouped products):
 // 3.47 -> 2.36 ms; error against 64 bits 5.5e-6 -> 4.6e-6 (draining every 3
-// chunks instead of 2: 2.28 ms, 5.8e-6).
+// chunks instead of 2: 2.28 ms, 5.8e-6).  A product takes 71 us, 0.46 of the
+// measured bf16 rate for its three; with the orbit transforms below, 2.17 ms.
 //
 // 128 x 128 output tile per CTA, STAGES-deep TMA ring of 128-byte-swizzled
 // K-major tiles.  Warp 0 lane 0 issues TMA loads, warp 1 lane 0 the MMAs;
 // warps 2..17 drain the chunks and run the fused epilogue, four per quarter
 // of the accumulator rows (a warp reaches only its quarter of tensor memory),
-// 32 columns each.  Four accumulator buffers (all 512 tensor-memory columns)
-// let the MMAs run up to three chunks ahead of the drain.
+// 32 columns each.  Two pairs of accumulators (all 512 tensor-memory columns)
+// let the MMAs fill one while the other is drained.
 // Split of the last, partial wave of tiles along K (see gemm_tc_kernel).
 struct SplitArgs {
     int full;       // tiles computed whole, by blocks 0 .. full-1
@@ -1259,7 +1260,7 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
                     }
                 }
             };
-            // c = T^T x written to this lane's row of `out` (tf32 split when out_lo)
+            // c = T^T x written to this lane's row of `out` (half planes when out_lo)
             auto from_amp = [&](const float (&x)[RMAX], float *out, float *out_lo) {
 if constexpr (FULL) {
                     orbit_from_members<RMAX>(x, c);

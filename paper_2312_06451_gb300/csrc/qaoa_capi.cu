@@ -113,7 +113,7 @@ struct LaunchRec {
     const GroupTile *gtiles = nullptr;
     OrbitTabs otab{};
     OrbitArgs oarg{};
-    // LK_OPERANDS: padded (and tf32-split) operand planes of an eigendecomposition
+    // LK_OPERANDS: padded (and split) operand planes of an eigendecomposition
     struct {
         int sym;
         const float *V;
