@@ -36,6 +36,7 @@
 // order, so results are bitwise reproducible run to run.
 #include "common.cuh"
 #include "bulk.cuh"
+#include "phase.cuh"
 
 #include <algorithm>
 #include <cstdlib>
@@ -57,28 +58,6 @@ constexpr uint32_t kR1TabOff = 512;
 constexpr uint32_t kR1HeadB = kR1TabOff + kPhaseTable * 8;
 static_assert(kR1RedOff + 3 * (kR1Threads / 32) * 8 + 8 * 8 <= kR1TabOff, "head layout");
 static_assert(kR1HeadB % 128 == 0, "stage area alignment");
-constexpr float kTwoPiF = 6.2831853071795864769f;
-
-__device__ __forceinline__ float2 r1_cmul(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-// a * conj(b)
-__device__ __forceinline__ float2 r1_cmul_conj(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
-}
-
-// e^{-i g C} for a float32 cost: the turn count (g_hi + g_lo) C formed as a
-// float pair (exact head product), its integer part removed exactly, the
-// remaining fraction of a turn to the hardware sine/cosine.
-__device__ __forceinline__ float2 r1_phase_f32(float C, float ghi, float glo) {
-    const float th = ghi * C;
-    const float te = fmaf(ghi, C, -th);
-    const float tl = fmaf(glo, C, te);
-    const float f = (th - rintf(th)) + tl;
-    float s, c;
-    __sincosf(kTwoPiF * f, &s, &c);
-    return make_float2(c, -s);
-}
 
 // Descriptor (unit) containing global tile t; tb has nd + 1 entries.
 __device__ __forceinline__ int r1_find(const uint32_t *__restrict__ tb, int nd, uint32_t t) {
@@ -190,7 +169,7 @@ __device__ __forceinline__ double r1_block_sum3(const Kahan (&acc)[3], float2 (*
 template <int COST>
 __device__ __forceinline__ float2 r1_phase(const float2 *stab, float C, int ci, const RoundCoef &cf) {
     if constexpr (COST == 1) return stab[ci];
-    else return r1_phase_f32(C, cf.g_hi, cf.g_lo);
+    else return phase_f32(C, cf.g_hi, cf.g_lo);
 }
 
 __device__ __forceinline__ void r1_st2(float2 *p, float2 a, float2 b) {
@@ -493,7 +472,7 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
                     float2 a[2];
 #pragma unroll
                     for (int e = 0; e < 2; e++) {
-                        a[e] = r1_cmul(make_float2(fo[e].x + U.dp.x, fo[e].y + U.dp.y),
+                        a[e] = cmul(make_float2(fo[e].x + U.dp.x, fo[e].y + U.dp.y),
                                        r1_phase<COST>(stab, c[j][e], ci[j][e], cf));
                         if (e == 0 || two) {
                             s0 += a[e].x;
@@ -526,11 +505,11 @@ __global__ void __launch_bounds__(kR1Block, 1) r1_pass_kernel(const R1Desc *__re
                         s0 = fmaf(cs, fmaf(lv.x, fo[e].y, -lv.y * fo[e].x), s0);  // (C - c0) Im(conj(mu) phi)
                         if (round > 0) {
                             const float2 ph = r1_phase<COST>(stab, C, ci[j][e], cf);
-                            nl[e] = r1_cmul_conj(lv, ph);  // mu e^{+i g C}
+                            nl[e] = cmul_conj(lv, ph);  // mu e^{+i g C}
                             s1 += nl[e].x;
                             s2 += nl[e].y;
                             if (!U.ckpt) {
-                                const float2 q = r1_cmul_conj(fo[e], ph);
+                                const float2 q = cmul_conj(fo[e], ph);
                                 np[e] = make_float2(q.x - U.dq.x, q.y - U.dq.y);
                             }
                         }

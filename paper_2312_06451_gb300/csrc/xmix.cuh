@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "bulk.cuh"
+#include "phase.cuh"
 
 #include <math.h>
 
@@ -19,8 +20,6 @@ constexpr int kTile = 1 << kT;
 constexpr int kNT = 256;
 constexpr int kNW = kNT / 32;
 
-constexpr float kTwoPiF = 6.2831853071795864769f;
-
 // XOR swizzle of a tile-local amplitude index into shared memory.  Bits 1..3
 // are flipped by a fold of bits 6..14, bit 0 is kept so that the amplitude
 // pair (l, l^1) stays one aligned 16-byte vector.  With it, every stage's
@@ -30,28 +29,6 @@ constexpr float kTwoPiF = 6.2831853071795864769f;
 // swz(a ^ b) = swz(a) ^ swz(b).
 __device__ __forceinline__ uint32_t swz(uint32_t l) {
     return l ^ ((((l >> 6) ^ (l >> 9) ^ (l >> 12)) & 7u) << 1);
-}
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-// a * conj(b)
-__device__ __forceinline__ float2 cmul_conj(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, a.y * b.y), fmaf(a.y, b.x, -a.x * b.y));
-}
-
-// e^{-i gamma C} for a float32 cost.  gamma/(2 pi) = g_hi + g_lo; the product
-// t = (g_hi + g_lo) C is formed as a float pair (exact head product by FMA),
-// its integer part removed exactly, and the remaining turn f in [-1/2, 1/2]
-// fed to the hardware sine/cosine at 2 pi f in [-pi, pi].
-__device__ __forceinline__ float2 phase_f32(float C, float ghi, float glo) {
-    const float th = ghi * C;
-    const float te = fmaf(ghi, C, -th);
-    const float tl = fmaf(glo, C, te);
-    const float f = (th - rintf(th)) + tl;
-    float s, c;
-    __sincosf(kTwoPiF * f, &s, &c);
-    return make_float2(c, -s);
 }
 
 // (sin, cos) of 2 pi t for a float64 turn count t, without float64
