@@ -213,7 +213,8 @@ int64_t qaoa_scratch_bytes(const qaoa_ctx *ctx);
 
 /* Cost vector over the feasible set (Sec. 2.1: C(x) is computed once, stored
  * for every feasible x and re-used by every evaluation).
- *   d_cost      device output, dim elements of cost_dtype
+ *   d_cost      device output, dim elements of cost_dtype, aligned for one element
+ *               (evaluations take cost vectors at 16-byte boundaries)
  *   cost_dtype  QAOA_COST_U8 (integer costs; fails with QAOA_ERR_INVALID if a
  *               value can exceed 255) or QAOA_COST_F32
  *   dim         2^n for unconstrained problems, binom(n,k) for DKS

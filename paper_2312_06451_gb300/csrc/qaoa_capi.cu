@@ -2492,6 +2492,8 @@ qaoa_status qaoa_cost_precompute(qaoa_ctx *ctx, const qaoa_problem *prob, void *
         const int n = prob->n;
         if (cost_dtype != QAOA_COST_F32 && cost_dtype != QAOA_COST_U8)
             return fail(ctx, QAOA_ERR_INVALID, "unknown cost dtype %d", cost_dtype);
+        if (cost_dtype == QAOA_COST_F32 && ((uintptr_t)d_cost & 3))
+            return fail(ctx, QAOA_ERR_INVALID, "float32 d_cost must be 4-byte aligned");
         const bool dks = prob->kind == QAOA_PROBLEM_DKS || prob->kind == QAOA_PROBLEM_KVC;
         if (n < 1 || n > (dks ? binom_table_max() : 34))
             return fail(ctx, QAOA_ERR_INVALID, "n=%d out of range", n);
