@@ -339,6 +339,16 @@ qaoa_status scratch(qaoa_ctx *ctx, const char *name, size_t bytes, void **out) {
     return QAOA_OK;
 }
 
+// Give a scratch buffer back (the cached plan may point into it).
+void release(qaoa_ctx *ctx, const char *name) {
+    auto it = ctx->bufs.find(name);
+    if (it == ctx->bufs.end() || !it->second.p) return;
+    cudaStreamSynchronize(ctx->stream);
+    cudaFree(it->second.p);
+    ctx->bufs.erase(it);
+    ctx->plan.valid = false;
+}
+
 qaoa_status host_stage(qaoa_ctx *ctx, size_t bytes) {
     if (ctx->h_stage_bytes >= bytes) return QAOA_OK;
     if (ctx->h_stage) {
@@ -1206,17 +1216,21 @@ GridPlan plan_grid(const qaoa_ctx *ctx, const std::vector<Unit> &units, bool gra
     return g;
 }
 
+// Vector stride of a Grover-mixer unit (amplitudes), and the state bytes of all
+// such units with all checkpoints (p + 1 vectors a gradient).
+int64_t grover_ld(int64_t dim) { return (dim + 63) / 64 * 64; }
+size_t grover_bytes(const std::vector<Unit> &units, bool grad, int ckpt) {
+    size_t b = 0;
+    for (const Unit &u : units)
+        if (u.mixer_kind == QAOA_MIXER_GROVER)
+            b += align_up((size_t)grover_ld(u.dim) * sizeof(float2) * (grad ? (ckpt != QAOA_CKPT_NONE ? u.p + 1 : 2) : 1));
+    return b;
+}
+
 // Build (or reuse) the launch plan for a unit list and enqueue it.
 qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, int ckpt) {
-    // the plan is reused when the units are byte for byte the ones it was made
-    // for (a compare of 256 units takes 2 us; hashing them byte by byte took 35)
-    const Plan &have = ctx->plan;
-    if (!(have.valid && have.grad == (grad ? 1 : 0) && have.ckpt == ckpt && have.epoch == ctx->tune_epoch &&
-          have.units.size() == units.size() &&
-          std::memcmp(have.units.data(), units.data(), units.size() * sizeof(Unit)) == 0)) {
-        if (capturing(ctx))
-            return fail(ctx, QAOA_ERR_INVALID,
-                        "launch plan not built; run the same call once before stream capture");
+    bool one_launch = false;  // the plan built last has one-launch units
+    auto build = [&](bool allow_grid) -> qaoa_status {
         // ---- per-unit metadata: coefficients, tables, partials
         const int nu = (int)units.size();
         const int smax = small_max_n();
@@ -1226,19 +1240,20 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         size_t free_b = 0, total_b = 0;
         cudaMemGetInfo(&free_b, &total_b);
         const size_t held = ctx->bufs.count("state") ? ctx->bufs["state"].bytes : 0;
-        const size_t held_grid = ctx->bufs.count("gridstate") ? ctx->bufs["gridstate"].bytes : 0;
+        const size_t held_r1 = ctx->bufs.count("r1state") ? ctx->bufs["r1state"].bytes : 0;
         auto budget_of = [&](size_t avail) -> size_t {
             const double b = (double)avail * 0.92 - 1.0 * (1ull << 30);
-            size_t v = b > 0 ? (size_t)b : 0;
+            const size_t v = b > 0 ? (size_t)b : 0;
             return ctx->state_limit >= 0 ? std::min(v, (size_t)ctx->state_limit) : v;
         };
-        GridPlan gp = plan_grid(ctx, units, grad, ckpt, budget_of(free_b + held + held_grid));
-        // what the cooperative launches take is not there for the passes
-        const size_t grid_more = gp.bytes > held_grid ? gp.bytes - held_grid : 0;
-        free_b -= std::min(free_b, grid_more);
-        size_t budget = budget_of(free_b + held);
-        if (ctx->state_limit >= 0)
-            budget = std::min(budget, (size_t)ctx->state_limit - std::min((size_t)ctx->state_limit, gp.bytes));
+        const size_t budget = budget_of(free_b + held), r1_all = budget_of(free_b + held + held_r1);
+        // Units that run in one launch use the state buffer before the passes
+        // do, so neither takes from the other.  Grover units have their own
+        // buffer beside it: all of them with all checkpoints must fit there too,
+        // else the X-mixer units run as passes, which take less at a time.
+        GridPlan gp = plan_grid(ctx, units, grad, ckpt, allow_grid ? budget : 0);
+        if (gp.bytes && gp.bytes + grover_bytes(units, grad, ckpt) > r1_all) gp = plan_grid(ctx, units, grad, ckpt, 0);
+        one_launch = gp.bytes > 0;
         const std::vector<char> &on_grid = gp.on;
         // coefficients of all units back to back (the sets of one eigenbasis
         // job are consecutive, so their rounds form a [set][round] array)
@@ -1302,7 +1317,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             std::vector<size_t> soff;
         };
         std::vector<Wave> waves;
-        size_t state_need = 0;
+        size_t state_need = gp.bytes;
         for (auto &kv : groups) {
             Wave w;
             w.gk = kv.first;
@@ -1422,8 +1437,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         }
         // cooperative launches (13 <= n <= 20), one per cost type and class
         if (gp.bytes) {
-            void *d_gs = nullptr, *d_bar = nullptr;
-            if ((st = scratch(ctx, "gridstate", gp.bytes, &d_gs))) return st;
+            void *d_bar = nullptr;
             if ((st = scratch(ctx, "gridbar", sizeof(unsigned) * gp.n_bar, &d_bar))) return st;
             for (int lw = 0; lw < 2 * kGridClasses * kGridWaves; lw++) {
                 // the cooperative launches first: the clusters fill what their last one leaves
@@ -1444,7 +1458,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                     d.angles = u.angles;
                     d.E_out = u.E;
                     d.grad_out = grad ? u.grad : nullptr;
-                    d.X = reinterpret_cast<float2 *>(static_cast<char *>(d_gs) + gp.off[i]);
+                    d.X = reinterpret_cast<float2 *>(static_cast<char *>(d_state) + gp.off[i]);
                     d.lam = grad ? d.X + (int64_t)u.p * N : nullptr;
                     d.part = reinterpret_cast<double *>(d.X + (int64_t)(grad ? u.p + 2 : 2) * N);
                     d.bar = static_cast<unsigned *>(d_bar) + gp.bar[i];
@@ -1648,11 +1662,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             if (!rgroups.empty()) {
                 const int64_t tile = r1_tile_amps();
                 const uint32_t gmax = r1_max_grid();
-                const size_t held_r1 = ctx->bufs.count("r1state") ? ctx->bufs["r1state"].bytes : 0;
-                const double rb = (double)(free_b + held + held_r1) * 0.92 - 1.0 * (1ull << 30);
-                size_t r1_budget = rb > 0 ? (size_t)rb : 0;
-                if (ctx->state_limit >= 0) r1_budget = std::min(r1_budget, (size_t)ctx->state_limit - std::min((size_t)ctx->state_limit, gp.bytes));
-                r1_budget = r1_budget > state_need ? r1_budget - state_need : 0;
+                const size_t r1_budget = r1_all > state_need ? r1_all - state_need : 0;
                 struct RUnit {
                     int i;
                     int64_t ld;
@@ -1676,7 +1686,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                         const Unit &u = units[i];
                         RUnit ru;
                         ru.i = i;
-                        ru.ld = (u.dim + 63) / 64 * 64;
+                        ru.ld = grover_ld(u.dim);
                         ru.nt = (uint32_t)((u.dim + tile - 1) / tile);
                         const size_t vb = (size_t)ru.ld * sizeof(float2);
                         // p + 1 vectors (phi_0..phi_{p-1} and lambda) with checkpoints,
@@ -2151,6 +2161,25 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         ctx->plan.ckpt = ckpt;
         ctx->plan.epoch = ctx->tune_epoch;
         ctx->plan.valid = true;
+        return QAOA_OK;
+    };
+    // the plan is reused when the units are byte for byte the ones it was made
+    // for (a compare of 256 units takes 2 us; hashing them byte by byte took 35)
+    const Plan &have = ctx->plan;
+    if (!(have.valid && have.grad == (grad ? 1 : 0) && have.ckpt == ckpt && have.epoch == ctx->tune_epoch &&
+          have.units.size() == units.size() &&
+          std::memcmp(have.units.data(), units.data(), units.size() * sizeof(Unit)) == 0)) {
+        if (capturing(ctx))
+            return fail(ctx, QAOA_ERR_INVALID,
+                        "launch plan not built; run the same call once before stream capture");
+        qaoa_status st = build(true);
+        if (st == QAOA_ERR_OOM && one_launch) {
+            // nothing of the call has run yet: as passes, in the memory the one-launch units would have held
+            release(ctx, "state");
+            ctx->err.clear();
+            st = build(false);
+        }
+        if (st) return st;
     }
 
     // ---- enqueue
