@@ -381,7 +381,8 @@ qaoa_status qaoa_set_state_limit(qaoa_ctx *ctx, int64_t bytes);
  *   split   0 equal chunks, 1 full chunks first, 2 remainder first
  *   nbuf_bwd_contig / nbuf_bwd_gather  1 or 2 tile buffers per CTA in the
  *           adjoint passes (1: two CTAs per SM; 2: one CTA per SM)
- *   ms      time of the tuning run that chose it (output only)
+ *   ms      time of the tuning run that chose it, 0 for a schedule that was not
+ *           tuned (see qaoa_set_xtune)
  * The schedule changes the rounding order only. */
 typedef struct {
     int n;
@@ -403,13 +404,17 @@ int qaoa_pass_schedule(int n, int cmin, int split, int *c, int *lo, int max);
  * (1..8) on the caller's cost vector for every schedule with the fewest
  * passes, then the adjoint buffer choices, on the context stream, and keeps
  * the fastest for (n, cost_dtype) in the context; out (may be NULL) receives
- * it.  Angles are fixed internal values; results of the runs are discarded.
+ * it.  Sizes that have a kernel for all rounds in one launch (n <= 20) go on
+ * taking it where it is faster than the best schedule; the schedule then serves
+ * the calls that need passes.  Angles are fixed internal values; results of the runs are discarded.
  * Synchronous.  Uses the context's scratch like a gradient call of p rounds. */
 qaoa_status qaoa_autotune_x(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, int n, int p,
                             int want_grad, qaoa_xtune *out);
 /* Set (e.g. restore a saved tuning) or read the schedule used for
- * (t->n, t->cost_dtype).  Without a stored entry the default is cmin 4,
- * split 0, one adjoint buffer. */
+ * (t->n, t->cost_dtype).  A tuned schedule (ms > 0) serves the calls that take
+ * passes; one with ms 0 is pinned: every call of that size takes passes with
+ * it.  Without a stored entry the default is cmin 4, split 0, one adjoint
+ * buffer. */
 qaoa_status qaoa_set_xtune(qaoa_ctx *ctx, const qaoa_xtune *t);
 qaoa_status qaoa_get_xtune(qaoa_ctx *ctx, int n, int cost_dtype, qaoa_xtune *out);
 

@@ -533,7 +533,8 @@ class Context:
     # ------------------------------------------------ pass-schedule tuning
     def autotune(self, cost: torch.Tensor, n: int, p: int = 2, want_grad: bool = True) -> dict:
         """Time every X-mixer pass schedule for (n, cost dtype) on this cost
-        vector and keep the fastest in the context (qaoa_autotune_x)."""
+        vector and keep the fastest in the context, for the calls that take
+        passes (qaoa_autotune_x)."""
         cost = _dev_tensor(cost, "cost")
         t = B.QaoaXTune()
         self._check(self._lib.qaoa_autotune_x(self._h, _ptr(cost), _cost_dtype(cost), n, p, 1 if want_grad else 0,
@@ -543,7 +544,9 @@ class Context:
         return d
 
     def set_tuning(self, t: dict):
-        """Install a schedule (e.g. one saved from autotune())."""
+        """Install a schedule: one saved from autotune() serves the calls that
+        take passes; one without "ms" is pinned, every call of its size takes
+        passes with it."""
         st = B.QaoaXTune(*(int(t[k]) for k in ("n", "cost_dtype", "cmin", "split", "nbuf_bwd_contig",
                                                "nbuf_bwd_gather")), float(t.get("ms", 0.0)))
         self._check(self._lib.qaoa_set_xtune(self._h, ctypes.byref(st)))

@@ -239,6 +239,7 @@ struct qaoa_ctx {
     Plan plan;
     std::set<std::string> eig_ready;  // prepared eigenbasis operands (by V, lambda, D)
     std::map<std::pair<int, int>, qaoa_xtune> xtune;  // X-mixer schedules by (n, cost dtype)
+    std::set<std::pair<int, int>> xpinned;            // those that the caller pins: passes, whatever else would be taken
     uint64_t tune_epoch = 0;                          // bumped on every schedule change
     int ckpt_mode = QAOA_CKPT_PASS;                   // checkpointing of batched gradients
     int64_t state_limit = -1;                         // caller's cap on state scratch (-1: none)
@@ -1149,8 +1150,8 @@ const char *dtype_name(int dt) { return dt == QAOA_COST_U8 ? "u8" : "f32"; }
 // while the passes' time grows more slowly: even at four launches (n = 20: 500 /
 // 495), so at most kGridWaves.
 constexpr int kGridWaves = 3;
-// Not taken where the caller asks for the passes: a schedule installed for the
-// size, a fusion mode, gradients without checkpoints (two vectors; this path
+// Not taken where the caller asks for the passes: a schedule pinned for the
+// size (qaoa_set_xtune), a fusion mode, gradients without checkpoints (two vectors; this path
 // keeps p + 2), or when the vectors do not fit the budget.
 // One launch per class and wave: each n of a cluster on its own, the larger ones together.
 constexpr int kGridClasses = kGridClusterN - kPassTileBits + 1;
@@ -1180,7 +1181,7 @@ GridPlan plan_grid(const qaoa_ctx *ctx, const std::vector<Unit> &units, bool gra
         for (int i = 0; i < nu; i++) {
             const Unit &u = units[i];
             if (u.mixer_kind != QAOA_MIXER_X || u.ma || u.gm || u.cost_dtype != dt || u.n <= kPassTileBits ||
-                u.n > kGridMaxN || grid_class(u.n) != gc || ctx->xtune.count({u.n, dt}))
+                u.n > kGridMaxN || grid_class(u.n) != gc || ctx->xpinned.count({u.n, dt}))
                 continue;
             us.push_back(i);
             off.push_back(bytes);
@@ -3041,6 +3042,8 @@ qaoa_status qaoa_set_xtune(qaoa_ctx *ctx, const qaoa_xtune *t) {
                     "schedule needs %d < n <= %d, cost dtype 0/1, cmin 4..8, split 0..2, buffers 1 or 2",
                     small_max_n(), kMaxXQubits);
     ctx->xtune[{t->n, t->cost_dtype}] = *t;
+    if (t->ms > 0.0) ctx->xpinned.erase({t->n, t->cost_dtype});
+    else ctx->xpinned.insert({t->n, t->cost_dtype});
     ctx->tune_epoch++;
     return QAOA_OK;
 }
@@ -3092,13 +3095,16 @@ qaoa_status qaoa_autotune_x(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, i
         const std::vector<Unit> us(1, u);
         const int ck = want_grad ? ctx->ckpt_mode : 0;
         const bool had = ctx->xtune.count({n, cost_dtype}) != 0;
+        const bool was_pinned = ctx->xpinned.count({n, cost_dtype}) != 0;
         const qaoa_xtune saved = tune_for(ctx, n, cost_dtype);
         cudaEvent_t e0 = take_event(ctx), e1 = take_event(ctx);
         auto restore = [&]() {
             if (had) ctx->xtune[{n, cost_dtype}] = saved;
             else ctx->xtune.erase({n, cost_dtype});
+            if (!was_pinned) ctx->xpinned.erase({n, cost_dtype});
             ctx->tune_epoch++;
         };
+        ctx->xpinned.insert({n, cost_dtype});  // the schedules are timed as passes
         // best of three timed sweeps after one untimed sweep that builds the plan
         auto time_it = [&](const qaoa_xtune &t, double *ms) -> qaoa_status {
             ctx->xtune[{n, cost_dtype}] = t;
@@ -3177,10 +3183,23 @@ qaoa_status qaoa_autotune_x(qaoa_ctx *ctx, const void *d_cost, int cost_dtype, i
                 }
             }
         }
+        // 3. without passes, where the size has a one-launch kernel: the schedule is
+        // kept for the calls that take passes all the same, and stays pinned only
+        // if the passes are the faster ones
+        ctx->xpinned.erase({n, cost_dtype});
+        double ms = 0.0;
+        st = time_it(best, &ms);
+        if (st) {
+            restore();
+            if (was_pinned) ctx->xpinned.insert({n, cost_dtype});
+            return st;
+        }
+        if (ctx->plan.n_bar > 0 && ms > best.ms) {
+            ctx->xpinned.insert({n, cost_dtype});
+            ctx->tune_epoch++;
+        }
         ctx->ev_pool.push_back(e0);
         ctx->ev_pool.push_back(e1);
-        ctx->xtune[{n, cost_dtype}] = best;
-        ctx->tune_epoch++;
         if (out) *out = best;
         return QAOA_OK;
     } catch (...) {
