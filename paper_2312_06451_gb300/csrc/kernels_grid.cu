@@ -116,7 +116,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
         return g ? ((l & ((1u << c) - 1u)) | (t << c) | ((l >> c) << kNB)) : ((t << kNB) | l);
     };
     auto first_chunk = [&]() {  // one warp: rounds 0 .. kChunk - 1
-        if (lane < p) s_rc[lane] = round_consts(make_coef(ang[lane], ang[p + lane]), M, hp, hq);
+        if (lane < p) s_rc[lane] = round_consts(make_coef(ang[lane], ang[p + lane], COST == 1), M, hp, hq);
     };
     {  // the tile's costs in both tilings, 16 bytes at a time (both keep local bits 0..3)
         constexpr int kPer = COST == 0 ? 4 : 16, kWords = 2 * kTile / kPer;
@@ -152,7 +152,7 @@ grid_kernel(const GridDesc *__restrict__ descs, const uint32_t *__restrict__ beg
         chunk = k / kChunk;
         __syncthreads();
         const int r = chunk * kChunk + tid;
-        if (tid < kChunk && r < p) s_rc[tid] = round_consts(make_coef(ang[r], ang[p + r]), M, hp, hq);
+        if (tid < kChunk && r < p) s_rc[tid] = round_consts(make_coef(ang[r], ang[p + r], COST == 1), M, hp, hq);
         __syncthreads();
     };
     auto coef = [&](int k, float sgn) -> RoundC { return signed_round(s_rc[k % kChunk], sgn); };

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(Chip<NB>::NT) onchip_kernel(const SmallDesc *_
     int chunk = 0;
     auto form = [&](int first, int j) {
         if (first + j < p)
-            s_rc[j] = round_consts(make_coef(ang[first + j], ang[p + first + j]), M, 0u, 0u);
+            s_rc[j] = round_consts(make_coef(ang[first + j], ang[p + first + j], COST == 1), M, 0u, 0u);
     };
     auto load_chunk = [&](int k) {
         if (k / kChunk == chunk) return;

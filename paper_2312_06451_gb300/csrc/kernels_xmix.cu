@@ -264,7 +264,7 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
         for (int e = tid - tab0; e < tot; e += nt - tab0) {
             const int k = e / D.tsize, cst = e - k * D.tsize;
             // e^{-i gamma c} from the turn count gamma c / (2 pi)
-            const double g = D.angles[D.p * nb + k] * kInvTwoPi;
+            const double g = whole_cost_turns(D.angles[D.p * nb + k] * kInvTwoPi);
             const float hi = (float)g;
             D.table[k * kPhaseTable + cst] = phase_turns(hi, (float)(g - (double)hi), (float)cst);
         }

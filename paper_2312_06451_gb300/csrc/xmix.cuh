@@ -48,8 +48,14 @@ __device__ __forceinline__ void sincos_turns(double t, float *s, float *c) {
     }
 }
 
-// e^{-i gamma c} for a small whole cost c, gamma/(2 pi) = g_hi + g_lo: the
-// quarter turns of the head product removed exactly in float32, the tail (the
+// gamma / (2 pi) for whole costs without its own whole turns, which change no
+// phase: what is left fits a float pair to 2^-49 of a turn however large gamma is.
+__device__ __forceinline__ double whole_cost_turns(double g) {
+    return ((uint32_t)__double2hiint(g) & 0x7fffffffu) >= 0x3fe00000u ? g - rint(g) : g;  // |g| >= 1/2
+}
+
+// e^{-i gamma c} for a small whole cost c, gamma/(2 pi) = g_hi + g_lo (see
+// whole_cost_turns): the quarter turns of the head product removed exactly in float32, the tail (the
 // head's rounding and g_lo c) added to the remainder, so the phase is as
 // accurate as from a float64 turn count, without float64 arithmetic (16 cycles
 // a warp instruction on this part).
@@ -77,8 +83,9 @@ __device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
     return make_float2(t, e - (t - p));
 }
 
-// Round coefficients from one beta (rotation) and the round's gamma.
-__device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
+// Round coefficients from one beta (rotation) and the round's gamma (whole:
+// for phases of whole costs only).
+__device__ __forceinline__ RoundCoef make_coef(double be, double ga, bool whole = false) {
     const double bb = be * kInvTwoPi;
     float sb, cb;
     sincos_turns(bb, &sb, &cb);
@@ -95,7 +102,7 @@ __device__ __forceinline__ RoundCoef make_coef(double be, double ga) {
         c.bt = 0.f;
     }
     c.rescale = fabsf(cb) < 0.25f ? 1 : 0;
-    const double g = ga * kInvTwoPi;
+    const double g = whole ? whole_cost_turns(ga * kInvTwoPi) : ga * kInvTwoPi;
     c.g_hi = (float)g;
     c.g_lo = (float)(g - (double)c.g_hi);
     c.b_hi = (float)bb;
