@@ -217,11 +217,15 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
     const PrepDesc D = descs[blockIdx.x];
     // nb angles per round's mixer (nq qubits for multi-angle, else 1):
     // beta_{k,q} = angles[k nb + q], gamma_k = angles[p nb + k]
-    // The coefficients' float64 chain is long: with a table to fill, one warp
-    // forms them while the others fill it.
+    // The coefficients' float64 chain is long: where one warp can form them all at
+    // once, it does while the others fill the table, else every thread takes part
+    // (always one warp: multi-angle, n = 14, p = 100 114 us, now 54; n = 20, p = 4
+    // 13.5, now 8.7).
     const int nb = D.nq ? D.nq : 1;
-    const int tid = threadIdx.x, nt = blockDim.x, tab0 = D.table ? 32 : nt;  // table threads from tab0
-    for (int e = tid; !D.gm_n && tid < tab0 && e < D.p * nb; e += tab0) {
+    const int tid = threadIdx.x, nt = blockDim.x;
+    const bool split = D.table && !D.gm_n && D.p * nb <= 32;
+    const int tab0 = split ? 32 : 0, nco = split ? 32 : nt;  // table threads from tab0, coefficient threads below nco
+    for (int e = tid; !D.gm_n && tid < nco && e < D.p * nb; e += nco) {
         const int k = e / nb;
         const double be = D.angles[e], ga = D.angles[D.p * nb + k];
         if (!isfinite(be) || !isfinite(ga)) atomicOr(err, DERR_BAD_ANGLE);
@@ -260,13 +264,16 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
         }
     }
     if (D.table && tid >= tab0) {
-        const int tot = D.p * D.tsize;
-        for (int e = tid - tab0; e < tot; e += nt - tab0) {
-            const int k = e / D.tsize, cst = e - k * D.tsize;
-            // e^{-i gamma c} from the turn count gamma c / (2 pi)
+        // e^{-i gamma c} from the turn count gamma c / (2 pi): a warp takes half a
+        // round's table at a time, so gamma's float64 part is formed once for four
+        // entries of a lane
+        const int lane = tid & 31, step = (nt - tab0) >> 5, half = kPhaseTable / 2;
+        for (int w = (tid - tab0) >> 5; w < 2 * D.p; w += step) {
+            const int k = w >> 1, c0 = (w & 1) * half;
             const double g = whole_cost_turns(D.angles[D.p * nb + k] * kInvTwoPi);
-            const float hi = (float)g;
-            D.table[k * kPhaseTable + cst] = phase_turns(hi, (float)(g - (double)hi), (float)cst);
+            const float hi = (float)g, lo = (float)(g - (double)hi);
+            for (int c = c0 + lane; c < min(c0 + half, D.tsize); c += 32)
+                D.table[k * kPhaseTable + c] = phase_turns(hi, lo, (float)c);
         }
     }
 }
