@@ -109,13 +109,22 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
     // (general X mixer); nb angles per round's mixer
     const int nb = D.nq ? D.nq : 1;
     const int cs = D.nq ? D.nq : (D.wts ? 2 : 1);
-    auto qcoef = [&](int k, int q) -> const RoundCoef & { return D.coef[k * cs + (D.nq ? q : 0)]; };
+    // the round's rotations, fetched together (one 96-byte entry per qubit and
+    // rotation, in front of each barrier, took 3% of a call)
+    __shared__ float2 s_rot[kSmallMaxN];
+    auto load_rot = [&](int k) {
+        if (!D.wts && tid < n) {
+            const RoundCoef &q = D.coef[k * cs + (D.nq ? tid : 0)];
+            s_rot[tid] = make_float2(q.cb, q.sb);
+        }
+    };
 
     for (int x = tid; x < N; x += kSmallThreads)
         psi[x] = D.init ? D.init[x] : make_float2(D.amp0, 0.f);
     for (int k = 0; k < p; k++) {
         const RoundCoef cf = D.coef[k * cs];
         __syncthreads();
+        load_rot(k);
         load_table(k);
         for (int x = tid; x < N; x += kSmallThreads) psi[x] = cmul(psi[x], phase(x, cf));
         if (D.wts) {
@@ -127,7 +136,7 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
         }
         for (int q = 0; q < n; q++) {
             __syncthreads();
-            mix(psi, q, qcoef(k, q).cb, qcoef(k, q).sb);
+            mix(psi, q, s_rot[q].x, s_rot[q].y);
         }
     }
     __syncthreads();
@@ -150,6 +159,7 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
     for (int k = p - 1; k >= 0; k--) {
         const RoundCoef cf = D.coef[k * cs];
         __syncthreads();
+        load_rot(k);
         float gb = 0.f;
         if (D.wts) {
             // in the Hadamard frame: beta partial sum_z d_|z| Im(conj(lam) psi),
@@ -189,8 +199,8 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
         }
         for (int q = 0; q < (D.wts ? 0 : n); q++) {
             __syncthreads();
-            mix(lam, q, qcoef(k, q).cb, -qcoef(k, q).sb);
-            mix(psi, q, qcoef(k, q).cb, -qcoef(k, q).sb);
+            mix(lam, q, s_rot[q].x, -s_rot[q].y);
+            mix(psi, q, s_rot[q].x, -s_rot[q].y);
         }
         __syncthreads();
         load_table(k);
