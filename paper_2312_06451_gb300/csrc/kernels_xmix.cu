@@ -255,14 +255,21 @@ __global__ void __launch_bounds__(256) prep_kernel(const PrepDesc *__restrict__ 
             if (!isfinite(D.angles[k]) || !isfinite(ga)) atomicOr(err, DERR_BAD_ANGLE);
             RoundCoef c;
             sincos_turns((e & 1) ? -0.125 : 0.125, &c.sb, &c.cb);  // t = -+pi/4
-            c.bmode = 2;
-            c.bt = 0.f;
+            // tan form: tan t = +-1 and the even cosine powers are exact, so a half
+            // round costs one or two rounded scale factors (the rounded cosine, 2 n
+            // times a round, is short of unit length by 1.7e-8 each)
+            c.bmode = 0;
+            c.bt = (e & 1) ? -1.f : 1.f;
             c.rescale = 0;
             const double g = ga * kInvTwoPi;
             c.g_hi = (float)g;
             c.g_lo = (float)(g - (double)c.g_hi);
             c.b_hi = c.b_lo = c.c_lo = c.pad = 0.f;
-            for (int j = 0; j <= kPassTileBits; j++) c.pw[j] = 1.f;  // direct form: no cosine factors
+            float pw = 1.f;
+            for (int j = 0; j <= kPassTileBits; j += 2, pw *= 0.5f) {
+                c.pw[j] = pw;
+                if (j < kPassTileBits) c.pw[j + 1] = pw * 0.70710678f;
+            }
             D.coef[e] = c;
         }
         for (int e = threadIdx.x; e < D.p * (n + 1); e += blockDim.x) {
