@@ -95,17 +95,16 @@ constexpr int kSkMaxN = 40;
 // outputs are +- combinations of five sums: about 4 adds an output instead of
 // n(n-1)/2 with a shared-memory load each.  n = 26, int32: a call 12.1 ms -> 81 us.
 // The output need only be aligned for one value: vectors that a caller packs one
-// behind the other take stores of single values.
+// behind the other take stores of single values (VEC 0).
 template <typename A>
 struct QuadParams {
     A K[kQuadMaxN][kQuadMaxN];  // symmetric, zero diagonal, zero beyond n
     A base;
     int n;
     float scale;  // 2^-shift (float32 output)
-    int vec;      // the output is aligned for stores of four values
 };
 
-template <typename A, int U8, int M>
+template <typename A, int U8, int M, int VEC>
 __global__ void __launch_bounds__(256) cost_quad_kernel(const __grid_constant__ QuadParams<A> Q, int64_t dim, void *out) {
     __shared__ A s_f[12 + M];  // fields of the block's qubits on the local ones
     __shared__ A s_e;          // base + the block qubits' own pairs
@@ -185,7 +184,7 @@ __global__ void __launch_bounds__(256) cost_quad_kernel(const __grid_constant__ 
                 const uchar4 o = make_uchar4((unsigned char)(c[0] >> 1), (unsigned char)(c[1] >> 1),
                                              (unsigned char)(c[2] >> 1), (unsigned char)(c[3] >> 1));
                 unsigned char *dst = reinterpret_cast<unsigned char *>(out) + x;
-                if (Q.vec && x + 4 <= dim) __stcs(reinterpret_cast<uchar4 *>(dst), o);
+                if (VEC && x + 4 <= dim) __stcs(reinterpret_cast<uchar4 *>(dst), o);
                 else
                     for (int i = 0; i < 4; i++)
                         if (x + i < dim) dst[i] = i == 0 ? o.x : i == 1 ? o.y : i == 2 ? o.z : o.w;
@@ -194,7 +193,7 @@ __global__ void __launch_bounds__(256) cost_quad_kernel(const __grid_constant__ 
 #pragma unroll
                 for (int i = 0; i < 4; i++) f[i] = (sizeof(A) == 8 ? __ll2float_rn((long long)c[i]) : __int2float_rn((int)c[i])) * Q.scale;
                 float *dst = reinterpret_cast<float *>(out) + x;
-                if (Q.vec && x + 4 <= dim) __stcs(reinterpret_cast<float4 *>(dst), make_float4(f[0], f[1], f[2], f[3]));
+                if (VEC && x + 4 <= dim) __stcs(reinterpret_cast<float4 *>(dst), make_float4(f[0], f[1], f[2], f[3]));
                 else
                     for (int i = 0; i < 4; i++)
                         if (x + i < dim) dst[i] = f[i];
@@ -307,17 +306,20 @@ cudaError_t go_quad(const CostQuad &C, int64_t dim, void *d_out, cudaStream_t s)
     Q.base = (A)C.base;
     Q.n = std::max(C.n, 12);  // qubits a small instance lacks: no couplings, states past dim not written
     Q.scale = ldexpf(1.f, -C.shift);
-    Q.vec = (reinterpret_cast<uintptr_t>(d_out) & (U8 ? 3 : 15)) == 0;
+    if (reinterpret_cast<uintptr_t>(d_out) & (U8 ? 3 : 15)) {
+        cost_quad_kernel<A, U8, 0, 0><<<1u << (Q.n - 12), 256, 0, s>>>(Q, dim, d_out);
+        return cudaGetLastError();
+    }
     // 2^M tiles a block: all 16 once that leaves two or more blocks an SM (M = 4 from n = 25), fewer
     // tiles and more blocks below
     const int M = std::max(0, std::min(4, Q.n - 21));
     const unsigned grid = 1u << (Q.n - 12 - M);
     switch (M) {
-    case 0: cost_quad_kernel<A, U8, 0><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
-    case 1: cost_quad_kernel<A, U8, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
-    case 2: cost_quad_kernel<A, U8, 2><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
-    case 3: cost_quad_kernel<A, U8, 3><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
-    default: cost_quad_kernel<A, U8, 4><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 0: cost_quad_kernel<A, U8, 0, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 1: cost_quad_kernel<A, U8, 1, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 2: cost_quad_kernel<A, U8, 2, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    case 3: cost_quad_kernel<A, U8, 3, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
+    default: cost_quad_kernel<A, U8, 4, 1><<<grid, 256, 0, s>>>(Q, dim, d_out); break;
     }
     return cudaGetLastError();
 }
