@@ -15,6 +15,7 @@
 // round k's second product).  The adjoint round needs one product per
 // direction as well, thanks to checkpoints of V^T phi_k and psi_{k-1}.
 #include "common.cuh"
+#include "phase.cuh"
 
 #include <type_traits>
 
@@ -24,24 +25,6 @@
 
 namespace qg {
 namespace {
-
-constexpr float kTwoPiF = 6.2831853071795864769f;
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-
-// e^{-i 2 pi (g_hi + g_lo) (x_hi + x_lo)} with the product formed as a float
-// pair and its integer part removed exactly (|g x| < 2^22).
-__device__ __forceinline__ float2 turn_phase(float ghi, float glo, float xhi, float xlo) {
-    const float th = ghi * xhi;
-    const float te = fmaf(ghi, xhi, -th);
-    const float tl = fmaf(ghi, xlo, fmaf(glo, xhi, te));
-    const float f = (th - rintf(th)) + tl;
-    float s, c;
-    __sincosf(kTwoPiF * f, &s, &c);
-    return make_float2(c, -s);
-}
 
 // --------------------------------------------------------------- SIMT GEMM
 // out^T[N][M] = A[M][K] * B^T[N][K]^T, fp32, CUDA cores.  Block tile 128 x 128
