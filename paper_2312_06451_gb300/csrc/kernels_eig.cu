@@ -1022,7 +1022,7 @@ __global__ void __launch_bounds__(1024) eig_scale_kernel(const void *cost, int c
                 if (!(bound > 0.f) || isinf(bound)) return 1.f;
                 int e;
                 frexpf(bound * 1.01f, &e);  // bound < 2^e
-                return ldexpf(kStateTop, -min(max(e, -100), 110));
+                return ldexpf(kStateTop, -max(e, -100));  // e <= 128: sc[1], sc[3] at most 2^102
             };
             const float norm = init ? sqrtf(nrm) : 1.f;
             const float dev = fmaxf(fabsf(hi - (float)s_mean), fabsf(lo - (float)s_mean));
