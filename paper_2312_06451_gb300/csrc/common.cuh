@@ -127,14 +127,13 @@ constexpr int kPassTileBits = 12;
 struct SmallDesc {
     const void *cost;
     const float2 *init;
-    const RoundCoef *coef;   // p entries (p n for multi-angle)
+    const RoundCoef *coef;   // multi-angle: p n entries, general X mixer: 2 p
     const float2 *table;     // p * kPhaseTable entries (uint8 costs)
     double *E_out;
     double *grad_out;        // 2p entries or nullptr
     int n;
     int p;
     float amp0;
-    int nq;                  // multi-angle: n coefficients per round (else 0)
     const double *wts;       // general X mixer: Hadamard-basis weights d_0..d_n (else nullptr)
     const double *angles_beta;  // beta_1..beta_p, then the gammas (the unit's angles)
 };

@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(1024) eig_scale_kernel(const void *cost, int c
 // gradients, a launch, before -> now: n = 11, k = 5 17.0 -> 8.3 us; 13, 6
 // 28.8 -> 11.2; 14, 7 40.2 -> 17.8; 15, 7 58.9 -> 19.3; 16, 8 50.6 -> 38.2
 // (the planes of all sets no longer fit L2); 18, 5 165 -> 26; 20, 4 102 -> 30.
-// n <= 9 has at most 126 states and other lengths no known use: they read M_r.
+// n <= 9 has at most 126 states; 17, 19 and 21..32 were not measured: they read M_r.
 constexpr bool orbit_folds(int r) { return (r >= 10 && r <= 16) || r == 18 || r == 20; }
 constexpr double cx_cos(double x) {  // |x| <= pi
     double t = 1.0, s = 1.0;
@@ -1245,7 +1245,7 @@ __global__ void __launch_bounds__(kOrbitThreads) orbit_kernel(OrbitTabs T, Orbit
             };
             // c = T^T x written to this lane's row of `out` (half planes when out_lo)
             auto from_amp = [&](const float (&x)[RMAX], float *out, float *out_lo) {
-if constexpr (FULL) {
+                if constexpr (FULL) {
                     orbit_from_members<RMAX>(x, c);
                 } else {
 #pragma unroll

@@ -618,7 +618,7 @@ degeneracy_runs_kernel(const __grid_constant__ DegParams P, const __grid_constan
             if (valid) {
 #pragma unroll
                 for (int s = 0; s < 2 * kNC; s++)
-                    if (s < 2 * kNC) h[(tin2 + s) * kDegThreads] += (uint32_t)(H[s] - E[s] + (s ? E[s - 1] : 0));
+                    h[(tin2 + s) * kDegThreads] += (uint32_t)(H[s] - E[s] + (s ? E[s - 1] : 0));
             }
             bound += (uint64_t)(a * (a - 1) / 2);
         }

@@ -34,9 +34,9 @@ namespace qg {
 namespace {
 
 // --------------------------------------------------------------------------
-// Whole state in shared memory (n <= kSmallMaxN): all p rounds, the
-// expectation and (GRAD) the adjoint sweep in one block per unit.  The adjoint
-// undoes each round on psi in place.
+// Multi-angle and general X mixers on a whole state in shared memory (n <=
+// kSmallMaxN): all p rounds, the expectation and (GRAD) the adjoint sweep in one
+// block per unit.  The adjoint undoes each round on psi in place.
 constexpr int kSmallMaxN = 12;
 constexpr int kSmallThreads = 256;
 
@@ -105,16 +105,15 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
         }
         __syncthreads();
     };
-    // coefficients of round k: one entry, one per qubit (multi-angle) or two
-    // (general X mixer); nb angles per round's mixer
-    const int nb = D.nq ? D.nq : 1;
-    const int cs = D.nq ? D.nq : (D.wts ? 2 : 1);
+    // coefficients of round k: one entry per qubit (multi-angle) or two (general X
+    // mixer); nb angles per round's mixer
+    const int nb = D.wts ? 1 : n, cs = D.wts ? 2 : n;
     // the round's rotations, fetched together (one 96-byte entry per qubit and
     // rotation, in front of each barrier, took 3% of a call)
     __shared__ float2 s_rot[kSmallMaxN];
     auto load_rot = [&](int k) {
         if (!D.wts && tid < n) {
-            const RoundCoef &q = D.coef[k * cs + (D.nq ? tid : 0)];
+            const RoundCoef &q = D.coef[k * cs + tid];
             s_rot[tid] = make_float2(q.cb, q.sb);
         }
     };
@@ -160,8 +159,8 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
         const RoundCoef cf = D.coef[k * cs];
         __syncthreads();
         load_rot(k);
-        float gb = 0.f;
         if (D.wts) {
+            float gb = 0.f;
             // in the Hadamard frame: beta partial sum_z d_|z| Im(conj(lam) psi),
             // then the diagonal undone and the frame left again
             weight_phases(D.angles_beta[k]);
@@ -186,16 +185,8 @@ small_kernel(const SmallDesc *__restrict__ descs, int *err) {
                 const float2 l0 = lam[x0], l1 = lam[x1], a0 = psi[x0], a1 = psi[x1];
                 gq += l0.x * a1.y - l0.y * a1.x + l1.x * a0.y - l1.y * a0.x;
             }
-            if (D.nq) {  // one partial per qubit
-                const double GQ = block_sum<kSmallThreads / 32>(gq, s_red);
-                if (tid == 0) D.grad_out[k * n + q] = 2.0 * GQ;
-            } else {
-                gb += gq;
-            }
-        }
-        if (!D.nq && !D.wts) {
-            const double GB = block_sum<kSmallThreads / 32>(gb, s_red);
-            if (tid == 0) D.grad_out[k] = 2.0 * GB;
+            const double GQ = block_sum<kSmallThreads / 32>(gq, s_red);
+            if (tid == 0) D.grad_out[k * n + q] = 2.0 * GQ;
         }
         for (int q = 0; q < (D.wts ? 0 : n); q++) {
             __syncthreads();

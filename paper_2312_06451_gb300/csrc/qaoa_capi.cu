@@ -1,8 +1,8 @@
 // C ABI of the library (include/qaoa.h): context, scratch arena, argument
 // validation, the pass schedule of the X mixer, launch planning and
 // measurement hooks.  All arithmetic of the method runs in the kernels of
-// kernels_xmix.cu / kernels_cost.cu / kernels_eig.cu; this file only decides
-// what to launch on which buffers.
+// kernels_*.cu and xpass.cuh; this file only decides what to launch on which
+// buffers.
 #include "qaoa.h"
 #include "common.cuh"
 
@@ -1259,8 +1259,14 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
         // coefficients of all units back to back (the sets of one eigenbasis
         // job are consecutive, so their rounds form a [set][round] array)
         std::vector<size_t> off_w(nu, 0);
+        // (the transverse field's kernels for all rounds form their own, and their tables)
+        auto forms_own = [&](int i) {
+            const Unit &u = units[i];
+            return u.mixer_kind == QAOA_MIXER_X && !u.ma && !u.gm && (u.n <= smax || on_grid[i]);
+        };
         for (int i = 0; i < nu; i++) {
             off_coef[i] = meta;
+            if (forms_own(i)) continue;
             meta += sizeof(RoundCoef) * units[i].p * (units[i].ma ? units[i].n : (units[i].gm ? 2 : 1));
         }
         meta = align_up(meta);
@@ -1271,7 +1277,7 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                 meta = align_up(meta + sizeof(float4) * u.p * (u.n + 1));
             }
             off_tab[i] = meta;
-            if (u.cost_dtype == QAOA_COST_U8) meta = align_up(meta + sizeof(float2) * kPhaseTable * u.p);
+            if (u.cost_dtype == QAOA_COST_U8 && !forms_own(i)) meta = align_up(meta + sizeof(float2) * kPhaseTable * u.p);
             off_part[i] = meta;
             if (u.mixer_kind == QAOA_MIXER_X && u.n > smax && !on_grid[i]) {
                 lay[i] = layout_for(ctx, u, grad, ckpt);
@@ -1378,13 +1384,9 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
             prep[i].wtab = u.gm ? reinterpret_cast<float4 *>(mb + off_w[i]) : nullptr;
         }
         {
-            // the on-chip and the cooperative kernels form their coefficients themselves
             std::vector<PrepDesc> todo;
-            for (int i = 0; i < nu; i++) {
-                const Unit &u = units[i];
-                if (!(u.mixer_kind == QAOA_MIXER_X && u.n <= smax && !u.ma && !u.gm) && !on_grid[i])
-                    todo.push_back(prep[i]);
-            }
+            for (int i = 0; i < nu; i++)
+                if (!forms_own(i)) todo.push_back(prep[i]);
             if (!todo.empty()) {
                 LaunchRec r;
                 r.kind = LK_PREP;
@@ -1415,7 +1417,6 @@ qaoa_status run_units(qaoa_ctx *ctx, const std::vector<Unit> &units, bool grad, 
                 s.grad_out = grad ? u.grad : nullptr;
                 s.n = u.n;
                 s.p = u.p;
-                s.nq = u.ma ? u.n : 0;
                 s.wts = u.gm ? u.wts : nullptr;
                 s.angles_beta = u.angles;
                 s.amp0 = 1.0f / std::sqrt((float)(1u << u.n));

@@ -1,6 +1,7 @@
-// Device helpers of the transverse-field (X) mixer kernels: phases, round
+// Device helpers of the transverse-field (X) mixer kernels: phase tables, round
 // coefficients, packed rotations and warp sums, shared by the pass kernels
-// (xpass.cuh) and the on-chip kernels (kernels_xmix.cu).
+// (xpass.cuh), the kernels for all rounds in one launch (kernels_onchip.cu,
+// kernels_grid.cu) and the coefficient and small-state kernels (kernels_xmix.cu).
 #pragma once
 
 #include "common.cuh"
@@ -14,22 +15,11 @@
 namespace qg {
 namespace {
 
-// Tile of the pass and n = 12 kernels: 2^12 amplitudes, 16 in each of 256 threads.
+// Tile of the pass and grid kernels: 2^12 amplitudes, 16 in each of 256 threads.
 constexpr int kT = kPassTileBits;
 constexpr int kTile = 1 << kT;
 constexpr int kNT = 256;
 constexpr int kNW = kNT / 32;
-
-// XOR swizzle of a tile-local amplitude index into shared memory.  Bits 1..3
-// are flipped by a fold of bits 6..14, bit 0 is kept so that the amplitude
-// pair (l, l^1) stays one aligned 16-byte vector.  With it, every stage's
-// accesses are conflict free: 16-byte accesses vary local bits 1..3 within a
-// quarter warp; 8-byte accesses vary local bits {0,6,7,8} (stage 2) or
-// {0,1,2,3} (stage 3) within a half warp.  The map is linear over GF(2):
-// swz(a ^ b) = swz(a) ^ swz(b).
-__device__ __forceinline__ uint32_t swz(uint32_t l) {
-    return l ^ ((((l >> 6) ^ (l >> 9) ^ (l >> 12)) & 7u) << 1);
-}
 
 // (sin, cos) of 2 pi t for a float64 turn count t, without float64
 // transcendentals (slow on this part): t = q/4 + r with the nearest quarter

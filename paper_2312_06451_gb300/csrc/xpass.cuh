@@ -233,9 +233,7 @@ struct PassConst {
     int rescale;
 };
 
-// A thread's place in the three layouts (local index of amplitude 0) and where
-// its P amplitudes go: element g + (amplitude i) * rs of the tile, or for ST 1
-// the offsets of its four amplitude bits.
+// A thread's place in the three layouts (local index of amplitude 0).
 struct ThreadPos {
     uint32_t lp, lq, lr;
 };
