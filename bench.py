@@ -845,6 +845,18 @@ def measure(args, W, qg, ctx, stream, dist, ws, rank, local, dev, graph_mode, st
     return out
 
 
+def degeneracy_popcounts(n, k):
+    """(kernel, 32-bit population counts) of the weight-k inside-edge count: per
+    (k-1)-set two for each of k-1 plane combinations (the swept vertices lie in
+    one 64-bit word but for 0.5% of the sets), or, from 2^21 such sets on, per
+    (k-2)-set with smallest vertex a and for each of its k-2 classes one a word
+    at or below w's for every w < a, and four for the class sizes."""
+    if k < 5 or math.comb(n, k - 1) < 1 << 21:
+        return "degeneracy_sliced_kernel", 2 * (k - 1) * math.comb(n, k - 1)
+    return "degeneracy_runs_kernel", sum(
+        math.comb(n - 1 - a, k - 3) * (k - 2) * (sum(w // 32 + 1 for w in range(a)) + 4) for a in range(1, n))
+
+
 def roofline(W, stats, gemm, steps):
     """Roofline of the dominant kernel family (most device time): its
     algorithmic bytes (or useful flops) per launch over its average launch
@@ -854,17 +866,14 @@ def roofline(W, stats, gemm, steps):
     roof = None
     if W.idx == 6:
         # integer enumeration: the bound is the SM's bit-count unit (16
-        # 32-bit population counts a clock per SM).  The bit-sliced count
-        # takes, per (k-1)-set T, one 64-bit population count (2 x 32-bit)
-        # per plane combination 1..k-1 (the swept vertices v < w lie in the
-        # low word for all but 0.5% of the T), and T covers (n-k+1)/k
-        # states on average: 2k(k-1)/(n-k+1) counts per state.  The count by
-        # runs needs fewer; the denominator stays the per-T count's.
+        # 32-bit population counts a clock per SM), for the counts that the
+        # kernel of this size takes
+        kernel, counts = degeneracy_popcounts(W.n, W.k)
         dms = W.degeneracy_ms(steps)
-        ops = 2 * W.k * (W.k - 1) / (W.n - W.k + 1)
+        ops = counts / math.comb(W.n, W.k)
         achieved = W.units / (dms * 1e-3) / 1e9
         peak = 152 * 16 * 2.07e9 / ops / 1e9
-        return {"bound": "alu", "kernel": "degeneracy_runs_kernel", "achieved": achieved, "peak": peak,
+        return {"bound": "alu", "kernel": kernel, "achieved": achieved, "peak": peak,
                 "unit": "Gstates/s", "frac": achieved / peak,
                 "peak_source": f"derived: 152 SM x 16 bit-count ops/clk x 2.07 GHz / {ops:.3f} counts per state",
                 "traffic": None, "launch_ms": dms}
