@@ -277,7 +277,8 @@ gemm_simt_kernel(const float *__restrict__ A, const float *__restrict__ B, int K
 // Ring mixer on 12870 states, 256 sets, p = 6 gradient (24 grouped products):
 // 3.47 -> 2.36 ms; error against 64 bits 5.5e-6 -> 4.6e-6 (draining every 3
 // chunks instead of 2: 2.28 ms, 5.8e-6).  A product takes 71 us, 0.46 of the
-// measured bf16 rate for its three; with the orbit transforms below, 2.17 ms.
+// measured bf16 rate for its three; with the orbit transforms below, 2.19 ms, and
+// with phases of unit length (phase.cuh) 2.24 ms and 3.6e-6.
 //
 // 128 x 128 output tile per CTA, STAGES-deep TMA ring of 128-byte-swizzled
 // K-major tiles.  Warp 0 lane 0 issues TMA loads, warp 1 lane 0 the MMAs;

@@ -61,9 +61,9 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void *tmap, int 
 // Shared-memory traffic, instructions and registers bound the adjoint, not
 // HBM: an earlier layout rotated {0, 9..11}, {1..4}, {5..8} for every tile and
 // so took two transposes (four at a round boundary) whatever was rotated.
-// n = 28, p = 8 gradient, float32 costs: 43.6 -> 38.9 ms; 4 sets of <C> at n = 24,
-// p = 10, uint8 costs: 4.68 -> 4.03 ms; 64 uneven gradients (n = 14..22, p = 6):
-// 7.00 -> 5.81 ms (both with chained launches).
+// n = 28, p = 8 gradient, float32 costs: 43.6 -> 39.1 ms; 4 sets of <C> at n = 24,
+// p = 10, uint8 costs: 4.69 -> 4.05 ms; 64 uneven gradients (n = 14..22, p = 6):
+// 7.5 -> 6.2 ms (all with chained launches).
 //
 // Pipeline: warp 0 loads the tiles of this CTA with TMA copies into NBUF
 // shared-memory buffers (completion on one mbarrier per buffer; the tile's

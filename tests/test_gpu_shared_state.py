@@ -112,3 +112,29 @@ def test_one_buffer_for_both(Q, oracle_mod, grid_first):
     second()
     assert took_grid(ctx)
     assert ctx.scratch_bytes() <= max(held, 384 * MIB) + 32 * MIB
+
+
+def test_capture(oracle_mod):
+    """On-chip, one-launch (clusters and cooperative, more than one launch) and pass units of one call captured in a
+    CUDA graph, replayed with other angles."""
+    import paper_2312_06451_gb300 as qg
+
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream), qg.Context(0, stream) as ctx:
+        made = [make(qg, ctx, oracle_mod, n, 2, sets) for n, sets in ((11, 3), (13, 2), (16, 2), (17, 1), (19, 2), (20, 1), (21, 1))]
+        call = ctx.batched_call([m[0] for m in made], want_grad=True)
+        call.run()
+        check(made)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            call.run()
+        for turn in (1, 2):
+            again = []
+            for job, _, c in made:
+                a = job["angles"].cpu().numpy() * (0.9 if turn == 1 else 1.2)
+                job["angles"].copy_(torch.from_numpy(a))
+                job["E"].zero_()
+                job["grad"].zero_()
+                again.append((job, [oracle_mod.qaoa_gradient(int(c.size).bit_length() - 1, c, x) for x in a], c))
+            graph.replay()
+            check(again)
