@@ -443,8 +443,8 @@ degeneracy_sliced_kernel(const DegParams P, const uint64_t *__restrict__ binom, 
 // adds its KK - 1 counts, 16 bits each, to the class of w in shared memory with
 // one 16-byte read and write.  Tasks (b, 32 sets U, a range of a of about
 // kRunSteps steps) are claimed from a counter.
-// The instruction rate bounds it.  C(100, 6) sets and 1024 reduced gradients, a
-// call: 654 -> 271 us.
+// Instruction issue (66%) and shared memory (70%) bound it.  C(100, 6) sets: 531 ->
+// 178 us, and with 1024 reduced gradients, a call: 654 -> 274.
 constexpr int kRunSteps = 256;
 struct RunPlan {
     uint64_t first[129];    // first task of b (first[n] = number of tasks)
